@@ -103,9 +103,9 @@ typedef struct {
 typedef enum { AMR_INTERP_NEAREST = 0, AMR_INTERP_TRILINEAR = 1 } amr_interp;
 
 /* amr_render_params.schedule value that lets the library choose (the default): deferred
- * shading (3) where it applies (Phong, trilinear, no learned proposal) for images of fewer
- * than 3,000,000 pixels, for batches of views and with secondary rays; the per-ray loop
- * (0) otherwise.  Not in the paper; every schedule renders the same image bit for bit
+ * shading (3) where it applies (Phong, trilinear, no learned proposal; texture storages only
+ * for images of fewer than 3,000,000 pixels); the per-ray loop (0) otherwise.  Not in the
+ * paper; every schedule renders the same image bit for bit
  * (with secondary rays: to rounding, see shadow). */
 #define AMR_SCHEDULE_AUTO (-1)
 

@@ -122,6 +122,31 @@ struct RayArgs {
   int32_t macro_dims[3];
 };
 
+// Workspace of the split march (march_split.cuh): the opaque samples of a launch's tiles as
+// tasks in chunks, and the segments they lie in.
+constexpr int kTaskChunk = 128;      // tasks per chunk
+constexpr int kSegBlock = 64;        // segment records a warp takes at a time
+constexpr int kTaskSampleBits = 23;  // sample number in a task; the lane's number above it
+static_assert(kMaxSamplesPerSegment <= (1 << kTaskSampleBits), "sample number in a task");
+// counters of the workspace: the first kRoundHeads are zeroed for every round
+enum { kHeadChunk = 0, kHeadSegBlock = 1, kHeadOuter = 2, kRoundHeads = 3, kHeadTile = 3,
+       kHeadLeft = 4, kHeadRest = 5, kHeadReady = 6, kHeadDense = 7, kHeads = 8 };
+struct TaskSpace {
+  float4* tasks;        // segment record, sample number | lane << 23, value, weight
+  float4* col;          // per task: colour, weight
+  int32_t* outer;       // tasks whose gradient leaves their leaf
+  int4* meta;           // per chunk: its tile, its tasks, the tile's next chunk
+  float4* segs;         // 3 per record: first sample and step (brick coordinates), margin,
+                        // packed leaf | plane ids, sample count
+  int2* tile;           // per tile: first chunk and number of tasks to add up, or -1
+  int32_t* left;        // tiles given up because the workspace was full (once per round)
+  int32_t* dense;       // tiles given up because they take more than tile_chunks
+  unsigned* heads;      // chunks, segment blocks, outer tasks, tiles handed out; left tiles,
+                        // those of them handed out again, those of earlier rounds; dense tiles
+  int32_t chunks, seg_blocks;
+  int32_t tile_chunks;  // most chunks of one tile
+};
+
 struct RenderArgs {
   RayArgs ray;
   DLevel lv[kMaxLevels];
@@ -158,6 +183,8 @@ struct RenderArgs {
   int32_t coarse_factor;         // learned mode 2: step multiplier below tau
   int32_t learned_min_samples;   // learned modes: segments shorter than this skip the MLP
   long long mdelta;              // stencil-maximum brick = value brick + mdelta bytes (ptr)
+  TaskSpace ts;                  // split march; heads null: none
+  float dense_below;             // a fifth of the cells lie below this value
 };
 
 struct TraceArgs {

@@ -37,15 +37,12 @@ __global__ void __launch_bounds__(TW * TH,
   __shared__ int s_item, s_tf_idx, s_w, s_h, s_item0, s_tiles_x;
   __shared__ long long s_out;
   const int tid = threadIdx.x + TW * threadIdx.y;
-  if (tid < B.n_tf) {
-    int acc = 0;
-    int* nz = s_nz + tid * (tf_n + 1);
-    const float4* tf = A.tf + tid * tf_n;
-    nz[0] = 0;
-    for (int k = 0; k < tf_n; ++k) {
-      acc += __ldg(&tf[k].w) != 0.0f ? 1 : 0;
-      nz[k + 1] = acc;
-    }
+  __shared__ float s_clear[8];
+  for (int t = tid >> 5; t < B.n_tf; t += TW * TH / 32) {
+    int* nz = s_nz + t * (tf_n + 1);
+    tf_prefix_warp(A.tf + t * tf_n, tf_n, nz, tid & 31);
+    const float below = tf_threshold_warp(A, nz, tid & 31);
+    if ((tid & 31) == 0) s_clear[t] = below;
   }
   if (tid == 0) s_ray = A.ray;
   __syncthreads();
@@ -106,11 +103,13 @@ __global__ void __launch_bounds__(TW * TH,
         const size_t area = ((size_t)B.n_tf * (tf_n + 1) * sizeof(int) + 15) & ~(size_t)15;
         DeferArea& Q = reinterpret_cast<DeferArea*>(reinterpret_cast<char*>(smem) + area)[tid >> 5];
         const bool act = i < W && j < H;
-        const float4 c = march_deferred<ST, SHADE>(A, s_ray, i, j, act, tf, nz, Q, nsamp, status);
+        const float4 c = march_deferred<ST, SHADE>(A, s_ray, i, j, act, tf, nz,
+                                                  s_clear[s_tf_idx], Q, nsamp, status);
         if (act) out[(size_t)j * W + i] = c;
       } else if (i < W && j < H) {
         RayF rf;
-        out[(size_t)j * W + i] = march_ray<ST, 1, SHADE>(A, s_ray, i, j, tf, nz, rf, nsamp, status);
+        out[(size_t)j * W + i] = march_ray<ST, 1, SHADE>(A, s_ray, i, j, tf, nz, s_clear[s_tf_idx], rf,
+                                                nsamp, status);
       }
     }
     __syncthreads();  // s_ray and the tile fields are rewritten by the next pop

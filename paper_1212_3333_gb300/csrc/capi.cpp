@@ -304,33 +304,37 @@ amr_status amr_build_kdtree(amr_ctx* c, amr_storage storage, void* cuda_stream) 
   }
 }
 
-// AMR_SCHEDULE_AUTO: the schedule measured fastest for the call's work.  Deferred shading
-// (schedule 3) wherever it applies - Phong, trilinear, no learned proposal - for images of
-// fewer than kAutoDeferredPixels pixels, for batches of views and with secondary rays; the
-// per-ray loop (schedule 0) otherwise.  Measured on the 5-level hierarchy (2,219 patches),
-// Phong + gradient bricks, Gsamples/s per-ray / deferred: 512^2 9.5 / 29.0, 1024^2 31.1 /
-// 46.0, 2048^2 65.4 / 61.1; 64 views of 256-2048 pixels: 21.6 / 30.6.  Every schedule
-// gives the same image bit for bit, so the choice affects time only.
-constexpr int64_t kAutoDeferredPixels = 3000000;
-
-static const amr_render_params* resolve_schedule(const amr_render_params* p, int64_t pixels,
-                                                 bool batch, amr_render_params* tmp) {
-  if (!p || p->schedule != AMR_SCHEDULE_AUTO) return p;
-  *tmp = *p;
-  const bool deferred_applies = p->interp == AMR_INTERP_TRILINEAR && p->shade == 1 &&
-                                p->learned == 0;
-  // secondary rays: the deferred schedule marches each light ray with a whole warp
-  tmp->schedule =
-      deferred_applies && (batch || p->shadow || pixels < kAutoDeferredPixels) ? 3 : 0;
-  return tmp;
-}
-
-// pixels a single-view call renders (its band), for the schedule choice
+// pixels a single-view call renders (its band)
 static int64_t call_pixels(const amr_camera* cam, const amr_render_params* p) {
   if (!cam || !p || cam->width <= 0 || cam->height <= 0) return 0;
   const int64_t row0 = std::max(0, std::min(p->row0, cam->height));
   const int64_t rows = p->rows <= 0 ? cam->height - row0 : std::min<int64_t>(p->rows, cam->height - row0);
   return (int64_t)cam->width * std::max<int64_t>(rows, 0);
+}
+
+static bool textures(const amr_ctx* c) {
+  return c && (c->storage == AMR_STORE_TEXOBJ || c->storage == AMR_STORE_ATLAS_TEX3D);
+}
+
+// AMR_SCHEDULE_AUTO: the schedule measured fastest for the call's work: deferred shading
+// (schedule 3) wherever it applies - Phong, trilinear, no learned proposal - and the per-ray
+// schedule otherwise.  Every schedule gives the same image bit for bit (with secondary rays to
+// rounding), so the choice affects time only.  Single images of kLargePixels pixels and more
+// stay on the per-ray schedule in texture storages, whose deferred march has no workspace and
+// loses there (1900 x 1800: 31.8 against 37 ms), and when samples_per_iter, which only
+// deferred shading reads, is outside its range.
+constexpr int64_t kLargePixels = 3000000;
+
+static const amr_render_params* resolve_schedule(const amr_render_params* p, int64_t pixels,
+                                                 bool textures, amr_render_params* tmp) {
+  if (!p || p->schedule != AMR_SCHEDULE_AUTO) return p;
+  *tmp = *p;
+  const bool deferred_applies = p->interp == AMR_INTERP_TRILINEAR && p->shade == 1 &&
+                                p->learned == 0;
+  const bool steps = p->samples_per_iter >= 1 && p->samples_per_iter <= 64;
+  tmp->schedule =
+      deferred_applies && ((steps && !textures) || p->shadow || pixels < kLargePixels) ? 3 : 0;
+  return tmp;
 }
 
 static amr_status prepare_render(amr_ctx* c, const amr_camera* cam, int32_t tf_n,
@@ -416,6 +420,7 @@ static amr_status prepare_render(amr_ctx* c, const amr_camera* cam, int32_t tf_n
   a->light_ambient = (float)p->light_ambient;
   a->coarse_factor = p->coarse_factor;
   a->learned_min_samples = p->learned_min_samples;
+  a->dense_below = c->dev.dense_below;
   a->mdelta = c->dev.mpool ? (long long)((char*)c->dev.mpool - (char*)c->dev.pool) : 0;
   if (c->dtype != AMR_F32 && (p->interp != AMR_INTERP_TRILINEAR || p->schedule == 1))
     return fail(c, AMR_ERR_ARG, "16-bit cells render trilinear with schedule 0, 2 or 3");
@@ -472,9 +477,10 @@ amr_status prepare_render_args(amr_ctx* c, const amr_camera* cam, int32_t tf_n,
                                const amr_render_params* p, RenderArgs* a) {
   return prepare_render(c, cam, tf_n, p, a);
 }
-amr_render_params resolve_render_schedule(const amr_camera* cam, const amr_render_params& p) {
+amr_render_params resolve_render_schedule(const amr_ctx* c, const amr_camera* cam,
+                                          const amr_render_params& p) {
   amr_render_params tmp;
-  return *resolve_schedule(&p, call_pixels(cam, &p), false, &tmp);
+  return *resolve_schedule(&p, call_pixels(cam, &p), textures(c), &tmp);
 }
 amr_status launch_render_args(amr_ctx* c, const RenderArgs& a, const amr_render_params* p,
                               void* stream) {
@@ -489,8 +495,7 @@ amr_status amr_render(amr_ctx* c, const amr_camera* cam, const float* tf_rgba_de
                       const amr_render_params* params_in, float* out_rgba_dev, void* cuda_stream,
                       uint64_t* samples_out) {
   amr_render_params tmp;
-  const amr_render_params* params =
-      resolve_schedule(params_in, call_pixels(cam, params_in), false, &tmp);
+  const amr_render_params* params = resolve_schedule(params_in, call_pixels(cam, params_in), textures(c), &tmp);
   RenderArgs a;
   amr_status s = prepare_render(c, cam, tf_n, params, &a);
   if (s != AMR_OK) return s;
@@ -510,8 +515,7 @@ amr_status amr_render_host(amr_ctx* c, const amr_camera* cam, const float* tf_rg
                            int32_t tf_n, const amr_render_params* params_in, float* out_rgba_host,
                            void* cuda_stream, uint64_t* samples_out) {
   amr_render_params tmp;
-  const amr_render_params* params =
-      resolve_schedule(params_in, call_pixels(cam, params_in), false, &tmp);
+  const amr_render_params* params = resolve_schedule(params_in, call_pixels(cam, params_in), textures(c), &tmp);
   RenderArgs a;
   amr_status s = prepare_render(c, cam, tf_n, params, &a);
   if (s != AMR_OK) return s;
@@ -639,7 +643,7 @@ amr_status amr_render_batch(amr_ctx* c, const amr_view* views, int32_t n_views,
                             uint64_t* samples_out) {
   if (!c) return AMR_ERR_ARG;
   amr_render_params tmp;
-  const amr_render_params* params = resolve_schedule(params_in, 0, true, &tmp);
+  const amr_render_params* params = resolve_schedule(params_in, 0, false, &tmp);
   const amr_batch_config cfg = config ? *config : c->batch_cfg;
   std::unique_ptr<BatchArgs> b(new (std::nothrow) BatchArgs());
   if (!b) return fail(c, AMR_ERR_OOM, "out of host memory");
@@ -661,7 +665,7 @@ amr_status amr_batch_autotune(amr_ctx* c, const amr_view* views, int32_t n_views
                               amr_batch_config* best_out, float* ms_out) {
   if (!c) return AMR_ERR_ARG;
   amr_render_params tmp;
-  const amr_render_params* params = resolve_schedule(params_in, 0, true, &tmp);
+  const amr_render_params* params = resolve_schedule(params_in, 0, false, &tmp);
   if (reps < 1 || reps > 1000) return fail(c, AMR_ERR_ARG, "reps must be in [1, 1000]");
   static const int shapes[3][2] = {{8, 8}, {16, 8}, {16, 16}};
   static const int rpts[3] = {1, 2, 4};

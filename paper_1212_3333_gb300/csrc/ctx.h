@@ -3,6 +3,7 @@
 #pragma once
 #include <stdint.h>
 
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <string>
@@ -88,6 +89,19 @@ struct DeviceState {
   int32_t macro_cell = 1;                        // finest cells per macro cell per axis
   int32_t macro_dims[3] = {1, 1, 1};
   int device = -1;
+  // workspaces of the split march, each for up to task_pixels pixels; the last is in use,
+  // earlier ones stay for CUDA graphs that hold their addresses (sizes at least double)
+  std::vector<void*> task_spaces;
+  TaskSpace tasks = {};
+  float dense_below = -INFINITY;     // a fifth of the cells lie below this value
+  int64_t task_pixels = 0;
+  int64_t task_refused = INT64_MAX;  // a workspace for this many pixels could not be allocated
+};
+
+// How a call uses the workspace: rows per band (0: no workspace) and rounds per band.
+struct TaskPlan {
+  TaskSpace ts = {};
+  int rows = 0, rounds = 0;
 };
 
 }  // namespace amr
@@ -133,6 +147,9 @@ amr_status pack_atlas(amr_ctx* c);
 // device.cpp
 amr_status upload(amr_ctx* c, void* stream);
 void release_device(amr_ctx* c);
+// The split march's workspace for an image or band, grown when it is too small and the stream
+// is not being captured; no rows when there is none (out of memory, or a first call captured).
+TaskPlan plan_tasks(amr_ctx* c, const RenderArgs& a, void* stream);
 // kernels (march.cu)
 amr_status launch_render(amr_ctx* c, const RenderArgs& a, int storage, int interp, int shade,
                          int schedule, void* stream);
@@ -156,6 +173,7 @@ amr_status prepare_render_args(amr_ctx* c, const amr_camera* cam, int32_t tf_n,
 amr_status launch_render_args(amr_ctx* c, const RenderArgs& a, const amr_render_params* p,
                               void* stream);
 // params with AMR_SCHEDULE_AUTO replaced by the schedule a single-view call would use
-amr_render_params resolve_render_schedule(const amr_camera* cam, const amr_render_params& p);
+amr_render_params resolve_render_schedule(const amr_ctx* c, const amr_camera* cam,
+                                          const amr_render_params& p);
 
 }  // namespace amr

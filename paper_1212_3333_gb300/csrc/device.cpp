@@ -264,6 +264,82 @@ amr_status upload_max_pool(amr_ctx* c, const std::vector<std::vector<T>>& mb, cu
 
 }  // namespace
 
+// Workspace of the split march (36 bytes a task, and a segment record of 48 bytes for every
+// third): kTasksPerPixel tasks for every pixel - the 5-level hierarchy with a ramp transfer
+// function takes 23, and 8 records -, up to kMaxTasks, but kTileChunks chunks (320 tasks a
+// pixel) for every tile under way, so that dense tiles need not be given up: 1.7 GB for most
+// images, 3.5 GB at most.  (With 40 tasks a pixel alone, at 640 x 479 tiles were given up
+// and the frame took 5.4 instead of 2.7 ms.)  A call gets enough rounds for kDensePerPixel
+// tasks a pixel; what is denser goes to deferred_kernel (every sample opaque, 640 x 479, 480
+// tasks a pixel: all tasks in the workspace 14.3 ms, deferred_kernel alone 16.1).
+static constexpr int64_t kTasksPerPixel = 40, kDensePerPixel = 128, kTileChunks = 80;
+static constexpr int64_t kMaxTasks = (int64_t)1 << 26;
+static constexpr int64_t kBandPixels = (int64_t)1 << 24;
+static constexpr int64_t kWarps = 152 * 16;  // of the march, at once
+
+static int64_t task_rounds(int64_t pixels, int64_t chunks) {
+  const int64_t usable = (chunks - chunks / 4) * kTaskChunk;
+  return std::min<int64_t>(64, (pixels * kDensePerPixel + usable - 1) / usable);
+}
+
+TaskPlan plan_tasks(amr_ctx* c, const RenderArgs& a, void* stream) {
+  TaskPlan plan;
+  DeviceState& d = c->dev;
+  const int64_t tiles_x = (a.ray.width + 7) / 8, row_pixels = 32 * tiles_x;  // of a row of tiles
+  const int64_t tile_rows = (a.ray.rows + 3) / 4;
+  if (tile_rows <= 0 || tiles_x <= 0) return plan;
+  const int64_t want = std::min(tile_rows * row_pixels, std::max(kBandPixels, row_pixels));
+  if (want > d.task_pixels && want < d.task_refused) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing((cudaStream_t)stream, &cap) != cudaSuccess) cudaGetLastError();
+    const int64_t px = std::max(want, std::min(2 * d.task_pixels, kBandPixels));
+    const int64_t tiles = px / 32;
+    const int64_t under_way = std::min(tiles, kWarps) * kTileChunks * kTaskChunk * 4 / 3;
+    const int64_t chunks = std::min(std::max(px * kTasksPerPixel, under_way), kMaxTasks) / kTaskChunk;
+    const size_t slots = (size_t)chunks * kTaskChunk;
+    const int64_t blocks = (int64_t)slots / 3 / kSegBlock + 2 * kWarps;
+    const int64_t rounds = task_rounds(px, chunks);
+    const size_t sizes[9] = {slots * sizeof(float4), slots * sizeof(float4), slots * sizeof(int32_t),
+                             (size_t)chunks * sizeof(int4),
+                             (size_t)blocks * kSegBlock * 3 * sizeof(float4),
+                             (size_t)tiles * sizeof(int2),
+                             (size_t)(tiles * rounds) * sizeof(int32_t),
+                             (size_t)tiles * sizeof(int32_t), kHeads * sizeof(unsigned)};
+    size_t off[10] = {0};
+    for (int k = 0; k < 9; ++k) off[k + 1] = off[k] + ((sizes[k] + 255) & ~(size_t)255);
+    char* p = nullptr;
+    if (cap == cudaStreamCaptureStatusNone) {
+      if (cudaMalloc((void**)&p, off[9]) != cudaSuccess) {
+        cudaGetLastError();
+        p = nullptr;
+        d.task_refused = want;
+      }
+    }
+    if (p) {
+      d.task_spaces.push_back(p);
+      d.task_pixels = px;
+      d.tasks.tasks = (float4*)(p + off[0]);
+      d.tasks.col = (float4*)(p + off[1]);
+      d.tasks.outer = (int32_t*)(p + off[2]);
+      d.tasks.meta = (int4*)(p + off[3]);
+      d.tasks.segs = (float4*)(p + off[4]);
+      d.tasks.tile = (int2*)(p + off[5]);
+      d.tasks.left = (int32_t*)(p + off[6]);
+      d.tasks.dense = (int32_t*)(p + off[7]);
+      d.tasks.heads = (unsigned*)(p + off[8]);
+      d.tasks.tile_chunks = (int32_t)std::max<int64_t>(1, 3 * chunks / std::min(tiles, kWarps));
+      d.tasks.chunks = (int32_t)chunks;
+      d.tasks.seg_blocks = (int32_t)blocks;
+    }
+  }
+  const int64_t rows = d.task_pixels / row_pixels * 4;
+  if (rows <= 0) return plan;
+  plan.ts = d.tasks;
+  plan.rows = (int)std::min<int64_t>(rows, tile_rows * 4);
+  plan.rounds = (int)task_rounds(plan.rows / 4 * row_pixels, d.tasks.chunks);
+  return plan;
+}
+
 void release_device(amr_ctx* c) {
   DeviceState& d = c->dev;
   if (d.device >= 0) cudaSetDevice(d.device);
@@ -295,14 +371,32 @@ void release_device(amr_ctx* c) {
   cudaFree(d.img_scratch);
   cudaFree(d.log_counts);
   cudaFree(d.log_offsets);
+  for (void* p : d.task_spaces) cudaFree(p);
   d = DeviceState();
   c->device_built = false;
+}
+
+// The value a fifth of the bricks' cells lie below, from at most about 2^16 of them.
+static float low_quantile(const amr_ctx* c) {
+  size_t cells = 0, at = 0;
+  for (const auto& b : c->bricks) cells += b.size();
+  const size_t stride = std::max<size_t>(1, cells >> 16);
+  std::vector<float> v;
+  for (const auto& b : c->bricks) {
+    for (; at < b.size(); at += stride)
+      if (!std::isnan(b[at])) v.push_back(b[at]);
+    at -= b.size();
+  }
+  if (v.empty()) return -INFINITY;
+  std::nth_element(v.begin(), v.begin() + v.size() / 5, v.end());
+  return v[v.size() / 5];
 }
 
 amr_status upload(amr_ctx* c, void* stream_v) {
   cudaStream_t stream = (cudaStream_t)stream_v;
   if (c->device_built) release_device(c);
   DeviceState& d = c->dev;
+  d.dense_below = low_quantile(c);
   CK(cudaGetDevice(&d.device));
   const Tree& t = c->tree;
   const size_t P = c->patches.size();

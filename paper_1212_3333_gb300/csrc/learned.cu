@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(128) log_kernel(const __grid_constant__ Render
       const float a_in = Acc;
       SegSetup g;
       setup_segment(A, rf, lf, lv, lid, pid0, pid1, tau0, e0, tau1, e1, n, i, j, g);
-      sample_segment<ST, 1, 0>(A, A.ray, s_tf, nullptr, g, lv, 0.f, 0.f, 0.f, C0, C1, C2, Acc,
+      sample_segment<ST, 1, 0>(A, A.ray, s_tf, 0.0f, g, lv, 0.f, 0.f, 0.f, C0, C1, C2, Acc,
                                nsamp);
       if (log_keep(L, i, j, seg)) {
         const unsigned long long idx = L.offsets[pix] + (unsigned long long)kept++;
@@ -165,23 +165,23 @@ __global__ void __launch_bounds__(1024) log_scan_kernel(const int32_t* __restric
   }
 }
 
-// The learned march samples a segment as the plain march does; with stencil-maximum bricks
-// it tests every sample's maximum on its own (AMR_LEARNED_GROUP 0) or G at a time.
+// stencil maxima the learned march loads together (segments are often a few coarse samples)
 #ifndef AMR_LEARNED_GROUP
-#define AMR_LEARNED_GROUP 0
+#define AMR_LEARNED_GROUP 4
 #endif
 template <int ST, int SHADE>
 __device__ __forceinline__ bool sample_learned(const RenderArgs& A, const float4* s_tf,
-                                               const int* s_nz, const SegSetup& g,
+                                               float clear_below, const SegSetup& g,
                                                const DLevel& lv, float Lx, float Ly, float Lz,
                                                float& C0, float& C1, float& C2, float& Acc,
                                                unsigned& nsamp) {
   if constexpr ((SHADE & kShadeMaxBit) != 0)
-    return sample_segment_grouped<ST, SHADE, AMR_LEARNED_GROUP>(A, A.ray, s_tf, s_nz, g, lv, Lx,
-                                                                Ly, Lz, C0, C1, C2, Acc, nsamp);
+    return sample_segment_grouped<ST, SHADE, AMR_LEARNED_GROUP>(A, A.ray, s_tf, clear_below, g,
+                                                                lv, Lx, Ly, Lz, C0, C1, C2, Acc,
+                                                                nsamp);
   else
-    return sample_segment<ST, 1, SHADE>(A, A.ray, s_tf, s_nz, g, lv, Lx, Ly, Lz, C0, C1, C2, Acc,
-                                        nsamp);
+    return sample_segment<ST, 1, SHADE>(A, A.ray, s_tf, clear_below, g, lv, Lx, Ly, Lz, C0, C1,
+                                        C2, Acc, nsamp);
 }
 
 #ifndef AMR_LEARNED_TILE_W
@@ -201,19 +201,11 @@ __global__ void __launch_bounds__(128, AMR_MIN_BLOCKS) learned_kernel(const __gr
   unsigned char* wsm = reinterpret_cast<unsigned char*>(smem) + ((tf_bytes + 15) & ~(size_t)15);
   __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(wsm + kPackBytes) + warp * 32 * kStride1;
   float* ys = reinterpret_cast<float*>(wsm + kPackBytes + 4 * 32 * kStride1 * 2) + warp * 32;
-  for (int k = tid; k < A.tf_n; k += blockDim.x * blockDim.y) s_tf[k] = A.tf[k];
+  __shared__ float s_clear;
   for (int k = tid; k < kPackBytes / 16; k += blockDim.x * blockDim.y)
     reinterpret_cast<uint4*>(wsm)[k] = reinterpret_cast<const uint4*>(A.mlp)[k];
-  __syncthreads();
-  if (tid == 0) {
-    int acc = 0;
-    s_nz[0] = 0;
-    for (int k = 0; k < A.tf_n; ++k) {
-      acc += s_tf[k].w != 0.0f ? 1 : 0;
-      s_nz[k + 1] = acc;
-    }
-  }
-  __syncthreads();
+  stage_tf(A, s_tf, s_nz, &s_clear, tid, blockDim.x * blockDim.y);
+  const float clear_below = s_clear;
 
   unsigned nsamp = 0;
   unsigned long long status = 0;
@@ -304,7 +296,8 @@ __global__ void __launch_bounds__(128, AMR_MIN_BLOCKS) learned_kernel(const __gr
         const DLevel& lv = A.lv[lf.level];
         SegSetup g;
         setup_segment(A, rf, lf, lv, lid, pid0, pid1, tau0, e0, tau1, e1, n, i, j, g);
-        if (sample_learned<ST, SHADE>(A, s_tf, s_nz, g, lv, Lx, Ly, Lz, C0, C1, C2, Acc, nsamp))
+        if (sample_learned<ST, SHADE>(A, s_tf, clear_below, g, lv, Lx, Ly, Lz, C0, C1, C2, Acc,
+                                      nsamp))
           live = false;  // early ray termination
       }
       if (lid >= 0) {

@@ -34,6 +34,12 @@ enum {
   ST_PTR_F16 = 4, ST_PTR_BF16 = 5, ST_ATLAS_LINEAR_F16 = 6, ST_ATLAS_LINEAR_BF16 = 7
 };
 
+// x 2^E: what ldexpf gives, in one multiplication
+template <int E>
+__device__ __forceinline__ float scale2(float x) {
+  return __fmul_rn(x, __int_as_float((127 + E) << 23));
+}
+
 // plane ids: split * 4 + axis; the two ray ends use axis field 3
 constexpr int kPidIn = 3;
 constexpr int kPidOut = 7;
@@ -211,7 +217,7 @@ __device__ __forceinline__ void make_frame(const RayArgs& A, const RayX& r, RayF
 }
 
 // error bound of tau_out (recomputed where needed instead of held per ray)
-__device__ __forceinline__ float exit_bound(const RayF& f) { return ldexpf(f.tau_out + 1.0f, -22); }
+__device__ __forceinline__ float exit_bound(const RayF& f) { return scale2<-22>(f.tau_out + 1.0f); }
 
 // Level-of-detail pruning (Sec. 3.1: a type-(a) node's region is held by at least two
 // levels; Sec. 3.3: the descent may stop there when the coarser cells project small
@@ -241,9 +247,9 @@ __device__ __forceinline__ int lod_min_level(const RayArgs& R, const DLevel* lv,
   if (!(R.lod_scale_f > 0.0f)) return kNoLod;
   const float t0 = rf.t_in + tau0;
   const float X = R.lod_scale_f * t0;
-  const float eX = R.lod_scale_f * (e0 + ldexpf(rf.t_in + fabsf(t0) + 1.0f, -22)) + ldexpf(X, -21);
+  const float eX = R.lod_scale_f * (e0 + scale2<-22>(rf.t_in + fabsf(t0) + 1.0f)) + scale2<-21>(X);
   for (int l = 0; l < R.levels; ++l) {
-    const float hm = lv[l].hmin, eh = ldexpf(hm, -22);
+    const float hm = lv[l].hmin, eh = scale2<-22>(hm);
     if (hm + eh < X - eX) return l;  // certainly h <= X
     if (hm - eh > X + eX) continue;  // certainly h > X
     return lod_min_exact(R, lv, px, py, pid0);
@@ -265,7 +271,7 @@ __device__ __forceinline__ float plane_tau(const RayF& rf, uint32_t ax, int s, f
   const float ts = fmaf(sf, sel3f(ax, rf.B[0], rf.B[1], rf.B[2]), sel3f(ax, rf.C[0], rf.C[1], rf.C[2])) +
                    fmaf(sf, sel3f(ax, rf.Bl[0], rf.Bl[1], rf.Bl[2]),
                         sel3f(ax, rf.Cl[0], rf.Cl[1], rf.Cl[2]));
-  es = ((rf.exact_axes >> ax) & 1) ? __int_as_float(0x7f800000) : ldexpf(fabsf(ts) + 1.0f, -22);
+  es = ((rf.exact_axes >> ax) & 1) ? __int_as_float(0x7f800000) : scale2<-22>(fabsf(ts) + 1.0f);
   return ts;
 }
 
@@ -954,6 +960,17 @@ __device__ __forceinline__ float4 tf_lookup(const float4* __restrict__ tf, int n
                      fmaf(w, b.w - a.w, a.w));
 }
 
+// The opacity entry of tf_lookup alone.
+__device__ __forceinline__ float tf_alpha(const float4* __restrict__ tf, int n, float v, float vmin,
+                                          float inv_range) {
+  float u = (v - vmin) * inv_range;
+  u = fminf(fmaxf(u, 0.0f), 1.0f) * (float)(n - 1);
+  const int i = min((int)u, n - 2);
+  const float w = u - (float)i;
+  const float a = tf[i].w, b = tf[i + 1].w;
+  return fmaf(w, b - a, a);
+}
+
 // true when the transfer function is fully transparent over [v0, v1] (conservative)
 __device__ __forceinline__ bool tf_transparent(const int* __restrict__ nz_prefix, int n, float v0,
                                                float v1, float vmin, float inv_range) {
@@ -973,7 +990,7 @@ __device__ __forceinline__ int segment_count(const RayArgs& R, int px, int py, c
   const float lenf = (tau1 - tau0) * f.dn;
   const float q = lenf * inv_step;
   // |q - exact| <= (e0 + e1) |d| / step + 5u q (subtraction, |d|, product, 1/step roundings)
-  const float eq = (e0 + e1) * f.dn * inv_step + ldexpf(q + 1.0f, -21);
+  const float eq = (e0 + e1) * f.dn * inv_step + scale2<-21>(q + 1.0f);
   if (q + eq <= 1.0f) return 1;
   const float c = ceilf(q);
   if (c - q > eq && q - (c - 1.0f) > eq && c <= (float)kMaxSamplesPerSegment) return (int)c;
@@ -1039,61 +1056,66 @@ __device__ __forceinline__ GradCorners grad_fetch(const RenderArgs& A, const Bri
   return c;
 }
 
+// The gradient at a brick position both of whose neighbours on every axis read the brick:
+// one interpolation of the gradient brick's per-cell differences (GB), or one 32-cell stencil.
+template <int ST, int GB>
+__device__ __forceinline__ void gradient_brick(const RenderArgs& A, const BrickRef& b,
+                                               const float* beta, const DLevel& lv, float* g) {
+  if constexpr (GB) {
+    grad_fetch<ST>(A, b, beta).gradient(lv, g);
+  } else {
+    const int ix = min(max((int)beta[0], 1), b.dim[0] - 3);
+    const int iy = min(max((int)beta[1], 1), b.dim[1] - 3);
+    const int iz = min(max((int)beta[2], 1), b.dim[2] - 3);
+    const float wx = beta[0] - (float)ix, wy = beta[1] - (float)iy, wz = beta[2] - (float)iz;
+    using I = typename BrickIndex<ST>::type;
+    const I l0 = (I)ix + (I)b.sy * iy + (I)b.sz * iz;
+    auto V = [&](int dx, int dy, int dz) {
+      return fetch<ST>(A, b, l0 + dx + (I)b.sy * dy + (I)b.sz * dz, ix + dx,
+                       iy + dy, iz + dz);
+    };
+    float c[2][2][2];
+#pragma unroll
+    for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
+      for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
+        for (int dx = 0; dx < 2; ++dx) c[dz][dy][dx] = V(dx, dy, dz);
+    float dxv[2][2], dyv[2][2], dzv[2][2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        // x: at (y = iy + u, z = iz + v)
+        const float xm = V(-1, u, v), xp = V(2, u, v);
+        dxv[v][u] = fmaf(wx, xp - c[v][u][1], c[v][u][1]) - fmaf(wx, c[v][u][0] - xm, xm);
+        // y: at (x = ix + u, z = iz + v)
+        const float ym = V(u, -1, v), yp = V(u, 2, v);
+        dyv[v][u] = fmaf(wy, yp - c[v][1][u], c[v][1][u]) - fmaf(wy, c[v][0][u] - ym, ym);
+        // z: at (x = ix + u, y = iy + v)
+        const float zm = V(u, v, -1), zp = V(u, v, 2);
+        dzv[v][u] = fmaf(wz, zp - c[1][v][u], c[1][v][u]) - fmaf(wz, c[0][v][u] - zm, zm);
+      }
+    // bilinear combination in the two transverse axes
+    const float gx0 = fmaf(wy, dxv[0][1] - dxv[0][0], dxv[0][0]);
+    const float gx1 = fmaf(wy, dxv[1][1] - dxv[1][0], dxv[1][0]);
+    const float gy0 = fmaf(wx, dyv[0][1] - dyv[0][0], dyv[0][0]);
+    const float gy1 = fmaf(wx, dyv[1][1] - dyv[1][0], dyv[1][0]);
+    const float gz0 = fmaf(wx, dzv[0][1] - dzv[0][0], dzv[0][0]);
+    const float gz1 = fmaf(wx, dzv[1][1] - dzv[1][0], dzv[1][0]);
+    g[0] = fmaf(wz, gx1 - gx0, gx0) * lv.ginv[0];
+    g[1] = fmaf(wz, gy1 - gy0, gy0) * lv.ginv[1];
+    g[2] = fmaf(wy, gz1 - gz0, gz0) * lv.ginv[2];
+  }
+}
+
 template <int ST, int INTERP, int GB>
 __device__ __forceinline__ void gradient(const RenderArgs& A, const RayArgs& R, const SegState& s,
                                          const float* beta,
                                          int k, const DLevel& lv, float* g) {
   if constexpr (INTERP == 1) {
-    const bool inner = gradient_inner(s, beta);
-    if (GB && inner) {
-      // gradient brick: trilinear interpolation of the per-cell central differences
-      grad_fetch<ST>(A, s.brick, beta).gradient(lv, g);
-      return;
-    }
-    if (inner) {
-      const BrickRef& b = s.brick;
-      const int ix = min(max((int)beta[0], 1), b.dim[0] - 3);
-      const int iy = min(max((int)beta[1], 1), b.dim[1] - 3);
-      const int iz = min(max((int)beta[2], 1), b.dim[2] - 3);
-      const float wx = beta[0] - (float)ix, wy = beta[1] - (float)iy, wz = beta[2] - (float)iz;
-      using I = typename BrickIndex<ST>::type;
-      const I l0 = (I)ix + (I)b.sy * iy + (I)b.sz * iz;
-      auto V = [&](int dx, int dy, int dz) {
-        return fetch<ST>(A, b, l0 + dx + (I)b.sy * dy + (I)b.sz * dz, ix + dx,
-                         iy + dy, iz + dz);
-      };
-      float c[2][2][2];
-#pragma unroll
-      for (int dz = 0; dz < 2; ++dz)
-#pragma unroll
-        for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-          for (int dx = 0; dx < 2; ++dx) c[dz][dy][dx] = V(dx, dy, dz);
-      float dxv[2][2], dyv[2][2], dzv[2][2];
-#pragma unroll
-      for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int v = 0; v < 2; ++v) {
-          // x: at (y = iy + u, z = iz + v)
-          const float xm = V(-1, u, v), xp = V(2, u, v);
-          dxv[v][u] = fmaf(wx, xp - c[v][u][1], c[v][u][1]) - fmaf(wx, c[v][u][0] - xm, xm);
-          // y: at (x = ix + u, z = iz + v)
-          const float ym = V(u, -1, v), yp = V(u, 2, v);
-          dyv[v][u] = fmaf(wy, yp - c[v][1][u], c[v][1][u]) - fmaf(wy, c[v][0][u] - ym, ym);
-          // z: at (x = ix + u, y = iy + v)
-          const float zm = V(u, v, -1), zp = V(u, v, 2);
-          dzv[v][u] = fmaf(wz, zp - c[1][v][u], c[1][v][u]) - fmaf(wz, c[0][v][u] - zm, zm);
-        }
-      // bilinear combination in the two transverse axes
-      const float gx0 = fmaf(wy, dxv[0][1] - dxv[0][0], dxv[0][0]);
-      const float gx1 = fmaf(wy, dxv[1][1] - dxv[1][0], dxv[1][0]);
-      const float gy0 = fmaf(wx, dyv[0][1] - dyv[0][0], dyv[0][0]);
-      const float gy1 = fmaf(wx, dyv[1][1] - dyv[1][0], dyv[1][0]);
-      const float gz0 = fmaf(wx, dzv[0][1] - dzv[0][0], dzv[0][0]);
-      const float gz1 = fmaf(wx, dzv[1][1] - dzv[1][0], dzv[1][0]);
-      g[0] = fmaf(wz, gx1 - gx0, gx0) * lv.ginv[0];
-      g[1] = fmaf(wz, gy1 - gy0, gy0) * lv.ginv[1];
-      g[2] = fmaf(wy, gz1 - gz0, gz0) * lv.ginv[2];
+    if (gradient_inner(s, beta)) {
+      gradient_brick<ST, GB>(A, s.brick, beta, lv, g);
       return;
     }
   }
@@ -1124,6 +1146,64 @@ struct SegSetup {
   SegState s;
   float b0[3], db[3];
   float delta;
+};
+
+// Walk over a segment's stencil maxima (pointer storages).  A sample's stencil corner is the
+// floor of its brick position; fmaf and floor are monotone in the sample number, so when the
+// first and the last sample lie inside the brick all of them do, and no position is clamped.
+// The floor is one addition of 2^23 rounded down (exact for 0 <= x < 2^23), whose low bits
+// are the integer; the three exponent fields fold into one constant of the offset.  14
+// instructions a sample instead of about 30 (clamps, conversions and the table test).
+template <int ST>
+struct MaxWalk {
+  float b0[3], db[3];
+  long long base;   // the maximum brick
+  int sy, sz, bias;
+  bool inside;      // every sample of the segment lies inside the brick
+
+  __device__ __forceinline__ void start(const RenderArgs& A, const SegSetup& g) {
+    const float kl = (float)(g.s.n - 1);
+    inside = true;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      b0[a] = g.b0[a];
+      db[a] = g.db[a];
+      const float end = fmaf(kl, db[a], b0[a]), hi = (float)(g.s.brick.dim[a] - 1);
+      inside = inside && b0[a] >= 0.0f && b0[a] < hi && end >= 0.0f && end < hi;
+    }
+    base = g.s.brick.base + A.mdelta;
+    sy = g.s.brick.sy;
+    sz = g.s.brick.sz;
+    bias = (int)(0u - 0x4B000000u * (1u + (unsigned)sy + (unsigned)sz));
+  }
+  // cell offset of sample kf's stencil corner
+  __device__ __forceinline__ int corner(float kf) const {
+    const int x = __float_as_int(__fadd_rd(fmaf(kf, db[0], b0[0]), 8388608.0f));
+    const int y = __float_as_int(__fadd_rd(fmaf(kf, db[1], b0[1]), 8388608.0f));
+    const int z = __float_as_int(__fadd_rd(fmaf(kf, db[2], b0[2]), 8388608.0f));
+    return (int)((unsigned)bias + (unsigned)x + (unsigned)sy * (unsigned)y +
+                 (unsigned)sz * (unsigned)z);
+  }
+  __device__ __forceinline__ float maximum(int lin) const {
+    if constexpr (ST == ST_PTR_F16)
+      return __half2float(__ldg(reinterpret_cast<const __half*>(base) + lin));
+    else if constexpr (ST == ST_PTR_BF16)
+      return __bfloat162float(__ldg(reinterpret_cast<const __nv_bfloat16*>(base) + lin));
+    else
+      return __ldg(reinterpret_cast<const float*>(base) + lin);
+  }
+  // bit q: sample k + q (the last one repeated beyond the segment's end) may be opaque
+  template <int G>
+  __device__ __forceinline__ unsigned opaque_mask(int k, int n, float clear_below) const {
+    const float kf = (float)k, kl = (float)(n - 1);
+    float m[G];
+#pragma unroll
+    for (int q = 0; q < G; ++q) m[q] = maximum(corner(fminf(kf + (float)q, kl)));
+    unsigned mask = 0;
+#pragma unroll
+    for (int q = 0; q < G; ++q) mask |= m[q] < clear_below ? 0u : 1u << q;
+    return mask;
+  }
 };
 
 // The leaf's corner and its box in brick coordinates, the region whose gradient neighbours
@@ -1167,7 +1247,7 @@ __device__ __forceinline__ void setup_segment(const RenderArgs& A, const RayF& r
   const float dtau = (tau1 - tau0) / nfl;
   g.delta = dtau * rf.dn;
   const float taum = fmaf(0.5f, dtau, tau0);
-  const float etau = fmaxf(e0, e1) + ldexpf(tau1 + 1.0f, -21);
+  const float etau = fmaxf(e0, e1) + scale2<-21>(tau1 + 1.0f);
   float ex = 0.0f, bmax = 0.0f;
   leaf_bounds(lf, lv, s.brick, lod_min, s.leaf_lo, s.bl, s.bh);
 #pragma unroll
@@ -1177,11 +1257,11 @@ __device__ __forceinline__ void setup_segment(const RenderArgs& A, const RayF& r
     g.b0[a] = fmaf(xm, lv.inv_sc, lo05);
     g.db[a] = dtau * rf.Dd[a] * lv.inv_sc;
     const float ea = fabsf(rf.Dd[a]) * etau +
-                     ldexpf(fabsf(rf.Xe[a]) + fabsf(xm) + nfl * fabsf(dtau * rf.Dd[a]) + 1.0f, -21);
+                     scale2<-21>(fabsf(rf.Xe[a]) + fabsf(xm) + nfl * fabsf(dtau * rf.Dd[a]) + 1.0f);
     ex = fmaxf(ex, ea);
     bmax = fmaxf(bmax, fabsf(g.b0[a]) + nfl * fabsf(g.db[a]) + (float)s.brick.dim[a]);
   }
-  s.margin = ex * lv.inv_sc + ldexpf(bmax + 2.0f, -21);
+  s.margin = ex * lv.inv_sc + scale2<-21>(bmax + 2.0f);
 }
 
 // Secondary ray from a sample to the point light (the global-illumination example of
@@ -1387,7 +1467,9 @@ __device__ __forceinline__ void phong(const RenderArgs& A, const DLevel& lv, con
   const float gf = A.gfloor_num / lv.hmin;
   const float den = fmaxf(gn, gf);
   const float inv = den > 0.0f ? 1.0f / den : 0.0f;
-  const float ndl = fabsf((gr[0] * Lx + gr[1] * Ly + gr[2] * Lz) * inv);
+  // explicit order: every kernel rounds the product alike, whatever it is inlined into
+  const float dot = fmaf(gr[2], Lz, fmaf(gr[0], Lx, __fmul_rn(gr[1], Ly)));
+  const float ndl = fabsf(dot * inv);
   const float spec = A.ks * __powf(ndl, A.shininess);
   const float diff = fmaf(A.kd, ndl, A.ka);
   cr = fminf(fmaxf(fmaf(cr, diff, spec), 0.0f), 1.0f);
@@ -1458,15 +1540,13 @@ __device__ __forceinline__ bool sample_one(const RenderArgs& A, const RayArgs& R
 
 // Samples of a segment whose stencil maxima are tested in groups (stencil-maximum bricks):
 // the maxima of G consecutive samples are loaded together, so a run of transparent
-// samples pays one load latency per group; a sample that may be opaque is then evaluated
-// in full.  Every sample is counted as it is taken, in order.  Unshaded, the group's
-// evaluations are unrolled; shaded (a large evaluation) they run in a rolled loop that
-// rotates the loaded maxima through registers.  G = 0 (shaded): one test per sample.
+// samples pays one load latency per group, and the test leaves a mask of the samples that
+// may be opaque, which are then evaluated in full, in order.
 #ifndef AMR_MAX_GROUP_PLAIN
-#define AMR_MAX_GROUP_PLAIN 4
+#define AMR_MAX_GROUP_PLAIN 8
 #endif
 #ifndef AMR_MAX_GROUP_SHADED
-#define AMR_MAX_GROUP_SHADED 4
+#define AMR_MAX_GROUP_SHADED 8
 #endif
 
 // Sample k of a segment whose stencil maximum did not prove it transparent: its value
@@ -1491,76 +1571,44 @@ __device__ __forceinline__ bool sample_candidate(const RenderArgs& A, const RayA
 
 template <int ST, int SHADE, int G>
 __device__ __forceinline__ bool sample_segment_grouped(const RenderArgs& A, const RayArgs& R,
-                                                       const float4* s_tf, const int* nz,
+                                                       const float4* s_tf, float clear_below,
                                                        const SegSetup& g, const DLevel& lv,
                                                        float Lx, float Ly, float Lz, float& C0,
                                                        float& C1, float& C2, float& Acc,
                                                        unsigned& nsamp) {
   const int n = g.s.n;
-  if constexpr (G == 0) {
-    for (int k = 0; k < n; ++k) {
-      ++nsamp;
-      float beta[3];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) beta[a] = fmaf((float)k, g.db[a], g.b0[a]);
-      const Stencil<ST> st = stencil_at<ST>(g.s.brick, beta[0], beta[1], beta[2]);
-      if (stencil_transparent(A, nz, fetch_max<ST>(A, g.s.brick, st.l0))) continue;
-      const float v = stencil_value<ST>(A, g.s.brick, st);
-      if (composite_sample<ST, 1, SHADE>(A, R, s_tf, g, lv, k, beta, v, Lx, Ly, Lz, C0, C1, C2,
-                                         Acc))
+  MaxWalk<ST> walk;
+  walk.start(A, g);
+  for (int k0 = 0; k0 < n; k0 += G) {
+    const int cnt = min(G, n - k0);
+    unsigned mask = 0xffffffffu;
+    if (walk.inside) mask = walk.template opaque_mask<G>(k0, n, clear_below);
+    mask &= (1u << cnt) - 1u;
+    nsamp += cnt;
+    while (mask != 0) {
+      const int q = __ffs(mask) - 1;
+      mask &= mask - 1;
+      if (sample_candidate<ST, SHADE>(A, R, s_tf, g, lv, k0 + q, Lx, Ly, Lz, C0, C1, C2, Acc)) {
+        nsamp -= (unsigned)(cnt - 1 - q);  // early ray termination
         return true;
-    }
-    return false;
-  } else {
-    for (int k0 = 0; k0 < n; k0 += G) {
-      float m[G];
-#pragma unroll
-      for (int j = 0; j < G; ++j) {
-        const int k = min(k0 + j, n - 1);
-        const Stencil<ST> st = stencil_at<ST>(g.s.brick, fmaf((float)k, g.db[0], g.b0[0]),
-                                              fmaf((float)k, g.db[1], g.b0[1]),
-                                              fmaf((float)k, g.db[2], g.b0[2]));
-        m[j] = fetch_max<ST>(A, g.s.brick, st.l0);
-      }
-      auto one = [&](int k, float mk) -> int {  // 1: stop (early termination)
-        ++nsamp;
-        if (stencil_transparent(A, nz, mk)) return 0;  // opacity zero: nothing to composite
-        return sample_candidate<ST, SHADE>(A, R, s_tf, g, lv, k, Lx, Ly, Lz, C0, C1, C2, Acc)
-                   ? 1 : 0;
-      };
-      if constexpr ((SHADE & 3) == 0) {
-#pragma unroll
-        for (int j = 0; j < G; ++j) {
-          if (k0 + j >= n) break;
-          if (one(k0 + j, m[j])) return true;
-        }
-      } else {
-#pragma unroll 1
-        for (int j = 0; j < G; ++j) {
-          if (k0 + j >= n) break;
-          const float mj = m[0];
-#pragma unroll
-          for (int q = 0; q + 1 < G; ++q) m[q] = m[q + 1];
-          if (one(k0 + j, mj)) return true;
-        }
       }
     }
-    return false;
   }
+  return false;
 }
 
 // March the samples of one segment front to back.  Returns true when early ray
-// termination stops the ray inside the segment.  nz: the prefix counts of the transfer
-// function's non-transparent entries (read by the stencil-maximum test only).
+// termination stops the ray inside the segment.  clear_below: the threshold of the
+// stencil-maximum test (tf_threshold_warp; read by that test only).
 template <int ST, int INTERP, int SHADE>
 __device__ __forceinline__ bool sample_segment(const RenderArgs& A, const RayArgs& R,
-                                               const float4* s_tf, const int* nz,
+                                               const float4* s_tf, float clear_below,
                                                const SegSetup& g, const DLevel& lv, float Lx,
                                                float Ly, float Lz, float& C0, float& C1, float& C2,
                                                float& Acc, unsigned& nsamp) {
   if constexpr (INTERP == 1 && (SHADE & kShadeMaxBit) != 0) {
     constexpr int G = (SHADE & 3) == 0 ? AMR_MAX_GROUP_PLAIN : AMR_MAX_GROUP_SHADED;
-    return sample_segment_grouped<ST, SHADE, G>(A, R, s_tf, nz, g, lv, Lx, Ly, Lz, C0, C1, C2,
+    return sample_segment_grouped<ST, SHADE, G>(A, R, s_tf, clear_below, g, lv, Lx, Ly, Lz, C0, C1, C2,
                                                 Acc, nsamp);
   } else if constexpr (INTERP == 1 && SHADE == 0) {
     // software pipeline: the cells of sample k + 1 are requested before sample k is
@@ -1617,8 +1665,9 @@ constexpr int kMinBlocks = (SHADE & 3) == 0 ? AMR_MIN_BLOCKS_PLAIN : AMR_MIN_BLO
 // sampling and compositing.  Returns premultiplied RGBA; adds to nsamp and status.
 template <int ST, int INTERP, int SHADE>
 __device__ __forceinline__ float4 march_ray(const RenderArgs& A, const RayArgs& R, int i, int j,
-                                            const float4* s_tf, const int* s_nz, RayF& rf,
-                                            unsigned& nsamp, unsigned long long& status) {
+                                            const float4* s_tf, const int* s_nz,
+                                            float clear_below, RayF& rf, unsigned& nsamp,
+                                            unsigned long long& status) {
   float C0 = 0.f, C1 = 0.f, C2 = 0.f, Acc = 0.f;
   RayX rx;
   if (make_ray(R, i, j, rx)) {
@@ -1662,7 +1711,7 @@ __device__ __forceinline__ float4 march_ray(const RenderArgs& A, const RayArgs& 
       }
       SegSetup g;
       setup_segment(A, rf, lf, lv, lid, pid0, pid1, tau0, e0, tau1, e1, n, i, j, g, lmin);
-      if (sample_segment<ST, INTERP, SHADE>(A, R, s_tf, s_nz, g, lv, Lx, Ly, Lz, C0, C1, C2, Acc,
+      if (sample_segment<ST, INTERP, SHADE>(A, R, s_tf, clear_below, g, lv, Lx, Ly, Lz, C0, C1, C2, Acc,
                                             nsamp))
         pid1 = kPidOut;  // early ray termination
       pid0 = pid1;
@@ -1673,19 +1722,54 @@ __device__ __forceinline__ float4 march_ray(const RenderArgs& A, const RayArgs& 
   return make_float4(C0, C1, C2, Acc);
 }
 
-// Stage a transfer function in shared memory with the prefix count of its non-transparent
-// entries (nz[k] = entries before k with alpha != 0), for exact empty-space skipping.
-__device__ __forceinline__ void stage_tf(const float4* __restrict__ tf, int n, float4* s_tf,
-                                         int* s_nz, int tid, int nthreads) {
-  for (int k = tid; k < n; k += nthreads) s_tf[k] = tf[k];
-  __syncthreads();
-  if (tid == 0) {
-    int acc = 0;
-    s_nz[0] = 0;
-    for (int k = 0; k < n; ++k) {
-      acc += s_tf[k].w != 0.0f ? 1 : 0;
-      s_nz[k + 1] = acc;
+// Prefix counts of a transfer function's non-transparent entries (nz[k] = entries before k
+// with alpha != 0), written by one warp, 32 entries a step.
+__device__ __forceinline__ void tf_prefix_warp(const float4* __restrict__ tf, int n, int* nz,
+                                               int lane) {
+  int base = 0;
+  if (lane == 0) nz[0] = 0;
+  for (int k0 = 0; k0 < n; k0 += 32) {
+    const int k = k0 + lane;
+    const unsigned b = __ballot_sync(0xffffffffu, k < n && tf[k].w != 0.0f);
+    if (k < n) nz[k + 1] = base + __popc(b & (0xffffffffu >> (31 - lane)));
+    base += __popc(b);
+  }
+  __syncwarp();
+}
+
+// The smallest float that stencil_transparent does not call transparent (+inf: none), by
+// bisection over the ordered floats, 32 probes a step: the test is monotone in its value, so
+// m < threshold decides it exactly, without its table index and load.  (A NaN compares
+// false, so it is evaluated in full.)  All 32 lanes of a warp call this together.
+__device__ __forceinline__ float tf_threshold_warp(const RenderArgs& A, const int* nz, int lane) {
+  auto value = [](uint32_t key) {
+    return __uint_as_float((key & 0x80000000u) ? key ^ 0x80000000u : ~key);
+  };
+  uint32_t lo = 0x007fffffu, hi = 0xff800000u;  // keys of -inf and +inf
+  while (lo < hi) {
+    const uint32_t step = (hi - lo) / 32u + 1u;
+    const uint32_t probe = min(lo + step * (uint32_t)lane, hi);
+    const unsigned opaque = __ballot_sync(0xffffffffu, !stencil_transparent(A, nz, value(probe)));
+    if (opaque == 0) {
+      lo = min(lo + step * 31u, hi - 1u) + 1u;
+    } else {
+      const int f = __ffs(opaque) - 1;
+      hi = min(lo + step * (uint32_t)f, hi);
+      if (f > 0) lo = lo + step * (uint32_t)(f - 1) + 1u;
     }
+  }
+  return value(hi);
+}
+
+// Stage a transfer function in shared memory with its prefix counts (for exact empty-space
+// skipping) and the threshold of the stencil-maximum test.
+__device__ __forceinline__ void stage_tf(const RenderArgs& A, float4* s_tf, int* s_nz,
+                                         float* s_clear, int tid, int nthreads) {
+  for (int k = tid; k < A.tf_n; k += nthreads) s_tf[k] = A.tf[k];
+  if (tid < 32) {
+    tf_prefix_warp(A.tf, A.tf_n, s_nz, tid);
+    const float t = tf_threshold_warp(A, s_nz, tid);
+    if (tid == 0) *s_clear = t;
   }
   __syncthreads();
 }
@@ -1711,7 +1795,9 @@ __global__ void __launch_bounds__(128, kMinBlocks<SHADE>)
   float4* s_tf = smem;
   int* s_nz = reinterpret_cast<int*>(smem + A.tf_n);
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-  stage_tf(A.tf, A.tf_n, s_tf, s_nz, tid, blockDim.x * blockDim.y);
+  __shared__ float s_clear;
+  stage_tf(A, s_tf, s_nz, &s_clear, tid, blockDim.x * blockDim.y);
+  const float clear_below = s_clear;
   const int lane = tid & 31;
   const RayArgs& R = A.ray;
   unsigned nsamp = 0;
@@ -1726,11 +1812,12 @@ __global__ void __launch_bounds__(128, kMinBlocks<SHADE>)
         // padding word keeps the odd-sized slots free of bank conflicts.
         __shared__ RayFSlot s_rf[128];
         A.out[(size_t)jr * R.width + i] =
-            march_ray<ST, INTERP, SHADE>(A, R, i, j, s_tf, s_nz, s_rf[tid].f, nsamp, status);
+            march_ray<ST, INTERP, SHADE>(A, R, i, j, s_tf, s_nz, clear_below, s_rf[tid].f, nsamp,
+                                         status);
       } else {
         RayF rf;
         A.out[(size_t)jr * R.width + i] =
-            march_ray<ST, INTERP, SHADE>(A, R, i, j, s_tf, s_nz, rf, nsamp, status);
+            march_ray<ST, INTERP, SHADE>(A, R, i, j, s_tf, s_nz, clear_below, rf, nsamp, status);
       }
     }
   };

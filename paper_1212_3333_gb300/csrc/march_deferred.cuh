@@ -22,24 +22,24 @@
 
 namespace amr {
 
-// An opaque sample waiting for its colour: position and segment, transfer-function colour
-// and compositing weight w = (1 - A) alpha.  19 words (odd, so a warp writing one task per
-// lane hits distinct banks).
+// An opaque sample waiting for its colour: position and segment, value (its transfer-function
+// colour is looked up again) and compositing weight w = (1 - A) alpha.  11 words (odd, so a
+// warp writing one task per lane hits distinct banks).
 struct ShadeTask {
   float beta[3];  // brick coordinates
-  float cr, cg, cb;
+  float v;
   float w;
   float margin;   // bound on the FP32 position error (brick units)
-  float Lx, Ly, Lz;
   int leaf;       // packed leaf id and pruning bound
-  int pid0, pid1, n, k;
-  int px, py;
+  int pid0, pid1, n;
+  int k_lane;     // sample number (bits 0..22) and the lane whose ray it belongs to (23..27)
 };
 
+// Ring of queued samples: at most 31 wait before a step adds up to 32.
+constexpr int kDeferRing = 64;
 struct DeferArea {
-  ShadeTask task[32];
+  ShadeTask task[kDeferRing];
   float3 col[32];
-  float T[32];    // secondary rays: transmittance from each task's sample to the light
 };
 
 // resident blocks per SM the register budget allows for (measured on C2, Phong, 2048^2 /
@@ -57,11 +57,13 @@ __device__ __forceinline__ float3 task_point(const RenderArgs& A, const ShadeTas
                      (t.beta[2] - 0.5f + (float)lf.blo[2]) * sc);
 }
 
-// Colour of queued sample t (what composite_sample computes for an opaque sample); T is
-// its transmittance to the light when SHADOW is set.
+// Colour of queued sample t of pixel (px, py), headlight direction (Lx, Ly, Lz): what
+// composite_sample computes for an opaque sample; T is its transmittance to the light when
+// SHADOW is set.
 template <int ST, int GB, bool SHADOW = false>
 __device__ __forceinline__ float3 shade_task(const RenderArgs& A, const RayArgs& R,
-                                             const ShadeTask& t, float T = 1.0f) {
+                                             const float4* s_tf, const ShadeTask& t, int px,
+                                             int py, float Lx, float Ly, float Lz, float T) {
   const DLeaf lf = A.leaves[leaf_of(t.leaf)];
   const DLevel& lv = A.lv[lf.level];
   SegState s;
@@ -73,13 +75,14 @@ __device__ __forceinline__ float3 shade_task(const RenderArgs& A, const RayArgs&
   s.pid0 = t.pid0;
   s.pid1 = t.pid1;
   s.n = t.n;
-  s.px = t.px;
-  s.py = t.py;
+  s.px = px;
+  s.py = py;
   const float beta[3] = {t.beta[0], t.beta[1], t.beta[2]};
   float gr[3];
-  gradient<ST, 1, GB>(A, R, s, beta, t.k, lv, gr);
-  float cr = t.cr, cg = t.cg, cb = t.cb;
-  phong(A, lv, gr, t.Lx, t.Ly, t.Lz, cr, cg, cb);
+  gradient<ST, 1, GB>(A, R, s, beta, t.k_lane & ((1 << kTaskSampleBits) - 1), lv, gr);
+  const float4 c = tf_lookup(s_tf, A.tf_n, t.v, A.vmin, A.inv_range);
+  float cr = c.x, cg = c.y, cb = c.z;
+  phong(A, lv, gr, Lx, Ly, Lz, cr, cg, cb);
   if constexpr (SHADOW) {
     const float I = fmaf(1.0f - A.light_ambient, T, A.light_ambient);
     cr *= I;
@@ -92,16 +95,20 @@ __device__ __forceinline__ float3 shade_task(const RenderArgs& A, const RayArgs&
 // The march of pixel (i, j) of view R by one lane of a warp whose 32 lanes all call this
 // together (lanes without a pixel pass active = false); Q is the warp's queue area.
 // Returns premultiplied RGBA (zero for inactive lanes); adds to nsamp and status.
-// samples whose stencil maxima the deferred loop loads together (stencil-maximum bricks)
+// samples whose stencil maxima (with stencil-maximum bricks) or values (without) the
+// deferred loop loads together
 #ifndef AMR_DEFER_GROUP
 #define AMR_DEFER_GROUP 8
 #endif
-constexpr int kDeferGroup = AMR_DEFER_GROUP;
+#ifndef AMR_DEFER_VALUES
+#define AMR_DEFER_VALUES 2
+#endif
 
 template <int ST, int SHADE>
 __device__ __forceinline__ float4 march_deferred(const RenderArgs& A, const RayArgs& R, int i,
                                                  int j, bool active, const float4* s_tf,
-                                                 const int* s_nz, DeferArea& Q, unsigned& nsamp,
+                                                 const int* s_nz, float clear_below,
+                                                 DeferArea& Q, unsigned& nsamp,
                                                  unsigned long long& status) {
   constexpr bool MX = (SHADE & kShadeMaxBit) != 0;  // the stencil-maximum test
   const unsigned FULL = 0xffffffffu;
@@ -126,45 +133,52 @@ __device__ __forceinline__ float4 march_deferred(const RenderArgs& A, const RayA
   float tau0 = 0.f, e0 = 0.f;
   uint32_t start = 0;
   SegSetup g;
+  MaxWalk<ST> walk;
   g.s.n = 0;
   int k = 0;
-  int queued = 0;      // warp-uniform: tasks in the queue
-  unsigned mine = 0;   // this lane's queue slots
+  int queued = 0, head = 0;      // warp-uniform: tasks in the ring, and the first one's slot
+  unsigned long long mine = 0;   // bit p: the p-th queued task is this lane's
 
-  // shade every queued task (one per lane), then each lane adds its own colours in order;
-  // with secondary rays the whole warp first marches each task's light ray together
-  auto drain = [&]() {
+  // shade the first `count` queued tasks (one per lane), then each lane adds its own colours
+  // in order; with secondary rays the whole warp first marches each task's light ray together
+  auto drain = [&](int count) {
     __syncwarp();
+    float T = 1.0f;
     if constexpr ((SHADE & kShadeShadow) != 0) {
-      for (int q = 0; q < queued; ++q) {
-        const float3 x = task_point(A, Q.task[q]);
-        const float T = warp_shadow_transmittance<ST>(A, R, s_tf, x.x, x.y, x.z);
-        if (lane == 0) Q.T[q] = T;
+      for (int q = 0; q < count; ++q) {
+        const float3 x = task_point(A, Q.task[(head + q) & (kDeferRing - 1)]);
+        const float Tq = warp_shadow_transmittance<ST>(A, R, s_tf, x.x, x.y, x.z);
+        if (lane == q) T = Tq;
       }
-      __syncwarp();
     }
-    if (lane < queued)
+    const ShadeTask& t = Q.task[(head + lane) & (kDeferRing - 1)];
+    const int owner = lane < count ? t.k_lane >> kTaskSampleBits : lane;
+    const int px = __shfl_sync(FULL, i, owner), py = __shfl_sync(FULL, j, owner);
+    const float tx = __shfl_sync(FULL, Lx, owner), ty = __shfl_sync(FULL, Ly, owner),
+                tz = __shfl_sync(FULL, Lz, owner);
+    if (lane < count)
       Q.col[lane] = shade_task<ST, (SHADE & 3) == 2, (SHADE & kShadeShadow) != 0>(
-          A, R, Q.task[lane], Q.T[lane]);
+          A, R, s_tf, t, px, py, tx, ty, tz, T);
     __syncwarp();
-    for (unsigned m = mine; m != 0; m &= m - 1) {
+    for (unsigned m = (unsigned)mine & (0xffffffffu >> (32 - count)); m != 0; m &= m - 1) {
       const int q = __ffs(m) - 1;
-      const float w = Q.task[q].w;
+      const float w = Q.task[(head + q) & (kDeferRing - 1)].w;
       const float3 c = Q.col[q];
       C0 = fmaf(w, c.x, C0);
       C1 = fmaf(w, c.y, C1);
       C2 = fmaf(w, c.z, C2);
     }
     __syncwarp();
-    queued = 0;
-    mine = 0;
+    queued -= count;
+    head += count;
+    mine >>= count;
   };
 
   // Every pass either fetches segments for at least one lane or takes samples, and each
   // ray has finitely many of both, so the loop ends with every lane's ray finished.
   for (;;) {
-    const unsigned live_mask = __ballot_sync(FULL, live);
-    if (live_mask == 0) break;
+    const bool flush = !__any_sync(FULL, live);  // every ray has ended: only the ring is left
+    if (flush && queued == 0) break;
     // lanes whose segment ended fetch their next non-empty one (measured on C2: fetching
     // as soon as any lane needs beats waiting for a quarter or half of them)
     const bool need = live && k >= g.s.n;
@@ -205,6 +219,7 @@ __device__ __forceinline__ float4 march_deferred(const RenderArgs& A, const RayA
           continue;
         }
         setup_segment(A, rf, lf, lv, lid, pid0, pid1, tau0, e0, tau1, e1, n, i, j, g, lmin);
+        if constexpr (MX) walk.start(A, g);
         k = 0;
         pid0 = pid1;  // where the next segment starts
         tau0 = tau1;
@@ -212,89 +227,90 @@ __device__ __forceinline__ float4 march_deferred(const RenderArgs& A, const RayA
         break;
       }
     }
-    // one sample step of every lane (the queue operations are warp-wide); mj: the sample's
-    // stencil maximum when the stencil-maximum test is on
-    auto take = [&](float mj) {
-      bool opaque = false;
-      float beta[3], cr = 0.f, cg = 0.f, cb = 0.f, w = 0.f;
-      if (live && k < g.s.n) {
-        ++nsamp;
+    // A lane takes its next G samples at a time: a mask of those that may be opaque (by
+    // their stencil maxima, or by their values), then, in step with the other lanes, each
+    // sample of the mask in order.  Most masks are empty, so the warp-wide steps are few.
+    constexpr int G = MX ? AMR_DEFER_GROUP : AMR_DEFER_VALUES;
+    for (int step = 0; step < A.samples_per_iter; step += G) {
+      const int kb = k;
+      const int cnt = live ? min(min(G, A.samples_per_iter - step), g.s.n - k) : 0;
+      unsigned mask = 0;
+      float val[MX ? 1 : G];
+      if (cnt > 0) {
+        if constexpr (MX) {
+          if (walk.inside) mask = walk.template opaque_mask<G>(kb, g.s.n, clear_below);
+          else mask = 0xffffffffu;
+        } else {
 #pragma unroll
-        for (int a = 0; a < 3; ++a) beta[a] = fmaf((float)k, g.db[a], g.b0[a]);
-        if (!(MX && stencil_transparent(A, s_nz, mj))) {  // else opacity zero
-          const float v = trilinear<ST>(A, g.s.brick, beta[0], beta[1], beta[2]);
-          const float4 c = tf_lookup(s_tf, A.tf_n, v, A.vmin, A.inv_range);
-          if (c.w > 0.0f) {
-            const float alpha = -expm1f(-A.kappa * c.w * g.delta);
-            w = (1.0f - Acc) * alpha;
-            Acc += w;
-            cr = c.x;
-            cg = c.y;
-            cb = c.z;
-            opaque = true;
+          for (int q = 0; q < G; ++q) {
+            const float kk = (float)min(kb + q, g.s.n - 1);
+            val[q] = trilinear<ST>(A, g.s.brick, fmaf(kk, g.db[0], g.b0[0]),
+                                   fmaf(kk, g.db[1], g.b0[1]), fmaf(kk, g.db[2], g.b0[2]));
           }
-        }
-        ++k;
-      }
-      const unsigned om = __ballot_sync(FULL, opaque);
-      if (om != 0) {
-        if (queued + __popc(om) > 32) drain();
-        if (opaque) {
-          const int q = queued + __popc(om & lt_mask);
-          ShadeTask& t = Q.task[q];
-          t.beta[0] = beta[0];
-          t.beta[1] = beta[1];
-          t.beta[2] = beta[2];
-          t.cr = cr;
-          t.cg = cg;
-          t.cb = cb;
-          t.w = w;
-          t.margin = g.s.margin;
-          t.Lx = Lx;
-          t.Ly = Ly;
-          t.Lz = Lz;
-          t.leaf = g.s.leaf;
-          t.pid0 = g.s.pid0;
-          t.pid1 = g.s.pid1;
-          t.n = g.s.n;
-          t.k = k - 1;
-          t.px = i;
-          t.py = j;
-          mine |= 1u << q;
-          if (Acc >= A.ert_thresh) live = false;  // early ray termination
-        }
-        queued += __popc(om);
-      }
-    };
-    if constexpr (MX) {
-      // the stencil maxima of a lane's next kDeferGroup samples are loaded together, then
-      // the steps take them in a rolled loop that rotates them through registers
-      for (int step = 0; step < A.samples_per_iter;) {
-        float m[kDeferGroup];
 #pragma unroll
-        for (int q = 0; q < kDeferGroup; ++q) {
-          m[q] = __int_as_float(0x7f800000);
-          if (live && k < g.s.n) {
-            const int kk = min(k + q, g.s.n - 1);
-            const Stencil<ST> st = stencil_at<ST>(g.s.brick, fmaf((float)kk, g.db[0], g.b0[0]),
-                                                  fmaf((float)kk, g.db[1], g.b0[1]),
-                                                  fmaf((float)kk, g.db[2], g.b0[2]));
-            m[q] = fetch_max<ST>(A, g.s.brick, st.l0);
+          for (int q = 0; q < G; ++q) mask |= val[q] < clear_below ? 0u : 1u << q;
+        }
+        mask &= (1u << cnt) - 1u;
+        k += cnt;
+        nsamp += cnt;
+      }
+      for (;;) {
+        const bool some = __any_sync(FULL, mask != 0);
+        if (some) {
+          bool opaque = false;
+          int kk = 0;
+          float beta[3], v = 0.f, w = 0.f;
+          if (mask != 0) {
+            const int q = __ffs(mask) - 1;
+            mask &= mask - 1;
+            kk = kb + q;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) beta[a] = fmaf((float)kk, g.db[a], g.b0[a]);
+            if constexpr (MX) {
+              v = trilinear<ST>(A, g.s.brick, beta[0], beta[1], beta[2]);
+            } else {
+              v = val[0];
+#pragma unroll
+              for (int e = 1; e < G; ++e) v = q == e ? val[e] : v;
+            }
+            const float a_tf = tf_alpha(s_tf, A.tf_n, v, A.vmin, A.inv_range);
+            if (a_tf > 0.0f) {
+              const float alpha = -expm1f(-A.kappa * a_tf * g.delta);
+              w = (1.0f - Acc) * alpha;
+              Acc += w;
+              opaque = true;
+              if (Acc >= A.ert_thresh) {  // early ray termination
+                nsamp -= (unsigned)(kb + cnt - 1 - kk);
+                live = false;
+                mask = 0;
+              }
+            }
           }
+          const unsigned om = __ballot_sync(FULL, opaque);
+          if (opaque) {
+            const int q = queued + __popc(om & lt_mask);
+            ShadeTask& t = Q.task[(head + q) & (kDeferRing - 1)];
+            t.beta[0] = beta[0];
+            t.beta[1] = beta[1];
+            t.beta[2] = beta[2];
+            t.v = v;
+            t.w = w;
+            t.margin = g.s.margin;
+            t.leaf = g.s.leaf;
+            t.pid0 = g.s.pid0;
+            t.pid1 = g.s.pid1;
+            t.n = g.s.n;
+            t.k_lane = kk | (lane << kTaskSampleBits);
+            mine |= 1ull << q;
+          }
+          queued += __popc(om);
         }
-#pragma unroll 1
-        for (int jj = 0; jj < kDeferGroup && step < A.samples_per_iter; ++jj, ++step) {
-          const float mj = m[0];
-#pragma unroll
-          for (int q = 0; q + 1 < kDeferGroup; ++q) m[q] = m[q + 1];
-          take(mj);
-        }
+        if (queued >= 32 || (flush && queued != 0)) drain(min(queued, 32));
+        else if (!some) break;
       }
-    } else {
-      for (int step = 0; step < A.samples_per_iter; ++step) take(0.0f);
+      if (flush) break;
     }
   }
-  if (queued != 0) drain();
   return make_float4(C0, C1, C2, Acc);
 }
 
@@ -303,6 +319,19 @@ __device__ __forceinline__ float4 march_deferred(const RenderArgs& A, const RayA
 template <int ST, int SHADE>
 __global__ void __launch_bounds__(128, AMR_MIN_BLOCKS_DEFERRED)
     deferred_kernel(const __grid_constant__ RenderArgs A) {
+  // every tile of the image, or (with a workspace) those the split march left: the tiles it
+  // gave up for lack of room and did not take up again, the dense ones, and the ones it did not
+  // start
+  const int all_tiles = ((A.ray.width + 7) / 8) * ((A.ray.rows + 3) / 4);
+  const bool rest = A.ts.heads != nullptr;
+  int left = 0, dense = 0, retried = 0, begun = all_tiles;
+  if (rest) {
+    retried = (int)__ldcg(A.ts.heads + kHeadRest);
+    left = (int)__ldcg(A.ts.heads + kHeadLeft) - retried;
+    dense = (int)__ldcg(A.ts.heads + kHeadDense);
+    begun = (int)min(__ldcg(A.ts.heads + kHeadTile), (unsigned)all_tiles);
+    if (left == 0 && dense == 0 && begun == all_tiles) return;
+  }
   extern __shared__ float4 smem[];
   float4* s_tf = smem;
   int* s_nz = reinterpret_cast<int*>(smem + A.tf_n);
@@ -310,11 +339,13 @@ __global__ void __launch_bounds__(128, AMR_MIN_BLOCKS_DEFERRED)
   const size_t tf_bytes = (size_t)A.tf_n * sizeof(float4) + (size_t)(A.tf_n + 1) * sizeof(int);
   DeferArea& Q = reinterpret_cast<DeferArea*>(reinterpret_cast<char*>(smem) +
                                               ((tf_bytes + 15) & ~(size_t)15))[tid >> 5];
-  stage_tf(A.tf, A.tf_n, s_tf, s_nz, tid, blockDim.x * blockDim.y);
+  __shared__ float s_clear;
+  stage_tf(A, s_tf, s_nz, &s_clear, tid, blockDim.x * blockDim.y);
+  const float clear_below = s_clear;
   const int lane = tid & 31;
   const RayArgs& R = A.ray;
   const int tiles_x = (R.width + 7) / 8;
-  const int n_tiles = tiles_x * ((R.rows + 3) / 4);
+  const int n_tiles = rest ? left + dense + all_tiles - begun : all_tiles;
   unsigned nsamp = 0;
   unsigned long long status = 0;
   // each pass takes one tile, and the queue hands out every tile once
@@ -326,11 +357,17 @@ __global__ void __launch_bounds__(128, AMR_MIN_BLOCKS_DEFERRED)
     }
     t = __shfl_sync(0xffffffffu, t, 0);
     if (t >= n_tiles) break;
+    if (rest) {
+      if (t < left) t = __ldcg(A.ts.left + retried + t);
+      else if (t < left + dense) t = __ldcg(A.ts.dense + t - left);
+      else t += begun - left - dense;
+    }
     const int i = (t % tiles_x) * 8 + (lane & 7);
     const int jr = (t / tiles_x) * 4 + (lane >> 3);
     const int j = R.row0 + jr;
     const bool active = i < R.width && jr < R.rows && j < R.height;
-    const float4 c = march_deferred<ST, SHADE>(A, R, i, j, active, s_tf, s_nz, Q, nsamp, status);
+    const float4 c = march_deferred<ST, SHADE>(A, R, i, j, active, s_tf, s_nz, clear_below, Q,
+                                              nsamp, status);
     if (active) A.out[(size_t)jr * R.width + i] = c;
   }
   const unsigned total = __reduce_add_sync(0xffffffffu, nsamp);

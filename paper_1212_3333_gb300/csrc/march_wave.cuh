@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(128) wave_kernel(const __grid_constant__ Rende
             const float dtau = (tau1 - tau0) / nfl;
             ws.delta = dtau * rf.dn;
             const float taum = fmaf(0.5f, dtau, tau0);
-            const float etau = fmaxf(e0, e1) + ldexpf(tau1 + 1.0f, -21);
+            const float etau = fmaxf(e0, e1) + scale2<-21>(tau1 + 1.0f);
             float ex = 0.0f, bmax = 0.0f;
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
@@ -155,11 +155,11 @@ __global__ void __launch_bounds__(128) wave_kernel(const __grid_constant__ Rende
               s.bl[a] = (float)(lf.lo[a] - s.brick.lo[a] * lv.sc) * lv.inv_sc + 0.5f;
               s.bh[a] = (float)(lf.hi[a] - s.brick.lo[a] * lv.sc) * lv.inv_sc + 0.5f;
               const float ea = fabsf(rf.Dd[a]) * etau +
-                               ldexpf(fabsf(rf.Xe[a]) + fabsf(xm) + nfl * fabsf(dtau * rf.Dd[a]) + 1.0f, -21);
+                               scale2<-21>(fabsf(rf.Xe[a]) + fabsf(xm) + nfl * fabsf(dtau * rf.Dd[a]) + 1.0f);
               ex = fmaxf(ex, ea);
               bmax = fmaxf(bmax, fabsf(b0) + nfl * fabsf(db) + (float)s.brick.dim[a]);
             }
-            s.margin = ex * lv.inv_sc + ldexpf(bmax + 2.0f, -21);
+            s.margin = ex * lv.inv_sc + scale2<-21>(bmax + 2.0f);
           }
           pid0 = pid1;
           tau0 = tau1;

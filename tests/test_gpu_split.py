@@ -1,0 +1,100 @@
+"""GPU checks of deferred shading through the task workspace (the split march): images and
+sample counts equal the per-ray schedule's bit for bit when the workspace goes through several
+rounds, gives tiles up and leaves some to the single-kernel march; when there is no workspace
+(a first call under stream capture); and the bounds on segments are reported for the same rays
+although a ray may be marched beyond the sample that ends it."""
+import numpy as np
+import pytest
+
+import synth
+from synth.amr import random_hierarchy
+from gpu_util import gpu_render, params_pair
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def amr():
+    import paper_1212_3333_gb300 as m
+
+    return m
+
+
+def _context(amr, seed=3, maxbrick=True, gradient=True):
+    h = random_hierarchy(seed, n0=12, num_levels=3, patches_per_level=6)
+    ctx = amr.from_hierarchy(h)
+    ctx.amr_build_kdtree("ptr", gradient=gradient, halo=2, maxbrick=maxbrick)
+    return ctx, h.value_range()
+
+
+def _opaque_tf(n=64, clear=16):
+    """Opaque but for its first `clear` entries (none: the split march leaves every tile)."""
+    tf = synth.ramp_tf(n)
+    tf[:, 3] = 1.0
+    tf[:clear, 3] = 0.0
+    return tf
+
+
+# samples per pixel from a few (one round) to far more than a tile may take (320 tasks per
+# pixel)
+@pytest.mark.parametrize("step", [0.5, 0.1, 0.01])
+@pytest.mark.parametrize("size", [(33, 29), (160, 121)])
+@pytest.mark.parametrize("maxbrick", [True, False])
+def test_full_workspace_equals_per_ray(amr, step, size, maxbrick):
+    ctx, (vmin, vmax) = _context(amr, maxbrick=maxbrick)
+    cam = synth.orbit_camera(2, *size)
+    for kappa, ert, clear in ((0.05, 0.0, 16), (3.0, 1e-3, 16), (0.05, 0.0, 0)):
+        got = []
+        for schedule in (0, 3):
+            p, _ = params_pair(amr, vmin, vmax, schedule=schedule, shade=1, step_factor=step,
+                               kappa=kappa, ert_eps=ert)
+            got.append(gpu_render(ctx, cam, _opaque_tf(clear=clear), p))
+        assert got[0][1] == got[1][1]
+        assert np.array_equal(got[0][0], got[1][0])
+
+
+def test_segment_bound_is_reported_for_the_same_rays(amr):
+    ctx, (vmin, vmax) = _context(amr)
+    cam = synth.orbit_camera(5, 40, 31)
+    seen = set()
+    for kappa in (0.5, 400.0):  # the second ends every ray in its first segments
+        for bound in (1, 2, 4, 64):
+            got = []
+            for schedule in (0, 3):
+                p, _ = params_pair(amr, vmin, vmax, schedule=schedule, shade=1, kappa=kappa,
+                                   ert_eps=0.2, max_segments=bound)
+                try:
+                    got.append(gpu_render(ctx, cam, _opaque_tf(clear=8), p))
+                except amr.AmrError as e:
+                    got.append(e.status)
+            seen.add(isinstance(got[0], int))
+            if isinstance(got[0], int):
+                assert got[0] == got[1]
+            else:
+                assert got[0][1] == got[1][1] and np.array_equal(got[0][0], got[1][0])
+    assert seen == {True, False}
+
+
+def test_first_call_captured(amr):
+    import torch
+
+    ctx, (vmin, vmax) = _context(amr)
+    cam = synth.orbit_camera(7, 61, 47)
+    tf = torch.as_tensor(_opaque_tf(), device="cuda")
+    p, _ = params_pair(amr, vmin, vmax, schedule=3, shade=1)
+    out = [torch.zeros((47, 61, 4), device="cuda") for _ in range(2)]
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):  # no workspace yet, and none may be allocated
+        ctx.amr_render(cam, tf, p, out[0])
+    ctx.amr_render(cam, tf, p, out[1])
+    g2 = torch.cuda.CUDAGraph()
+    again = torch.zeros_like(out[0])
+    with torch.cuda.graph(g2):  # with the workspace of the call before
+        ctx.amr_render(cam, tf, p, again)
+    big = torch.zeros((300, 400, 4), device="cuda")
+    ctx.amr_render(synth.orbit_camera(8, 400, 300), tf, p, big)  # a larger workspace
+    for graph in (g, g2):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert float(out[1].abs().max()) > 0
+    assert torch.equal(out[0], out[1]) and torch.equal(again, out[1])
