@@ -68,6 +68,40 @@ def test_mlp_gradient_matches_oracle(mods):
             assert a @ b / (np.linalg.norm(a) * np.linalg.norm(b)) >= 0.995, k
 
 
+# one row, the edges of a 128-row tile, a ragged batch, and more tiles than blocks (152)
+@pytest.mark.parametrize("n", [1, 16, 127, 128, 129, 1000, 152 * 128 + 5])
+def test_mlp_gradient_against_64_bits(mods, n):
+    """Against 64 bits with the forward's BF16 roundings in place.  FP32 sums leave about 1e-6;
+    a pre-activation within rounding of a BF16 boundary may fall the other way, which changes
+    its row's share of the gradient by up to 2^-7, and a few rows of n do."""
+    torch, amr, proposal = mods
+    rng = np.random.default_rng(n)
+    p = proposal.init_params(7) + rng.normal(0, 0.05, size=9217).astype(np.float32)
+    x = rng.uniform(-1, 1, size=(n, 12)).astype(np.float32)
+    t = rng.uniform(0, 1, size=n).astype(np.float32)
+    prop = proposal.Proposal(p)
+    prop.loss_grad(torch.as_tensor(x, device="cuda"), torch.as_tensor(t, device="cuda"))
+    torch.cuda.synchronize()
+    W1, b1, W2, b2, W3, b3, W4, b4 = _oracle_params(proposal, p)
+    acts = [bf16_round(x)]
+    for W, b in ((W1, b1), (W2, b2), (W3, b3)):
+        acts.append(bf16_round(np.maximum(acts[-1] @ W.T + b, 0.0)))
+    z = acts[3] @ W4[0] + b4[0]
+    d = ((1.0 / (1.0 + np.exp(-z)) - t) / n)[:, None]
+    ref = [None] * 8
+    for k, W in ((3, W4), (2, W3), (1, W2), (0, W1)):
+        ref[2 * k], ref[2 * k + 1] = (d.T @ acts[k]).ravel(), d.sum(0)
+        d = (d @ W) * (acts[k] > 0)
+    loss = np.mean(np.logaddexp(0.0, z) - t * z)
+    assert abs(float(prop.loss.item()) - loss) <= 1e-5 * loss
+    g = prop.grad.cpu().numpy().astype(np.float64)
+    k = 0
+    for r in ref:
+        err = np.linalg.norm(g[k:k + r.size] - r) / np.linalg.norm(r)
+        assert err <= 1e-5 + 2.0 ** -7 * np.sqrt(4.0 / n), (k, err)
+        k += r.size
+
+
 def test_adam_step_matches_formula(mods):
     torch, amr, proposal = mods
     rng = np.random.default_rng(2)
