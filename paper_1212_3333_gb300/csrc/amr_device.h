@@ -135,7 +135,7 @@ struct TaskSpace {
   float4* tasks;        // segment record, sample number | lane << 23, value, weight
   float4* col;          // per task: colour, weight
   int32_t* outer;       // tasks whose gradient leaves their leaf
-  int4* meta;           // per chunk: its tile, its tasks, the tile's next chunk
+  int4* meta;           // per chunk: its tile, its tasks, the tile's next chunk, its view
   float4* segs;         // 3 per record: first sample and step (brick coordinates), margin,
                         // packed leaf | plane ids, sample count
   int2* tile;           // per tile: first chunk and number of tasks to add up, or -1
@@ -143,6 +143,7 @@ struct TaskSpace {
   int32_t* dense;       // tiles given up because they take more than tile_chunks
   unsigned* heads;      // chunks, segment blocks, outer tasks, tiles handed out; left tiles,
                         // those of them handed out again, those of earlier rounds; dense tiles
+  struct RayArgs* views; // batches: per view its rays (rows of the whole image)
   int32_t chunks, seg_blocks;
   int32_t tile_chunks;  // most chunks of one tile
 };

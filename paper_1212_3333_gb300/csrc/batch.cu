@@ -12,6 +12,9 @@
 // addition for throughput over many small and large views.
 #include <cuda_runtime.h>
 
+#include <memory>
+#include <new>
+
 #include "ctx.h"
 #include "march_launch.cuh"
 
@@ -160,6 +163,34 @@ amr_status launch_batch(amr_ctx* c, const BatchArgs& b, int storage, int shade, 
   const bool mx = (shade & kShadeMaxBit) != 0;  // the stencil-maximum test
   shade &= ~kShadeMaxBit;
   if (storage != ST_PTR) return fail(c, AMR_ERR_ARG, "batched rendering needs the ptr storage (FP32)");
+  if (schedule == 3 && (shade == 1 || shade == 2)) {
+    // the split march over 8x4 tiles of all views, when the workspace has records for them
+    std::unique_ptr<BatchArgs> t(new (std::nothrow) BatchArgs(b));
+    if (!t) return fail(c, AMR_ERR_OOM, "out of host memory");
+    int64_t tiles = 0;
+    for (int v = 0; v < b.n_views; ++v) {
+      t->v[v].tiles_x = (b.v[v].width + 7) / 8;
+      t->v[v].item0 = (int32_t)std::min<int64_t>(tiles, INT32_MAX);
+      tiles += (int64_t)t->v[v].tiles_x * ((b.v[v].height + 3) / 4);
+    }
+    const TaskPlan plan = plan_tasks(c, tiles, stream);
+    if (tiles <= plan.tiles) {
+      t->n_items = (int32_t)tiles;
+      t->A.ts = plan.ts;
+      batch_views_kernel<<<1, kMaxBatchViews, 0, s>>>(*t);
+      cudaError_t e = cudaGetLastError();
+      const int rounds = plan.rounds(tiles);
+      if (e == cudaSuccess) {
+        if (shade == 1) e = mx ? launch_rounds<ST_PTR, 1 | kShadeMaxBit>(rounds, s, *t)
+                               : launch_rounds<ST_PTR, 1>(rounds, s, *t);
+        else e = mx ? launch_rounds<ST_PTR, 2 | kShadeMaxBit>(rounds, s, *t)
+                    : launch_rounds<ST_PTR, 2>(rounds, s, *t);
+      }
+      if (e != cudaSuccess)
+        return fail(c, AMR_ERR_CUDA, std::string("batch launch: ") + cudaGetErrorString(e));
+      return AMR_OK;
+    }
+  }
   if (schedule == 3) {
     if (shade == 1) return mx ? launch_st<ST_PTR, 1 | kShadeMaxBit, true>(c, b, cfg, s)
                               : launch_st<ST_PTR, 1, true>(c, b, cfg, s);

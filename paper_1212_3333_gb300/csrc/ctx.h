@@ -98,10 +98,11 @@ struct DeviceState {
   int64_t task_refused = INT64_MAX;  // a workspace for this many pixels could not be allocated
 };
 
-// How a call uses the workspace: rows per band (0: no workspace) and rounds per band.
+// The workspace of a call: the tiles it has records for (0: none), and the rounds for some.
 struct TaskPlan {
   TaskSpace ts = {};
-  int rows = 0, rounds = 0;
+  long long tiles = 0;
+  int rounds(long long tiles_of_band) const;
 };
 
 }  // namespace amr
@@ -147,9 +148,10 @@ amr_status pack_atlas(amr_ctx* c);
 // device.cpp
 amr_status upload(amr_ctx* c, void* stream);
 void release_device(amr_ctx* c);
-// The split march's workspace for an image or band, grown when it is too small and the stream
-// is not being captured; no rows when there is none (out of memory, or a first call captured).
-TaskPlan plan_tasks(amr_ctx* c, const RenderArgs& a, void* stream);
+// The split march's workspace for a call with that many 8x4 tiles, grown when it is too small
+// and the stream is not being captured; it may have fewer tiles (out of memory, or a first
+// call captured: none).
+TaskPlan plan_tasks(amr_ctx* c, long long tiles, void* stream);
 // kernels (march.cu)
 amr_status launch_render(amr_ctx* c, const RenderArgs& a, int storage, int interp, int shade,
                          int schedule, void* stream);

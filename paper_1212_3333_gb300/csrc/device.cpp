@@ -282,13 +282,13 @@ static int64_t task_rounds(int64_t pixels, int64_t chunks) {
   return std::min<int64_t>(64, (pixels * kDensePerPixel + usable - 1) / usable);
 }
 
-TaskPlan plan_tasks(amr_ctx* c, const RenderArgs& a, void* stream) {
+int TaskPlan::rounds(long long band) const { return (int)task_rounds(band * 32, ts.chunks); }
+
+TaskPlan plan_tasks(amr_ctx* c, long long call_tiles, void* stream) {
   TaskPlan plan;
   DeviceState& d = c->dev;
-  const int64_t tiles_x = (a.ray.width + 7) / 8, row_pixels = 32 * tiles_x;  // of a row of tiles
-  const int64_t tile_rows = (a.ray.rows + 3) / 4;
-  if (tile_rows <= 0 || tiles_x <= 0) return plan;
-  const int64_t want = std::min(tile_rows * row_pixels, std::max(kBandPixels, row_pixels));
+  if (call_tiles <= 0) return plan;
+  const int64_t want = std::min<int64_t>(call_tiles * 32, std::max<int64_t>(kBandPixels, 32 * 8192));
   if (want > d.task_pixels && want < d.task_refused) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing((cudaStream_t)stream, &cap) != cudaSuccess) cudaGetLastError();
@@ -299,17 +299,18 @@ TaskPlan plan_tasks(amr_ctx* c, const RenderArgs& a, void* stream) {
     const size_t slots = (size_t)chunks * kTaskChunk;
     const int64_t blocks = (int64_t)slots / 3 / kSegBlock + 2 * kWarps;
     const int64_t rounds = task_rounds(px, chunks);
-    const size_t sizes[9] = {slots * sizeof(float4), slots * sizeof(float4), slots * sizeof(int32_t),
+    const size_t sizes[10] = {slots * sizeof(float4), slots * sizeof(float4), slots * sizeof(int32_t),
                              (size_t)chunks * sizeof(int4),
                              (size_t)blocks * kSegBlock * 3 * sizeof(float4),
                              (size_t)tiles * sizeof(int2),
                              (size_t)(tiles * rounds) * sizeof(int32_t),
-                             (size_t)tiles * sizeof(int32_t), kHeads * sizeof(unsigned)};
-    size_t off[10] = {0};
-    for (int k = 0; k < 9; ++k) off[k + 1] = off[k] + ((sizes[k] + 255) & ~(size_t)255);
+                             (size_t)tiles * sizeof(int32_t), kHeads * sizeof(unsigned),
+                             kMaxBatchViews * sizeof(RayArgs)};
+    size_t off[11] = {0};
+    for (int k = 0; k < 10; ++k) off[k + 1] = off[k] + ((sizes[k] + 255) & ~(size_t)255);
     char* p = nullptr;
     if (cap == cudaStreamCaptureStatusNone) {
-      if (cudaMalloc((void**)&p, off[9]) != cudaSuccess) {
+      if (cudaMalloc((void**)&p, off[10]) != cudaSuccess) {
         cudaGetLastError();
         p = nullptr;
         d.task_refused = want;
@@ -327,16 +328,14 @@ TaskPlan plan_tasks(amr_ctx* c, const RenderArgs& a, void* stream) {
       d.tasks.left = (int32_t*)(p + off[6]);
       d.tasks.dense = (int32_t*)(p + off[7]);
       d.tasks.heads = (unsigned*)(p + off[8]);
+      d.tasks.views = (RayArgs*)(p + off[9]);
       d.tasks.tile_chunks = (int32_t)std::max<int64_t>(1, 3 * chunks / std::min(tiles, kWarps));
       d.tasks.chunks = (int32_t)chunks;
       d.tasks.seg_blocks = (int32_t)blocks;
     }
   }
-  const int64_t rows = d.task_pixels / row_pixels * 4;
-  if (rows <= 0) return plan;
   plan.ts = d.tasks;
-  plan.rows = (int)std::min<int64_t>(rows, tile_rows * 4);
-  plan.rounds = (int)task_rounds(plan.rows / 4 * row_pixels, d.tasks.chunks);
+  plan.tiles = d.task_pixels / 32;
   return plan;
 }
 

@@ -314,15 +314,117 @@ __device__ __forceinline__ float4 march_deferred(const RenderArgs& A, const RayA
   return make_float4(C0, C1, C2, Acc);
 }
 
-// Schedule 3: persistent warps taking 8x4-pixel tiles from the global queue (as
-// march_kernel does for the per-ray loop), each marching its tile with deferred shading.
-template <int ST, int SHADE>
+// An 8x4-pixel tile of a launch: of its one image, or of one of a batch's views.
+struct TileAt {
+  int tile, tiles_x;  // in its image
+  int tf;             // transfer function (batches)
+  int view;
+  float4* out;
+  int width, rows;
+
+  __device__ __forceinline__ void pixel(int lane, int& i, int& jr) const {
+    i = (tile % tiles_x) * 8 + (lane & 7);
+    jr = (tile / tiles_x) * 4 + (lane >> 3);
+  }
+  __device__ __forceinline__ size_t at(int i, int jr) const { return (size_t)jr * width + i; }
+};
+
+__device__ __forceinline__ const RenderArgs& render_args(const RenderArgs& A) { return A; }
+__device__ __forceinline__ const RenderArgs& render_args(const BatchArgs& B) { return B.A; }
+
+__device__ __forceinline__ int count_tiles(const RenderArgs& A) {
+  return ((A.ray.width + 7) / 8) * ((A.ray.rows + 3) / 4);
+}
+__device__ __forceinline__ int count_tiles(const BatchArgs& B) { return B.n_items; }
+
+__device__ __forceinline__ TileAt tile_at(const RenderArgs& A, int t) {
+  return {t, (A.ray.width + 7) / 8, 0, 0, A.out, A.ray.width, A.ray.rows};
+}
+__device__ __forceinline__ TileAt view_tile(const BatchArgs& B, int t, int view) {
+  const BatchView& v = B.v[view];
+  return {t - v.item0, v.tiles_x, v.tf, view, B.A.out + v.out, v.width, v.height};
+}
+__device__ __forceinline__ TileAt tile_at(const BatchArgs& B, int t) {
+  int lo = 0, hi = B.n_views - 1;  // last view whose first tile is <= t
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (B.v[mid].item0 <= t) lo = mid;
+    else hi = mid - 1;
+  }
+  return view_tile(B, t, lo);
+}
+// the tile of a chunk (its view is known)
+__device__ __forceinline__ TileAt chunk_tile(const RenderArgs& A, int4 meta) { return tile_at(A, meta.x); }
+__device__ __forceinline__ TileAt chunk_tile(const BatchArgs& B, int4 meta) {
+  return view_tile(B, meta.x, meta.w);
+}
+
+__device__ __forceinline__ const RayArgs& tile_rays(const RenderArgs& A, const TileAt&) { return A.ray; }
+__device__ __forceinline__ const RayArgs& tile_rays(const BatchArgs& B, const TileAt& p) {
+  return B.A.ts.views[p.view];
+}
+
+// Transfer functions for a launch's tiles: one image's staged in shared memory with its prefix
+// counts and threshold; a batch's read where they are (staging up to eight would take the L1
+// cache from the bricks), with their prefix counts and thresholds staged.
+template <typename Args>
+struct StagedTf;
+template <>
+struct StagedTf<RenderArgs> {
+  float4* s_tf;
+  int* s_nz;
+  float clear;
+  static __host__ __device__ size_t bytes(const RenderArgs& A) {
+    return (((size_t)A.tf_n * sizeof(float4) + (size_t)(A.tf_n + 1) * sizeof(int)) + 15) & ~(size_t)15;
+  }
+  __device__ __forceinline__ StagedTf(const RenderArgs& A, float4* smem, int tid) {
+    __shared__ float s_clear;
+    s_tf = smem;
+    s_nz = reinterpret_cast<int*>(smem + A.tf_n);
+    stage_tf(A, s_tf, s_nz, &s_clear, tid, 128);
+    clear = s_clear;
+  }
+  __device__ __forceinline__ const float4* tf(const TileAt&) const { return s_tf; }
+  __device__ __forceinline__ const int* nz(const TileAt&) const { return s_nz; }
+  __device__ __forceinline__ float clear_below(const TileAt&) const { return clear; }
+};
+template <>
+struct StagedTf<BatchArgs> {
+  const float4* all;
+  int* s_nz;
+  const float* s_clear;
+  int n;
+  static __host__ __device__ size_t bytes(const BatchArgs& B) {
+    return ((size_t)B.n_tf * (B.A.tf_n + 1) * sizeof(int) + 15) & ~(size_t)15;
+  }
+  __device__ __forceinline__ StagedTf(const BatchArgs& B, float4* smem, int tid) {
+    __shared__ float below[8];
+    all = B.A.tf;
+    s_nz = reinterpret_cast<int*>(smem);
+    s_clear = below;
+    n = B.A.tf_n;
+    for (int t = tid >> 5; t < B.n_tf; t += 4) {
+      int* z = s_nz + t * (n + 1);
+      tf_prefix_warp(all + t * n, n, z, tid & 31);
+      const float m = tf_threshold_warp(B.A, z, tid & 31);
+      if ((tid & 31) == 0) below[t] = m;
+    }
+    __syncthreads();
+  }
+  __device__ __forceinline__ const float4* tf(const TileAt& p) const { return all + p.tf * n; }
+  __device__ __forceinline__ const int* nz(const TileAt& p) const { return s_nz + p.tf * (n + 1); }
+  __device__ __forceinline__ float clear_below(const TileAt& p) const { return s_clear[p.tf]; }
+};
+
+// Schedule 3 in one kernel: persistent warps taking 8x4-pixel tiles from the global queue (as
+// march_kernel does for the per-ray loop), each marching its tile with deferred shading.  With
+// a workspace (A.ts) it takes the tiles that the split march left: those it gave up for lack of
+// room and did not take up again, the dense ones, and the ones it did not start.
+template <int ST, int SHADE, typename Args = RenderArgs>
 __global__ void __launch_bounds__(128, AMR_MIN_BLOCKS_DEFERRED)
-    deferred_kernel(const __grid_constant__ RenderArgs A) {
-  // every tile of the image, or (with a workspace) those the split march left: the tiles it
-  // gave up for lack of room and did not take up again, the dense ones, and the ones it did not
-  // start
-  const int all_tiles = ((A.ray.width + 7) / 8) * ((A.ray.rows + 3) / 4);
+    deferred_kernel(const __grid_constant__ Args P) {
+  const RenderArgs& A = render_args(P);
+  const int all_tiles = count_tiles(P);
   const bool rest = A.ts.heads != nullptr;
   int left = 0, dense = 0, retried = 0, begun = all_tiles;
   if (rest) {
@@ -333,18 +435,11 @@ __global__ void __launch_bounds__(128, AMR_MIN_BLOCKS_DEFERRED)
     if (left == 0 && dense == 0 && begun == all_tiles) return;
   }
   extern __shared__ float4 smem[];
-  float4* s_tf = smem;
-  int* s_nz = reinterpret_cast<int*>(smem + A.tf_n);
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-  const size_t tf_bytes = (size_t)A.tf_n * sizeof(float4) + (size_t)(A.tf_n + 1) * sizeof(int);
   DeferArea& Q = reinterpret_cast<DeferArea*>(reinterpret_cast<char*>(smem) +
-                                              ((tf_bytes + 15) & ~(size_t)15))[tid >> 5];
-  __shared__ float s_clear;
-  stage_tf(A, s_tf, s_nz, &s_clear, tid, blockDim.x * blockDim.y);
-  const float clear_below = s_clear;
+                                              StagedTf<Args>::bytes(P))[tid >> 5];
+  const StagedTf<Args> staged(P, smem, tid);
   const int lane = tid & 31;
-  const RayArgs& R = A.ray;
-  const int tiles_x = (R.width + 7) / 8;
   const int n_tiles = rest ? left + dense + all_tiles - begun : all_tiles;
   unsigned nsamp = 0;
   unsigned long long status = 0;
@@ -362,13 +457,15 @@ __global__ void __launch_bounds__(128, AMR_MIN_BLOCKS_DEFERRED)
       else if (t < left + dense) t = __ldcg(A.ts.dense + t - left);
       else t += begun - left - dense;
     }
-    const int i = (t % tiles_x) * 8 + (lane & 7);
-    const int jr = (t / tiles_x) * 4 + (lane >> 3);
+    const TileAt p = tile_at(P, t);
+    const RayArgs& R = tile_rays(P, p);
+    int i, jr;
+    p.pixel(lane, i, jr);
     const int j = R.row0 + jr;
-    const bool active = i < R.width && jr < R.rows && j < R.height;
-    const float4 c = march_deferred<ST, SHADE>(A, R, i, j, active, s_tf, s_nz, clear_below, Q,
-                                              nsamp, status);
-    if (active) A.out[(size_t)jr * R.width + i] = c;
+    const bool active = i < p.width && jr < p.rows && j < R.height;
+    const float4 c = march_deferred<ST, SHADE>(A, R, i, j, active, staged.tf(p), staged.nz(p),
+                                              staged.clear_below(p), Q, nsamp, status);
+    if (active) p.out[p.at(i, jr)] = c;
   }
   const unsigned total = __reduce_add_sync(0xffffffffu, nsamp);
   if (lane == 0 && total) atomicAdd(A.counters, (unsigned long long)total);

@@ -72,31 +72,17 @@ cudaError_t launch_persist(K kernel, size_t smem, cudaStream_t s, const RenderAr
   return cudaGetLastError();
 }
 
-// Persistent launch of the tile-queue kernels (march_kernel, deferred_kernel): the queue
-// head is zeroed (every launch owns its queue, also when a caller renders a frame in
-// several bands on one set of counters), then as many 128-thread blocks as are resident at
-// once start, at most one warp per 8x4 tile.
-template <typename K>
-cudaError_t launch_tiles(K kernel, size_t smem, cudaStream_t s, const RenderArgs& a) {
-  cudaError_t e = cudaMemsetAsync(a.counters + kQueueCounter, 0, sizeof(unsigned long long), s);
-  if (e == cudaSuccess && smem > 48 * 1024)
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int dev = 0, sms = 0, occ = 0;
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = fit_carveout(kernel, smem, 128, occ);
-  if (e != cudaSuccess) return e;
-  const long long tiles = (long long)((a.ray.width + 7) / 8) * ((a.ray.rows + 3) / 4);
-  const long long grid = std::max(1LL, std::min((long long)sms * std::max(occ, 1), (tiles + 3) / 4));
-  kernel<<<(unsigned)grid, dim3(8, 16), smem, s>>>(a);
-  return cudaGetLastError();
+inline long long tiles_of(const RenderArgs& a) {
+  return (long long)((a.ray.width + 7) / 8) * ((a.ray.rows + 3) / 4);
 }
+inline long long tiles_of(const BatchArgs& b) { return b.n_items; }
+inline const RenderArgs& args_of(const RenderArgs& a) { return a; }
+inline const RenderArgs& args_of(const BatchArgs& b) { return b.A; }
 
-// Persistent launch of the split march's kernels: as many blocks as are resident at once, at
-// most `per_tile` of them per tile.
-template <typename K>
-cudaError_t launch_stride(K kernel, size_t smem, cudaStream_t s, const RenderArgs& a,
-                          int per_tile = 4) {
+// Persistent launch: as many 128-thread blocks as are resident at once, at most `per_tile`
+// of them per tile, and at least a warp per tile while they last.
+template <typename K, typename Args>
+cudaError_t launch_stride(K kernel, size_t smem, cudaStream_t s, const Args& a, int per_tile) {
   cudaError_t e = cudaSuccess;
   if (smem > 48 * 1024)
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -105,47 +91,64 @@ cudaError_t launch_stride(K kernel, size_t smem, cudaStream_t s, const RenderArg
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = fit_carveout(kernel, smem, 128, occ);
   if (e != cudaSuccess) return e;
-  const long long tiles = (long long)((a.ray.width + 7) / 8) * ((a.ray.rows + 3) / 4);
-  const long long grid = std::max(1LL, std::min((long long)sms * std::max(occ, 1), tiles * per_tile));
+  const long long want = per_tile > 0 ? tiles_of(a) * per_tile : (tiles_of(a) + 3) / 4;
+  const long long grid = std::max(1LL, std::min((long long)sms * std::max(occ, 1), want));
   kernel<<<(unsigned)grid, dim3(8, 16), smem, s>>>(a);
   return cudaGetLastError();
 }
 
-// The split march, in rounds that each fill the workspace at most once, then the tiles that
-// were left.
-template <int ST, int SHADE>
-cudaError_t launch_split(const TaskPlan& plan, size_t tf_bytes, cudaStream_t s, const RenderArgs& a) {
-  const size_t base = (tf_bytes + 15) & ~(size_t)15;
-  cudaError_t e = cudaSuccess;
-  for (int row = 0; e == cudaSuccess && row < a.ray.rows; row += plan.rows) {
-    RenderArgs b = a;
-    b.ts = plan.ts;
-    b.ray.row0 = a.ray.row0 + row;
-    b.ray.rows = std::min(plan.rows, a.ray.rows - row);
-    b.out = a.out + (size_t)row * a.ray.width;
-    const size_t tiles = (size_t)((b.ray.width + 7) / 8) * (size_t)((b.ray.rows + 3) / 4);
-    e = cudaMemsetAsync(b.ts.heads, 0, kHeads * sizeof(unsigned), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b.ts.tile, 0xff, tiles * sizeof(int2), s);
-    for (int r = 0; e == cudaSuccess && r < plan.rounds; ++r) {
-      if (r > 0) e = cudaMemsetAsync(b.ts.heads, 0, kRoundHeads * sizeof(unsigned), s);
-      if (e == cudaSuccess)
-        e = launch_stride(split_march_kernel<ST, SHADE>, base + 4 * sizeof(CandArea<true>), s, b, 1);
-      if (e == cudaSuccess) e = launch_stride(split_shade_kernel<ST, SHADE>, base, s, b);
-      if (e == cudaSuccess) e = launch_stride(split_outer_kernel<ST, SHADE>, base, s, b);
-      if (e == cudaSuccess) e = launch_stride(split_sum_kernel, 0, s, b);
-    }
+// The same for the tile-queue kernels (march_kernel, deferred_kernel), whose queue head is
+// zeroed first (every launch owns its queue, also when a caller renders a frame in several
+// bands on one set of counters); at most one warp per tile.
+template <typename K, typename Args>
+cudaError_t launch_tiles(K kernel, size_t smem, cudaStream_t s, const Args& a) {
+  cudaError_t e = cudaMemsetAsync(args_of(a).counters + kQueueCounter, 0, sizeof(unsigned long long), s);
+  return e == cudaSuccess ? launch_stride(kernel, smem, s, a, 0) : e;
+}
+
+// One band of the split march (b carries its workspace), in rounds that each fill the
+// workspace at most once, then the tiles that were left.
+template <int ST, int SHADE, typename Args>
+cudaError_t launch_rounds(int rounds, cudaStream_t s, const Args& b) {
+  const TaskSpace& ts = args_of(b).ts;
+  const size_t base = StagedTf<Args>::bytes(b);
+  cudaError_t e = cudaMemsetAsync(ts.heads, 0, kHeads * sizeof(unsigned), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(ts.tile, 0xff, (size_t)tiles_of(b) * sizeof(int2), s);
+  for (int r = 0; e == cudaSuccess && r < rounds; ++r) {
+    if (r > 0) e = cudaMemsetAsync(ts.heads, 0, kRoundHeads * sizeof(unsigned), s);
     if (e == cudaSuccess)
-      e = launch_tiles(deferred_kernel<ST, SHADE>, base + 4 * sizeof(DeferArea), s, b);
+      e = launch_stride(split_march_kernel<ST, SHADE, Args>, base + 4 * sizeof(CandArea<true>), s, b, 1);
+    if (e == cudaSuccess) e = launch_stride(split_shade_kernel<ST, SHADE, Args>, base, s, b, 4);
+    if (e == cudaSuccess) e = launch_stride(split_outer_kernel<ST, SHADE, Args>, base, s, b, 4);
+    if (e == cudaSuccess) e = launch_stride(split_sum_kernel<Args>, 0, s, b, 4);
   }
+  if (e == cudaSuccess)
+    e = launch_tiles(deferred_kernel<ST, SHADE, Args>, base + 4 * sizeof(DeferArea), s, b);
   return e;
 }
 
+// Deferred shading of one image: the split march in bands of rows that the workspace has tile
+// records for, or without a workspace the one-kernel march.
 template <int ST, int SHADE>
-cudaError_t launch_shaded(const TaskPlan& plan, size_t tf_bytes, cudaStream_t s, const RenderArgs& a) {
-  if constexpr (ST != ST_TEXOBJ && ST != ST_ATLAS_TEX3D)
-    if (plan.rows > 0) return launch_split<ST, SHADE>(plan, tf_bytes, s, a);
-  return launch_tiles(deferred_kernel<ST, SHADE>,
-                      ((tf_bytes + 15) & ~(size_t)15) + 4 * sizeof(DeferArea), s, a);
+cudaError_t launch_shaded(const TaskPlan& plan, cudaStream_t s, const RenderArgs& a) {
+  if constexpr (ST != ST_TEXOBJ && ST != ST_ATLAS_TEX3D) {
+    const long long tiles_x = (a.ray.width + 7) / 8;
+    const int band = 4 * (int)std::min(plan.tiles / tiles_x, 1LL << 20);  // rows
+    if (band > 0) {
+      cudaError_t e = cudaSuccess;
+      for (int row = 0; e == cudaSuccess && row < a.ray.rows; row += band) {
+        RenderArgs b = a;
+        b.ts = plan.ts;
+        b.ray.row0 = a.ray.row0 + row;
+        b.ray.rows = std::min(band, a.ray.rows - row);
+        b.out = a.out + (size_t)row * a.ray.width;
+        e = launch_rounds<ST, SHADE>(plan.rounds(tiles_of(b)), s, b);
+      }
+      return e;
+    }
+  }
+  return launch_tiles(deferred_kernel<ST, SHADE>, StagedTf<RenderArgs>::bytes(a) + 4 * sizeof(DeferArea),
+                      s, a);
 }
 
 template <int ST>
@@ -164,7 +167,7 @@ amr_status launch_storage(amr_ctx* c, const RenderArgs& a, int interp, int shade
   // (not for texture storages, where it measured slower at 1900 x 1800: 37.1 against 31.8 ms;
   // nor for a caller that brings its own counters and may not allocate)
   constexpr bool kLinear = ST != ST_TEXOBJ && ST != ST_ATLAS_TEX3D;
-  if (kLinear && schedule == 3 && a.counters == c->dev.counters) plan = plan_tasks(c, a, s);
+  if (kLinear && schedule == 3 && a.counters == c->dev.counters) plan = plan_tasks(c, tiles_of(a), s);
   cudaError_t e;
   if (shade & kShadeShadow) {
     // secondary rays to the point light: per-ray schedule (a lane marches its samples'
@@ -176,8 +179,8 @@ amr_status launch_storage(amr_ctx* c, const RenderArgs& a, int interp, int shade
         return fail(c, AMR_ERR_ARG,
                     "secondary rays render trilinear with schedule 0, or 3 with shade = 1");
       if (schedule == 3) {
-        if (base == 1) e = launch_shaded<ST, 1 | kShadeShadow>(plan, tf_bytes, s, a);
-        else e = launch_shaded<ST, 2 | kShadeShadow>(plan, tf_bytes, s, a);
+        if (base == 1) e = launch_shaded<ST, 1 | kShadeShadow>(plan, s, a);
+        else e = launch_shaded<ST, 2 | kShadeShadow>(plan, s, a);
       } else {
         const size_t smem = tf_bytes;
         if (base == 0) e = launch_tiles(march_kernel<ST, 1, kShadeShadow>, smem, s, a);
@@ -193,13 +196,13 @@ amr_status launch_storage(amr_ctx* c, const RenderArgs& a, int interp, int shade
       return fail(c, AMR_ERR_ARG, "deferred shading renders trilinear with shade = 1");
     if constexpr (kPtr) {
       if (mx) {
-        if (shade == 1) e = launch_shaded<ST, 1 | kShadeMaxBit>(plan, tf_bytes, s, a);
-        else e = launch_shaded<ST, 2 | kShadeMaxBit>(plan, tf_bytes, s, a);
+        if (shade == 1) e = launch_shaded<ST, 1 | kShadeMaxBit>(plan, s, a);
+        else e = launch_shaded<ST, 2 | kShadeMaxBit>(plan, s, a);
         goto launched;
       }
     }
-    if (shade == 1) e = launch_shaded<ST, 1>(plan, tf_bytes, s, a);
-    else e = launch_shaded<ST, 2>(plan, tf_bytes, s, a);
+    if (shade == 1) e = launch_shaded<ST, 1>(plan, s, a);
+    else e = launch_shaded<ST, 2>(plan, s, a);
   } else if (schedule == 2) {
     // persistent warps with ray refill (trilinear)
     if (interp != 1) return fail(c, AMR_ERR_ARG, "the refill schedule renders trilinear");

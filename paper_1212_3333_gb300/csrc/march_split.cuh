@@ -34,7 +34,7 @@
 // later round.  Dense tiles, and what the last round leaves, go to deferred_kernel, which needs
 // no workspace.
 #pragma once
-#include "march.cuh"
+#include "march_deferred.cuh"
 
 namespace amr {
 
@@ -102,7 +102,7 @@ template <int ST, int SHADE>
 __device__ __forceinline__ int march_tile(const RenderArgs& A, const RayArgs& R, int i, int j,
                                            bool active, const float4* s_tf, const int* s_nz,
                                            float clear_below, CandArea<(SHADE & 3) != 0>& Q,
-                                           RayF& rf, SegBlock& blk, int tile_id, float4& px,
+                                           RayF& rf, SegBlock& blk, int tile_id, int view, float4& px,
                                            int2& tile, unsigned& nsamp, unsigned long long& status) {
   constexpr bool MX = (SHADE & kShadeMaxBit) != 0;  // the stencil-maximum test
   constexpr bool SHADED = (SHADE & 3) != 0;
@@ -224,7 +224,7 @@ __device__ __forceinline__ int march_tile(const RenderArgs& A, const RayArgs& R,
                                    ? atomicAdd(A.ts.heads + kHeadChunk, 1u) : ~0u;
             fresh = c < (unsigned)A.ts.chunks ? (int)c : -1;
             if (fresh >= 0) {
-              A.ts.meta[fresh] = make_int4(tile_id, 0, -1, 0);
+              A.ts.meta[fresh] = make_int4(tile_id, 0, -1, view);
               if (tasks != 0) {  // the chunk is full
                 A.ts.meta[chunk].y = kTaskChunk;
                 A.ts.meta[chunk].z = fresh;
@@ -417,13 +417,12 @@ __device__ __forceinline__ int march_tile(const RenderArgs& A, const RayArgs& R,
 #endif
 
 // Persistent warps taking 8x4-pixel tiles from a queue, as march_kernel does.
-template <int ST, int SHADE>
+template <int ST, int SHADE, typename Args = RenderArgs>
 __global__ void __launch_bounds__(128, AMR_SPLIT_MARCH_BLOCKS)
-    split_march_kernel(const __grid_constant__ RenderArgs A) {
+    split_march_kernel(const __grid_constant__ Args P) {
   constexpr bool SHADED = (SHADE & 3) != 0;
-  const RayArgs& R = A.ray;
-  const int tiles_x = (R.width + 7) / 8;
-  const int n_tiles = tiles_x * ((R.rows + 3) / 4);
+  const RenderArgs& A = render_args(P);
+  const int n_tiles = count_tiles(P);
   unsigned ready = 0;  // tiles that earlier rounds gave up
   if constexpr (SHADED) {
     ready = __ldcg(A.ts.heads + kHeadReady);
@@ -433,19 +432,11 @@ __global__ void __launch_bounds__(128, AMR_SPLIT_MARCH_BLOCKS)
     if (ready != 0 && (blockIdx.x & 1)) return;  // there was no room: half as many tiles at once
   }
   extern __shared__ float4 smem[];
-  float4* s_tf = smem;
-  int* s_nz = reinterpret_cast<int*>(smem + A.tf_n);
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-  const size_t tf_bytes = (size_t)A.tf_n * sizeof(float4) + (size_t)(A.tf_n + 1) * sizeof(int);
   using Area = CandArea<SHADED>;
   Area& Q = reinterpret_cast<Area*>(reinterpret_cast<char*>(smem) +
-                                    ((tf_bytes + 15) & ~(size_t)15))[tid >> 5];
-  __shared__ float s_clear;
-  stage_tf(A, s_tf, s_nz, &s_clear, tid, blockDim.x * blockDim.y);
-  const float clear_below = s_clear;
-  // nearly everything opaque: one kernel is faster (640 x 479, 480 opaque samples a pixel: 16.1
-  // ms alone, 24.7 after a workspace full of tasks), so the tiles are left to it
-  if (SHADED && clear_below <= A.dense_below) return;
+                                    StagedTf<Args>::bytes(P))[tid >> 5];
+  const StagedTf<Args> staged(P, smem, tid);
   const int lane = tid & 31;
   unsigned nsamp = 0;
   unsigned long long status = 0;
@@ -476,17 +467,24 @@ __global__ void __launch_bounds__(128, AMR_SPLIT_MARCH_BLOCKS)
     }
     t = __shfl_sync(0xffffffffu, t, 0);
     if (t >= n_tiles) break;
-    const int i = (t % tiles_x) * 8 + (lane & 7);
-    const int jr = (t / tiles_x) * 4 + (lane >> 3);
+    const TileAt p = tile_at(P, t);
+    const RayArgs& R = tile_rays(P, p);
+    int i, jr;
+    p.pixel(lane, i, jr);
     const int j = R.row0 + jr;
-    const bool active = i < R.width && jr < R.rows && j < R.height;
+    const bool active = i < p.width && jr < p.rows && j < R.height;
     float4 px;
     int2 tile;
-    const int how = march_tile<ST, SHADE>(A, R, i, j, active, s_tf, s_nz, clear_below, Q,
-                                            rf, blk, t, px, tile, nsamp, status);
+    // nearly everything opaque: one kernel is faster (640 x 479, 480 opaque samples a pixel:
+    // 16.1 ms alone, 24.7 after a workspace full of tasks), so the tile is left to it
+    int how = kTileDense;
+    if (!SHADED || staged.clear_below(p) > A.dense_below)
+      how = march_tile<ST, SHADE>(A, R, i, j, active, staged.tf(p), staged.nz(p),
+                                  staged.clear_below(p), Q, rf, blk, t, p.view, px, tile, nsamp,
+                                  status);
     if (how == kTileDone) {
       if (SHADED && tile.y == 0) px = make_float4(0.f, 0.f, 0.f, px.w);  // nothing to shade
-      if (active) A.out[(size_t)jr * R.width + i] = px;
+      if (active) p.out[p.at(i, jr)] = px;
       if (SHADED && lane == 0 && tile.y != 0) A.ts.tile[t] = tile;
     } else if (lane == 0) {
       if (how == kTileDense) A.ts.dense[atomicAdd(A.ts.heads + kHeadDense, 1u)] = t;
@@ -538,39 +536,24 @@ __device__ __forceinline__ float3 task_colour(const RenderArgs& A, const float4*
   return make_float3(cr, cg, cb);
 }
 
-// Stage the transfer function (and, for light rays, its prefix counts).
-template <int SHADE>
-__device__ __forceinline__ const float4* stage_shade(const RenderArgs& A, float4* smem, int tid) {
-  for (int k = tid; k < A.tf_n; k += 128) smem[k] = A.tf[k];
-  if constexpr ((SHADE & kShadeShadow) != 0) {
-    if (tid < 32) tf_prefix_warp(A.tf, A.tf_n, reinterpret_cast<int*>(smem + A.tf_n), tid);
-  }
-  __syncthreads();
-  return smem;
-}
-
-// Pixel of a task (the lane it belongs to, in its chunk's tile).
-__device__ __forceinline__ void task_pixel(const RayArgs& R, int tile, int kl, int& i, int& jr) {
-  const int tiles_x = (R.width + 7) / 8, owner = kl >> kTaskSampleBits;
-  i = (tile % tiles_x) * 8 + (owner & 7);
-  jr = (tile / tiles_x) * 4 + (owner >> 3);
-}
-
 // Shade every task whose gradient stays in its leaf, one per lane, and list the others.
-template <int ST, int SHADE>
+template <int ST, int SHADE, typename Args = RenderArgs>
 __global__ void __launch_bounds__(128, AMR_SPLIT_SHADE_BLOCKS)
-    split_shade_kernel(const __grid_constant__ RenderArgs A) {
+    split_shade_kernel(const __grid_constant__ Args P) {
   extern __shared__ float4 smem[];
+  const RenderArgs& A = render_args(P);
   const unsigned FULL = 0xffffffffu;
   const int tid = threadIdx.x + blockDim.x * threadIdx.y, lane = tid & 31;
-  const RayArgs& R = A.ray;
   const int units = (int)min(__ldcg(A.ts.heads + kHeadChunk), (unsigned)A.ts.chunks) * (kTaskChunk / 32);
   if ((int)blockIdx.x * 4 >= units) return;
-  const float4* s_tf = stage_shade<SHADE>(A, smem, tid);
+  const StagedTf<Args> staged(P, smem, tid);
   for (int u = blockIdx.x * 4 + (tid >> 5); u < units; u += gridDim.x * 4) {
     const int4 meta = __ldcg(A.ts.meta + u / (kTaskChunk / 32));
     const int count = min(32, meta.y - (u % (kTaskChunk / 32)) * 32);
     if (count <= 0) continue;
+    const TileAt p = chunk_tile(P, meta);
+    const RayArgs& R = tile_rays(P, p);
+    const float4* tf = staged.tf(p);
     const int slot = u * 32 + lane;
     bool inner = true;
     float4 t;
@@ -581,8 +564,8 @@ __global__ void __launch_bounds__(128, AMR_SPLIT_SHADE_BLOCKS)
       t = __ldcg(A.ts.tasks + slot);
       const int kl = __float_as_int(t.y);
       int i, jr;
-      task_pixel(R, meta.x, kl, i, jr);
-      L = __ldcg(A.out + (size_t)jr * R.width + i);
+      p.pixel(kl >> kTaskSampleBits, i, jr);
+      L = __ldcg(p.out + p.at(i, jr));
       float beta[3];
       const SegState s = task_segment(A, __float_as_int(t.x), kl & ((1 << kTaskSampleBits) - 1),
                                       i, R.row0 + jr, beta);
@@ -599,7 +582,7 @@ __global__ void __launch_bounds__(128, AMR_SPLIT_SHADE_BLOCKS)
     if constexpr ((SHADE & kShadeShadow) != 0) {
       // the samples' light rays, one after the other, each by the whole warp
       for (int e = 0; e < count; ++e) {
-        const float Te = warp_shadow_transmittance<ST>(A, R, s_tf, __shfl_sync(FULL, x[0], e),
+        const float Te = warp_shadow_transmittance<ST>(A, R, tf, __shfl_sync(FULL, x[0], e),
                                                        __shfl_sync(FULL, x[1], e),
                                                        __shfl_sync(FULL, x[2], e));
         if (lane == e) T = Te;
@@ -607,7 +590,7 @@ __global__ void __launch_bounds__(128, AMR_SPLIT_SHADE_BLOCKS)
     }
     if (lane < count) {
       float3 c = make_float3(T, 0.f, 0.f);  // an outer task's transmittance waits here
-      if (inner) c = task_colour<SHADE>(A, s_tf, t.z, A.lv[level], gr, L, T);
+      if (inner) c = task_colour<SHADE>(A, tf, t.z, A.lv[level], gr, L, T);
       A.ts.col[slot] = make_float4(c.x, c.y, c.z, t.w);
     }
     const unsigned outer = __ballot_sync(FULL, !inner);
@@ -621,16 +604,16 @@ __global__ void __launch_bounds__(128, AMR_SPLIT_SHADE_BLOCKS)
 }
 
 // Shade the listed tasks: six lanes take one's six neighbours, five tasks per warp.
-template <int ST, int SHADE>
+template <int ST, int SHADE, typename Args = RenderArgs>
 __global__ void __launch_bounds__(128, AMR_SPLIT_OUTER_BLOCKS)
-    split_outer_kernel(const __grid_constant__ RenderArgs A) {
+    split_outer_kernel(const __grid_constant__ Args P) {
   extern __shared__ float4 smem[];
+  const RenderArgs& A = render_args(P);
   const unsigned FULL = 0xffffffffu;
   const int tid = threadIdx.x + blockDim.x * threadIdx.y, lane = tid & 31;
-  const RayArgs& R = A.ray;
   const int n = (int)__ldcg(A.ts.heads + kHeadOuter);
   if ((int)blockIdx.x * 20 >= n) return;
-  const float4* s_tf = stage_shade<SHADE>(A, smem, tid);
+  const StagedTf<Args> staged(P, smem, tid);
   const int e = lane / 6, q = lane % 6, ax = q >> 1;
   const float sg = (q & 1) ? -1.0f : 1.0f;
   for (int b = (blockIdx.x * 4 + (tid >> 5)) * 5; b < n; b += gridDim.x * 20) {
@@ -638,11 +621,14 @@ __global__ void __launch_bounds__(128, AMR_SPLIT_OUTER_BLOCKS)
     int slot = 0, level = 0, i = 0, jr = 0;
     float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
     float v = 0.f;
+    TileAt p = {};
     if (on) {
       slot = __ldcg(A.ts.outer + b + e);
       t = __ldcg(A.ts.tasks + slot);
       const int kl = __float_as_int(t.y), k = kl & ((1 << kTaskSampleBits) - 1);
-      task_pixel(R, __ldcg(&A.ts.meta[slot / kTaskChunk].x), kl, i, jr);
+      p = chunk_tile(P, __ldcg(A.ts.meta + slot / kTaskChunk));
+      const RayArgs& R = tile_rays(P, p);
+      p.pixel(kl >> kTaskSampleBits, i, jr);
       float bn[3];
       const SegState s = task_segment(A, __float_as_int(t.x), k, i, R.row0 + jr, bn);
       level = s.level;
@@ -658,9 +644,9 @@ __global__ void __launch_bounds__(128, AMR_SPLIT_OUTER_BLOCKS)
       const DLevel& lv = A.lv[level];
       const float gr[3] = {(w[0] - w[1]) * lv.ginv[0], (w[2] - w[3]) * lv.ginv[1],
                            (w[4] - w[5]) * lv.ginv[2]};
-      const float4 L = __ldcg(A.out + (size_t)jr * R.width + i);
+      const float4 L = __ldcg(p.out + p.at(i, jr));
       const float T = (SHADE & kShadeShadow) != 0 ? __ldcg(&A.ts.col[slot].x) : 1.0f;
-      const float3 c = task_colour<SHADE>(A, s_tf, t.z, lv, gr, L, T);
+      const float3 c = task_colour<SHADE>(A, staged.tf(p), t.z, lv, gr, L, T);
       A.ts.col[slot] = make_float4(c.x, c.y, c.z, t.w);
     }
   }
@@ -671,17 +657,17 @@ struct SumArea {
   float4 col[32];
   unsigned own[32];
 };
-static __global__ void __launch_bounds__(128) split_sum_kernel(const __grid_constant__ RenderArgs A) {
+template <typename Args>
+__global__ void __launch_bounds__(128) split_sum_kernel(const __grid_constant__ Args P) {
   __shared__ SumArea area[4];
+  const RenderArgs& A = render_args(P);
   if (blockIdx.x == 0 && threadIdx.x + threadIdx.y == 0)
     A.ts.heads[kHeadReady] = __ldcg(A.ts.heads + kHeadLeft);
   if (__ldcg(A.ts.heads + kHeadChunk) == 0) return;  // an empty round
   const int tid = threadIdx.x + blockDim.x * threadIdx.y, lane = tid & 31;
   const unsigned lt_mask = (1u << lane) - 1u;
   SumArea& Q = area[tid >> 5];
-  const RayArgs& R = A.ray;
-  const int tiles_x = (R.width + 7) / 8;
-  const int n_tiles = tiles_x * ((R.rows + 3) / 4);
+  const int n_tiles = count_tiles(P);
   for (int t = blockIdx.x * 4 + (tid >> 5); t < n_tiles; t += gridDim.x * 4) {
     const int2 tile = __ldcg(A.ts.tile + t);
     if (tile.y < 0) continue;  // none, or of another round
@@ -704,14 +690,38 @@ static __global__ void __launch_bounds__(128) split_sum_kernel(const __grid_cons
       }
       __syncwarp();
     }
-    const int i = (t % tiles_x) * 8 + (lane & 7);
-    const int jr = (t / tiles_x) * 4 + (lane >> 3);
-    if (i < R.width && jr < R.rows && R.row0 + jr < R.height) {
-      float4* o = A.out + (size_t)jr * R.width + i;
+    const TileAt p = tile_at(P, t);
+    int i, jr;
+    p.pixel(lane, i, jr);
+    if (i < p.width && jr < p.rows && tile_rays(P, p).row0 + jr < tile_rays(P, p).height) {
+      float4* o = p.out + p.at(i, jr);
       *o = make_float4(C0, C1, C2, __ldcg(&o->w));
     }
     if (lane == 0) A.ts.tile[t].y = -1;
   }
+}
+
+// The rays of a batch's views.
+static __global__ void __launch_bounds__(kMaxBatchViews) batch_views_kernel(const __grid_constant__ BatchArgs B) {
+  const int v = threadIdx.x;
+  if (v >= B.n_views) return;
+  RayArgs r = B.A.ray;
+  const BatchView& b = B.v[v];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    r.eye[a] = b.eye[a];
+    r.fwd[a] = b.fwd[a];
+    r.right[a] = b.right[a];
+    r.up[a] = b.up[a];
+  }
+  r.tan_half_fov_y = b.tan_half_fov_y;
+  r.width = b.width;
+  r.height = b.height;
+  r.row0 = 0;
+  r.rows = b.height;
+  r.lod_scale = b.lod_scale;
+  r.lod_scale_f = b.lod_scale_f;
+  B.A.ts.views[v] = r;
 }
 
 }  // namespace amr
