@@ -28,6 +28,8 @@ constexpr uint32_t kIndexMask = 0x3fffffffu;
 constexpr int kMaxDepth = 256;          // descent bound (tree depth is checked at build)
 constexpr int kMaxSamplesPerSegment = 1 << 22;
 constexpr uint32_t kFaceLeaf = 0x80000000u;  // face-table entry names a leaf (id in bits 0..30)
+constexpr uint32_t kFaceList = 0x40000000u;  // or a list of leaves (its 16-byte word, bits 0..29)
+constexpr int kFaceListMax = 14;             // leaves in a list
 
 // device counters: [0] samples, [1] status bits, [2] exact descent decisions,
 // [3] exact sample counts, [4] exact neighbour / nearest positions
@@ -120,6 +122,11 @@ struct RayArgs {
   const uint32_t* macro;
   int32_t macro_cell;
   int32_t macro_dims[3];
+  // leaf lists of the face table.  First word: the lower corner of the leaves' rectangles
+  // (finest cells on the face's two axes, in axis order), the node slot they replace, and
+  // their number + 32 log2 of the unit of the rectangles.  Then two leaves a word: u0, u1, v0,
+  // v1 (a byte each, units from the corner) and the leaf id
+  const int4* face_list;
 };
 
 // Workspace of the split march (march_split.cuh): the opaque samples of a launch's tiles as
@@ -156,7 +163,8 @@ struct RenderArgs {
   const int32_t* face_node;    // per leaf, 12: per face (2a + side) the node slot holding the
                                // leaf and the cell beyond the face, then the cell alone
                                // (starts of neighbour lookups; the second half: ropes);
-                               // an entry with kFaceLeaf set names a leaf id instead
+                               // an entry with kFaceLeaf set names a leaf id instead, one
+                               // with kFaceList (second half) a list of the leaves beyond
   const int4* node_box;        // per node slot, 2: box lo (x, y, z, highest label level of
                                // a type-(a) node above it or -1), hi (x, y, z, 0), finest
                                // cells (rope restarts)

@@ -68,6 +68,7 @@ void fill_ray(const amr_ctx* c, const amr_camera* cam, int row0, int rows, RayAr
   ra->lod = c->dev.lod;
   ra->macro = c->dev.macro;
   ra->macro_cell = c->dev.macro_cell;
+  ra->face_list = c->dev.face_list;
   for (int a = 0; a < 3; ++a) ra->macro_dims[a] = c->dev.macro_dims[a];
   ra->levels = c->tree.lod_levels;  // levels a pruned node can have
   ra->lod_scale = 0.0;

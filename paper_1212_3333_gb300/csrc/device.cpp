@@ -359,6 +359,7 @@ void release_device(amr_ctx* c) {
   cudaFree(d.nodes);
   cudaFree(d.lod);
   cudaFree(d.face_node);
+  cudaFree(d.face_list);
   cudaFree(d.node_box);
   cudaFree(d.macro);
   cudaFree(d.leaves);
@@ -373,6 +374,58 @@ void release_device(amr_ctx* c) {
   for (void* p : d.task_spaces) cudaFree(p);
   d = DeviceState();
   c->device_built = false;
+}
+
+// The leaves beyond face f (2 axis + side) of leaf m, all in the subtree of pre-order node
+// `pre`, as a list at the end of `lists` (RayArgs::face_list): its word, or 0 when there are too
+// many, their rectangles do not fit the bytes, or the face is one of the root's.
+static uint32_t face_list(const Tree& t, const int64_t* root, size_t m, int f, int32_t pre,
+                          int32_t slot, std::vector<int4>& lists) {
+  const int32_t* box = &t.leaf_box[6 * m];
+  const int a = f >> 1, b = a == 0 ? 1 : 0, c = a == 2 ? 1 : 2;
+  const int64_t plane = (f & 1) ? box[3 + a] : box[a];
+  if (plane == ((f & 1) ? root[3 + a] : root[a])) return 0;
+  const int64_t cell = (f & 1) ? plane : plane - 1;  // the finest cells beyond the face
+  struct Rect { int32_t u0, u1, v0, v1, id; };
+  std::vector<Rect> r;
+  std::vector<int32_t> stack(1, pre);
+  while (!stack.empty()) {
+    const int32_t i = stack.back();
+    stack.pop_back();
+    const int ax = t.axis[i];
+    if (ax < 0) {
+      const int32_t id = t.leaf[i];
+      const int32_t* q = &t.leaf_box[6 * (size_t)id];
+      if (r.size() == (size_t)kFaceListMax) return 0;
+      r.push_back({std::max(q[b], box[b]) - box[b], std::min(q[3 + b], box[3 + b]) - box[b],
+                   std::max(q[c], box[c]) - box[c], std::min(q[3 + c], box[3 + c]) - box[c], id});
+      continue;
+    }
+    const int64_t sp = t.split[i], lo = ax == a ? cell : box[ax], hi = ax == a ? cell + 1 : box[3 + ax];
+    if (lo < sp) stack.push_back(t.left[i]);
+    if (hi > sp) stack.push_back(t.right[i]);
+  }
+  int32_t bits = 0;  // the rectangles' unit: the largest power of two in all their corners
+  for (const Rect& q : r) bits |= q.u0 | q.u1 | q.v0 | q.v1;
+  if (bits == 0) return 0;
+  const int shift = __builtin_ctz((unsigned)bits);
+  for (const Rect& q : r)
+    if ((q.u1 >> shift) > 255 || (q.v1 >> shift) > 255) return 0;
+  const size_t word = lists.size();
+  if (word + 1 + kFaceListMax / 2 >= (size_t)kFaceList) return 0;
+  lists.push_back(int4{box[b], box[c], slot, (int)r.size() + 32 * shift});
+  for (size_t k = 0; k < r.size(); k += 2) {
+    int4 w = {0, 0, 0, 0};
+    for (size_t e = 0; e < 2 && k + e < r.size(); ++e) {
+      const Rect& q = r[k + e];
+      const uint32_t p = (uint32_t)(q.u0 >> shift) | (uint32_t)(q.u1 >> shift) << 8 |
+                         (uint32_t)(q.v0 >> shift) << 16 | (uint32_t)(q.v1 >> shift) << 24;
+      (e == 0 ? w.x : w.z) = (int)p;
+      (e == 0 ? w.y : w.w) = q.id;
+    }
+    lists.push_back(w);
+  }
+  return (uint32_t)word;
 }
 
 // The value a fifth of the bricks' cells lie below, from at most about 2^16 of them.
@@ -410,10 +463,16 @@ amr_status upload(amr_ctx* c, void* stream_v) {
       (nodes[0].meta >> 30) != (uint32_t)kLeafAxis)
     nodes[0].meta &= ~kIndexMask;  // the root's children become slots 0 (itself) and 1
   std::vector<int32_t> face_slots(std::max<size_t>(1, t.face_node.size()), 0);
+  std::vector<int4> face_lists(1, int4{0, 0, 0, 0});
   for (size_t k = 0; k < t.face_node.size(); ++k) {
     const int32_t pre = t.face_node[k];
     face_slots[k] = t.axis[pre] < 0 ? (int32_t)(kFaceLeaf | (uint32_t)t.leaf[pre]) : slot_of[pre];
+    if (t.axis[pre] >= 0 && k % 12 >= 6) {
+      const uint32_t list = face_list(t, c->root, k / 12, (int)(k % 12) - 6, pre, slot_of[pre], face_lists);
+      if (list) face_slots[k] = (int32_t)(kFaceList | list);
+    }
   }
+  face_lists.resize(face_lists.size() + kFaceListMax / 2, int4{0, 0, 0, 0});
   const size_t ML = t.lod_patch.size();
   if (M + ML >= ((size_t)1 << 26)) return fail(c, AMR_ERR_CAPACITY, "too many leaves");
   std::vector<DLeaf> leaves(M + ML);
@@ -445,6 +504,7 @@ amr_status upload(amr_ctx* c, void* stream_v) {
   CK(cudaMalloc(&d.nodes, nodes.size() * sizeof(DNode)));
   CK(cudaMalloc(&d.lod, lodv.size() * sizeof(int32_t)));
   CK(cudaMalloc(&d.face_node, face_slots.size() * sizeof(int32_t)));
+  CK(cudaMalloc(&d.face_list, face_lists.size() * sizeof(int4)));
   CK(cudaMalloc(&d.node_box, boxes.size() * sizeof(int4)));
   CK(cudaMalloc(&d.leaves, std::max<size_t>(1, M + ML) * sizeof(DLeaf)));
   CK(cudaMalloc(&d.patches, P * sizeof(DPatch)));
@@ -511,6 +571,8 @@ amr_status upload(amr_ctx* c, void* stream_v) {
                      stream));
   CK(cudaMemcpyAsync(d.lod, lodv.data(), lodv.size() * sizeof(int32_t), cudaMemcpyHostToDevice,
                      stream));
+  CK(cudaMemcpyAsync(d.face_list, face_lists.data(), face_lists.size() * sizeof(int4),
+                     cudaMemcpyHostToDevice, stream));
   CK(cudaMemcpyAsync(d.face_node, face_slots.data(), face_slots.size() * sizeof(int32_t),
                      cudaMemcpyHostToDevice, stream));
   CK(cudaMemcpyAsync(d.node_box, boxes.data(), boxes.size() * sizeof(int4), cudaMemcpyHostToDevice,

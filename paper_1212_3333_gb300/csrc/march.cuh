@@ -361,6 +361,44 @@ __device__ __forceinline__ int descend(const DNode* __restrict__ nodes, const Ra
                       lod_min);
 }
 
+// The leaf of a face list whose rectangle holds the point (u, v) on the face (finest cells on
+// its two axes, relative to (base_u, base_v)), -1 for none; slot: the node the list replaces.
+// The caller checks the leaf's box.  The list's words are loaded together, where a descent
+// from the node (31 % of the segments had one, 3.2 steps on average, the warp's longest
+// deciding) waits for one load a step.  Measured, descents / lists, ms: 640 x 479 2.76 / 2.45,
+// 1024^2 7.43 / 6.99, f16 unshaded 1917 x 1083 4.85 / 4.38, 32-view batch 27.9 / 25.1.
+__device__ __forceinline__ int face_list_leaf(const int4* __restrict__ lists, uint32_t ent, float u,
+                                              float v, int base_u, int base_v, uint32_t& slot) {
+  const int4* w = lists + (ent & (kFaceList - 1u));
+  const int4 h = __ldg(w);
+  int4 q[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) q[k] = __ldg(w + 1 + k);  // (the array is padded)
+  slot = (uint32_t)h.z;
+  const int n = h.w & 31;
+  const float inv = __int_as_float((127 - (h.w >> 5)) << 23);  // 1 / unit
+  const unsigned iu = (unsigned)(int)floorf((u + (float)(base_u - h.x)) * inv);
+  const unsigned iv = (unsigned)(int)floorf((v + (float)(base_v - h.y)) * inv);
+  int leaf = -1;
+  auto test = [&](int rect, int id, int k) {
+    const unsigned r = (unsigned)rect;
+    if (k < n && iu >= (r & 255u) && iu < ((r >> 8) & 255u) && iv >= ((r >> 16) & 255u) &&
+        iv < (r >> 24))
+      leaf = id;
+  };
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    test(q[k].x, q[k].y, 2 * k);
+    test(q[k].z, q[k].w, 2 * k + 1);
+  }
+  for (int k = 6; leaf < 0 && k < n; k += 2) {
+    const int4 e = __ldg(w + 1 + k / 2);
+    test(e.x, e.y, k);
+    test(e.z, e.w, k + 1);
+  }
+  return leaf;
+}
+
 // Rope restart (neighbour links in the manner of Havran's ropes; the paper restarts every
 // segment by kd-restart).  The segment after leaf `prev`, which the ray left through its
 // face on plane pid0, begins in node N = the deepest node holding the level cell beyond
@@ -385,7 +423,15 @@ __device__ __forceinline__ int rope_start(const int32_t* __restrict__ face_node,
                                           float& e1, int lod_min) {
   const int a = pid0 & 3;
   const bool up = sel3f(a, rf.B[0], rf.B[1], rf.B[2]) > 0.0f;
-  const uint32_t ent = (uint32_t)__ldg(face_node + 12 * prev + 6 + 2 * a + (up ? 1 : 0));
+  uint32_t ent = (uint32_t)__ldg(face_node + 12 * prev + 6 + 2 * a + (up ? 1 : 0));
+  if ((ent & (kFaceLeaf | kFaceList)) == kFaceList) {
+    // several leaves beyond the face: the one the ray enters, to be checked like any other
+    const float x0 = fmaf(tau0, rf.Dd[0], rf.Xe[0]), x1 = fmaf(tau0, rf.Dd[1], rf.Xe[1]),
+                x2 = fmaf(tau0, rf.Dd[2], rf.Xe[2]);
+    uint32_t slot;
+    const int id = face_list_leaf(R.face_list, ent, a == 0 ? x1 : x0, a == 2 ? x1 : x2, 0, 0, slot);
+    ent = id >= 0 ? kFaceLeaf | (uint32_t)id : slot;
+  }
   int blo[3], bhi[3], anc;
   if (ent & kFaceLeaf) {
     const int4* w = reinterpret_cast<const int4*>(leaves + (ent & ~kFaceLeaf));
@@ -434,6 +480,9 @@ __device__ __forceinline__ int rope_start(const int32_t* __restrict__ face_node,
   return (ent & kFaceLeaf) ? (int)(ent & ~kFaceLeaf) : -2 - (int)ent;
 }
 
+// (A leaf picked from a list holds the ray just after t0 when these checks say so, on the
+// exit-face axis because it lies beyond the very face; when they do not, the descent is from
+// the push-down start.)
 // Leaf of the segment starting at (pid0, tau0) that follows leaf `prev` (-1 on the first
 // segment): by rope when prev is a leaf of the unpruned tree, else (or when the rope's
 // filter cannot decide, or a node above the rope's target may stop the pruned descent) by
@@ -800,9 +849,25 @@ __device__ __forceinline__ float neighbour_slow(const RenderArgs& A, const RayAr
   // from a pruned leaf (the table covers the unpruned leaves)
   uint32_t i = 0;
   if (leaf < R.n_leaves) {
-    const uint32_t ent =
+    uint32_t ent =
         (uint32_t)__ldg(A.face_node + 12 * leaf + (beyond ? 6 : 0) + 2 * a + (sign > 0.0f ? 1 : 0));
     bool ok = true;
+    if ((ent & (kFaceLeaf | kFaceList)) == kFaceList) {
+      // several leaves beyond the face: the one whose box holds the point beyond the margin,
+      // which no descent could miss then; else from the node they replace
+      uint32_t slot;
+      const int id = face_list_leaf(R.face_list, ent, a == 0 ? x1 : x0, a == 2 ? x1 : x2,
+                                    a == 0 ? lo1 : lo0, a == 2 ? lo1 : lo2, slot);
+      ent = slot;
+      if (id >= 0) {
+        const int4* w = reinterpret_cast<const int4*>(A.leaves + id);
+        const int4 w1 = __ldg(w + 1), w2 = __ldg(w + 2);  // lo[3], hi[0] | hi[1], hi[2], ...
+        const bool holds = x0 - (float)(w1.x - lo0) > mf && (float)(w1.w - lo0) - x0 > mf &&
+                           x1 - (float)(w1.y - lo1) > mf && (float)(w2.x - lo1) - x1 > mf &&
+                           x2 - (float)(w1.z - lo2) > mf && (float)(w2.y - lo2) - x2 > mf;
+        if (holds) ent = kFaceLeaf | (uint32_t)id;
+      }
+    }
     if (pruning) {
       const int anc = (ent & kFaceLeaf) ? __ldg(&A.leaves[ent & ~kFaceLeaf].lod_anc)
                                         : __ldg(&A.node_box[2 * ent].w);
