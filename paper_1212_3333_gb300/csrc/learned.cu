@@ -64,34 +64,74 @@ __device__ __forceinline__ bool log_keep(const LogArgs& L, int i, int j, int seg
   return (float)(h >> 8) * (1.0f / 16777216.0f) < L.keep_prob;
 }
 
-// WRITE = false: count the records each pixel keeps (the segments alone, no sampling);
-// WRITE = true: the march, each kept record written at its pixel's offset, so the records
-// of a view follow pixel and segment order whatever the thread schedule.
-template <int ST, bool WRITE>
-__global__ void __launch_bounds__(128) log_kernel(const __grid_constant__ RenderArgs A,
-                                                  const LogArgs L) {
-  extern __shared__ float4 smem[];
-  float4* s_tf = smem;
-  const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-  if constexpr (WRITE) {
-    for (int k = tid; k < A.tf_n; k += blockDim.x * blockDim.y) s_tf[k] = A.tf[k];
-    __syncthreads();
-  }
+// The records each pixel keeps (the segments alone, no sampling), one ray per thread.
+static __global__ void __launch_bounds__(32) log_count_kernel(const __grid_constant__ RenderArgs A,
+                                                              const LogArgs L) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int jr = blockIdx.y * blockDim.y + threadIdx.y;
   const int j = A.ray.row0 + jr;
   if (i >= A.ray.width || jr >= A.ray.rows || j >= A.ray.height) return;
-  const size_t pix = (size_t)jr * A.ray.width + i;
   int kept = 0;
   RayX rx;
-  if (!make_ray(A.ray, i, j, rx)) {
-    if constexpr (!WRITE) L.counts[pix] = 0;
-    return;
+  if (make_ray(A.ray, i, j, rx)) {
+    RayF rf;
+    make_frame(A.ray, rx, rf);
+    int pid0 = kPidIn;
+    float tau0 = 0.0f, e0 = 0.0f;
+    uint32_t start = 0;
+    int prev = -1;
+    for (int seg = 0; pid0 != kPidOut && seg < A.max_segments; ++seg) {
+      int pid1 = kPidOut;
+      float tau1 = rf.tau_out, e1 = exit_bound(rf);
+      const int lid = next_leaf(A.nodes, A.leaves, A.face_node, A.node_box, A.ray, i, j, rf, start,
+                                prev, pid0, tau0, e0, pid1, tau1, e1);
+      if (lid < 0) break;
+      prev = lid;
+      kept += log_keep(L, i, j, seg) ? 1 : 0;
+      pid0 = pid1;
+      tau0 = tau1;
+      e0 = e1;
+    }
   }
+  L.counts[(size_t)jr * A.ray.width + i] = kept;
+}
+
+// The march, each kept record written at its pixel's offset, so the records of a view follow
+// pixel and segment order whatever the thread schedule.  Eight lanes march one ray: they hold
+// the same ray state, take eight consecutive samples at once (two rounds of them in flight)
+// and add the opacities in sample order, lane by lane.  Views for logging are small (96^2 is
+// 288 warps of rays on 152 SMs), so with one ray per lane a view takes as long as its longest
+// rays' chains of loads; 8 views of the 5-level hierarchy, ms, one / eight lanes a ray:
+// 96^2 29.2 / 5.8, 2 views 160^2 7.0 / 1.9, 240^2 6.3 / 2.6.  With more rays than the chip holds
+// warps for, lanes on rays of their own do more: one view 400^2 (4 levels) 1.25 / 1.48, 600^2
+// 4.2 / 5.5, so views of more than kLogWidePixels keep one.
+constexpr int kLogRounds = 2;
+constexpr long long kLogWidePixels = 110000;
+template <int ST, int kLogLanes>
+__global__ void __launch_bounds__(128) log_kernel(const __grid_constant__ RenderArgs A,
+                                                  const LogArgs L) {
+  extern __shared__ float4 smem[];
+  float4* s_tf = smem;
+  for (int k = threadIdx.x; k < A.tf_n; k += 128) s_tf[k] = A.tf[k];
+  __syncthreads();
+  const int part = threadIdx.x % kLogLanes;
+  const unsigned group = ((1u << kLogLanes) - 1u) << (threadIdx.x & 31 & ~(kLogLanes - 1));
+  long long pix = (long long)blockIdx.x * (128 / kLogLanes) + threadIdx.x / kLogLanes;
+  if constexpr (kLogLanes == 1) {  // 8x4-pixel tiles
+    const int tiles_x = (A.ray.width + 7) / 8, lane = threadIdx.x & 31;
+    const long long t = pix >> 5;
+    const long long x = (t % tiles_x) * 8 + (lane & 7), y = (t / tiles_x) * 4 + (lane >> 3);
+    if (x >= A.ray.width) return;
+    pix = y * A.ray.width + x;
+  }
+  if (pix >= (long long)A.ray.width * A.ray.rows) return;
+  const int i = (int)(pix % A.ray.width), j = A.ray.row0 + (int)(pix / A.ray.width);
+  RayX rx;
+  if (j >= A.ray.height || !make_ray(A.ray, i, j, rx)) return;
   RayF rf;
   make_frame(A.ray, rx, rf);
-  float C0 = 0.f, C1 = 0.f, C2 = 0.f, Acc = 0.f;
-  unsigned nsamp = 0;
+  float Acc = 0.f;
+  int kept = 0;
   int pid0 = kPidIn;
   float tau0 = 0.0f, e0 = 0.0f;
   uint32_t start = 0;
@@ -103,34 +143,51 @@ __global__ void __launch_bounds__(128) log_kernel(const __grid_constant__ Render
                               prev, pid0, tau0, e0, pid1, tau1, e1);
     if (lid < 0) break;
     prev = lid;
-    if constexpr (WRITE) {
-      const DLeaf lf = A.leaves[lid];
-      const DLevel& lv = A.lv[lf.level];
-      int n = min(segment_count(A.ray, i, j, rf, pid0, tau0, e0, pid1, tau1, e1, lv),
-                  kMaxSamplesPerSegment);
-      float f[kMlpIn];
-      segment_features(A, rf, tau0, tau1, lf, Acc, f);
-      const float a_in = Acc;
-      SegSetup g;
-      setup_segment(A, rf, lf, lv, lid, pid0, pid1, tau0, e0, tau1, e1, n, i, j, g);
-      sample_segment<ST, 1, 0>(A, A.ray, s_tf, 0.0f, g, lv, 0.f, 0.f, 0.f, C0, C1, C2, Acc,
-                               nsamp);
-      if (log_keep(L, i, j, seg)) {
-        const unsigned long long idx = L.offsets[pix] + (unsigned long long)kept++;
-        if ((long long)idx < L.cap) {
+    const DLeaf lf = A.leaves[lid];
+    const DLevel& lv = A.lv[lf.level];
+    const int n = min(segment_count(A.ray, i, j, rf, pid0, tau0, e0, pid1, tau1, e1, lv),
+                      kMaxSamplesPerSegment);
+    const float a_in = Acc;
+    SegSetup g;
+    setup_segment(A, rf, lf, lv, lid, pid0, pid1, tau0, e0, tau1, e1, n, i, j, g);
+    if constexpr (kLogLanes == 1) {
+      float C0 = 0.f, C1 = 0.f, C2 = 0.f;
+      unsigned nsamp = 0;
+      sample_segment<ST, 1, 0>(A, A.ray, s_tf, 0.0f, g, lv, 0.f, 0.f, 0.f, C0, C1, C2, Acc, nsamp);
+    } else {
+      for (int k0 = 0; k0 < n; k0 += kLogLanes * kLogRounds) {
+        float v[kLogRounds], alpha[kLogRounds];
 #pragma unroll
-          for (int k = 0; k < kMlpIn; ++k) L.features[idx * kMlpIn + k] = f[k];
-          L.targets[idx] = Acc - a_in;
+        for (int r = 0; r < kLogRounds; ++r) {
+          const float k = (float)min(k0 + r * kLogLanes + part, n - 1);
+          v[r] = trilinear<ST>(A, g.s.brick, fmaf(k, g.db[0], g.b0[0]), fmaf(k, g.db[1], g.b0[1]),
+                               fmaf(k, g.db[2], g.b0[2]));
+        }
+#pragma unroll
+        for (int r = 0; r < kLogRounds; ++r) {
+          const float a = tf_alpha(s_tf, A.tf_n, v[r], A.vmin, A.inv_range);
+          const bool on = k0 + r * kLogLanes + part < n && a > 0.0f;
+          alpha[r] = on ? -expm1f(-A.kappa * a * g.delta) : 0.0f;
+          unsigned m = __ballot_sync(group, on) & group;
+          for (; m != 0; m &= m - 1)
+            Acc += (1.0f - Acc) * __shfl_sync(group, alpha[r], __ffs(m) - 1);
         }
       }
-    } else if (log_keep(L, i, j, seg)) {
-      ++kept;
+    }
+    if (log_keep(L, i, j, seg)) {
+      const unsigned long long idx = L.offsets[pix] + (unsigned long long)kept++;
+      if (part == 0 && (long long)idx < L.cap) {
+        float f[kMlpIn];
+        segment_features(A, rf, tau0, tau1, lf, a_in, f);
+#pragma unroll
+        for (int k = 0; k < kMlpIn; ++k) L.features[idx * kMlpIn + k] = f[k];
+        L.targets[idx] = Acc - a_in;
+      }
     }
     pid0 = pid1;
     tau0 = tau1;
     e0 = e1;
   }
-  if constexpr (!WRITE) L.counts[pix] = kept;
 }
 
 // Exclusive prefix sums of the view's per-pixel record counts, starting at the running
@@ -140,25 +197,31 @@ __global__ void __launch_bounds__(1024) log_scan_kernel(const int32_t* __restric
                                                         long long n,
                                                         unsigned long long* __restrict__ offsets,
                                                         unsigned long long* __restrict__ count) {
-  __shared__ unsigned long long part[1024];
-  const int t = threadIdx.x;
+  __shared__ unsigned long long warp_sum[32];
+  const int t = threadIdx.x, lane = t & 31;
   const long long chunk = (n + 1023) / 1024;
   const long long lo = min(n, (long long)t * chunk), hi = min(n, lo + chunk);
   unsigned long long s = 0;
   for (long long k = lo; k < hi; ++k) s += (unsigned long long)counts[k];
-  part[t] = s;
-  __syncthreads();
-  if (t == 0) {
-    unsigned long long run = *count;
-    for (int q = 0; q < 1024; ++q) {
-      const unsigned long long v = part[q];
-      part[q] = run;
-      run += v;
+  auto scan = [&](unsigned long long v) {  // inclusive, over the warp
+#pragma unroll
+    for (int d = 1; d < 32; d *= 2) {
+      const unsigned long long u = __shfl_up_sync(0xffffffffu, v, d);
+      if (lane >= d) v += u;
     }
-    *count = run;
+    return v;
+  };
+  const unsigned long long in_warp = scan(s);
+  if (lane == 31) warp_sum[t >> 5] = in_warp;
+  const unsigned long long run0 = *count;
+  __syncthreads();
+  if (t < 32) {
+    const unsigned long long v = warp_sum[lane], w = scan(v);
+    warp_sum[lane] = w - v;
+    if (lane == 31) *count = run0 + w;
   }
   __syncthreads();
-  unsigned long long run = part[t];
+  unsigned long long run = run0 + warp_sum[t >> 5] + in_warp - s;
   for (long long k = lo; k < hi; ++k) {
     offsets[k] = run;
     run += (unsigned long long)counts[k];
@@ -351,9 +414,9 @@ amr_status launch_learned(amr_ctx* c, const RenderArgs& a, int storage, int shad
 amr_status launch_log(amr_ctx* c, const RenderArgs& a, int storage, float* features,
                       float* targets, long long cap, unsigned long long* count, float keep_prob,
                       uint32_t seed, void* stream) {
-  const dim3 block(8, 16);
-  const dim3 grid((unsigned)((a.ray.width + 7) / 8), (unsigned)((a.ray.rows + 15) / 16));
-  if (grid.x == 0 || grid.y == 0) return AMR_OK;
+  const dim3 block(8, 4);
+  const dim3 grid((unsigned)((a.ray.width + 7) / 8), (unsigned)((a.ray.rows + 3) / 4));
+  if (a.ray.width <= 0 || a.ray.rows <= 0) return AMR_OK;
   if (storage != ST_PTR && storage != ST_ATLAS_LINEAR)
     return fail(c, AMR_ERR_ARG, "segment logging needs the ptr or atlas_linear storage");
   // per-pixel counts and offsets of the view (grown as needed, kept with the context)
@@ -377,11 +440,13 @@ amr_status launch_log(amr_ctx* c, const RenderArgs& a, int storage, float* featu
   LogArgs L{features, targets, cap, count, keep_prob, seed, d.log_counts, d.log_offsets};
   const size_t smem = (size_t)a.tf_n * sizeof(float4);
   cudaStream_t s = (cudaStream_t)stream;
-  if (storage == ST_PTR) log_kernel<ST_PTR, false><<<grid, block, 0, s>>>(a, L);
-  else log_kernel<ST_ATLAS_LINEAR, false><<<grid, block, 0, s>>>(a, L);
+  log_count_kernel<<<grid, block, 0, s>>>(a, L);
   log_scan_kernel<<<1, 1024, 0, s>>>(d.log_counts, (long long)pixels, d.log_offsets, count);
-  if (storage == ST_PTR) log_kernel<ST_PTR, true><<<grid, block, smem, s>>>(a, L);
-  else log_kernel<ST_ATLAS_LINEAR, true><<<grid, block, smem, s>>>(a, L);
+  const bool wide = (long long)pixels <= kLogWidePixels;
+  const size_t lanes = wide ? pixels * 8 : (size_t)grid.x * grid.y * 32;
+  auto run = [&](auto kernel) { kernel<<<(unsigned)((lanes + 127) / 128), 128, smem, s>>>(a, L); };
+  if (storage == ST_PTR) wide ? run(log_kernel<ST_PTR, 8>) : run(log_kernel<ST_PTR, 1>);
+  else wide ? run(log_kernel<ST_ATLAS_LINEAR, 8>) : run(log_kernel<ST_ATLAS_LINEAR, 1>);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess)
     return fail(c, AMR_ERR_CUDA, std::string("segment log launch: ") + cudaGetErrorString(e));

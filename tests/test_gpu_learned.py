@@ -183,6 +183,29 @@ def test_segment_log_invariants(mods, c1_learned):
     assert abs(seen_half - 0.5 * seen) <= 0.05 * seen
 
 
+@pytest.mark.parametrize("storage", ["ptr", "atlas_linear"])
+def test_segment_log_bands_equal_the_whole_view(mods, c1_learned, storage):
+    """A view of more than 110,000 pixels is logged one ray per lane, its bands eight lanes a
+    ray: the bands' records, one after the other, are the view's bit for bit."""
+    torch, amr, proposal = mods
+    w, _ = c1_learned
+    ctx = amr.from_hierarchy(w["hier"])
+    ctx.amr_build_kdtree(storage)
+    cam = synth.orbit_camera(11, 401, 301)
+    tf = torch.as_tensor(w["tf"], device="cuda")
+
+    def log(row0, rows):
+        p, _ = params_pair(amr, w["vmin"], w["vmax"], row0=row0, rows=rows)
+        x, y, n = proposal.log_segments(ctx, [cam], tf, p, capacity=1 << 20, keep_prob=0.3, seed=5)
+        return x.clone(), y.clone(), n
+
+    whole = log(0, 0)
+    bands = [log(0, 33), log(33, 199), log(232, 69)]
+    assert whole[2] == sum(b[2] for b in bands) > 10000
+    for k in (0, 1):
+        assert torch.equal(whole[k], torch.cat([b[k] for b in bands]))
+
+
 def test_learned_render_with_zero_threshold_is_the_plain_march(mods, c1_learned):
     torch, amr, proposal = mods
     w, ctx = c1_learned
