@@ -406,8 +406,16 @@ __device__ __forceinline__ int march_tile(const RenderArgs& A, const RayArgs& R,
   return kTileDone;
 }
 
+// resident blocks the register budgets allow for.  The ray frame (22 words, read once per
+// segment) lies in shared memory; measured, ms, frame in registers / shared, shaded with 4
+// blocks: atlas 512^2 1.87 / 1.78, 640 x 479 2.44 / 2.39, 1024^2 7.00 / 6.81, 32-view batch 25.2 /
+// 24.3 (5 blocks 2.03, 2.59, 7.16, 26.0); unshaded f16 1917 x 1083 4.39 in registers with 4
+// blocks, shared with 4 / 5 / 6 / 7 blocks 4.54 / 4.28 / 4.65 / 5.09.
 #ifndef AMR_SPLIT_MARCH_BLOCKS
 #define AMR_SPLIT_MARCH_BLOCKS 4
+#endif
+#ifndef AMR_SPLIT_PLAIN_BLOCKS
+#define AMR_SPLIT_PLAIN_BLOCKS 5
 #endif
 #ifndef AMR_SPLIT_SHADE_BLOCKS
 #define AMR_SPLIT_SHADE_BLOCKS 6
@@ -418,7 +426,7 @@ __device__ __forceinline__ int march_tile(const RenderArgs& A, const RayArgs& R,
 
 // Persistent warps taking 8x4-pixel tiles from a queue, as march_kernel does.
 template <int ST, int SHADE, typename Args = RenderArgs>
-__global__ void __launch_bounds__(128, AMR_SPLIT_MARCH_BLOCKS)
+__global__ void __launch_bounds__(128, (SHADE & 3) != 0 ? AMR_SPLIT_MARCH_BLOCKS : AMR_SPLIT_PLAIN_BLOCKS)
     split_march_kernel(const __grid_constant__ Args P) {
   constexpr bool SHADED = (SHADE & 3) != 0;
   const RenderArgs& A = render_args(P);
@@ -441,7 +449,8 @@ __global__ void __launch_bounds__(128, AMR_SPLIT_MARCH_BLOCKS)
   unsigned nsamp = 0;
   unsigned long long status = 0;
   SegBlock blk;
-  RayF rf;
+  __shared__ RayFSlot s_rf[128];
+  RayF& rf = s_rf[tid].f;
   // each pass takes one tile, and the queue hands out every tile once
   for (;;) {
     int t = n_tiles;
