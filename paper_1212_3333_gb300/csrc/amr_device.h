@@ -38,6 +38,8 @@ constexpr int kQueueCounter = 5;       // counters[5]: head of the batched work 
 constexpr int kShadeShadowBit = 4;     // kernel shading variant bit: secondary rays
 constexpr int kShadeMaxBit = 8;        // kernel variant bit: stencil-maximum opacity test
 constexpr int kMaxBatchViews = 128;
+constexpr long long kLargePixels = 3000000;  // images where the per-ray loop beats the
+                                             // one-kernel deferred march
 // status bits raised by kernels (OR-ed into counters[1])
 constexpr unsigned long long kStatusCapacity = 1ull;   // segment or sample bound hit
 constexpr unsigned long long kStatusDevice = 2ull;     // malformed tree reached

@@ -324,7 +324,6 @@ static bool textures(const amr_ctx* c) {
 // stay on the per-ray schedule in texture storages, whose deferred march has no workspace and
 // loses there (1900 x 1800: 31.8 against 37 ms), and when samples_per_iter, which only
 // deferred shading reads, is outside its range.
-constexpr int64_t kLargePixels = 3000000;
 
 static const amr_render_params* resolve_schedule(const amr_render_params* p, int64_t pixels,
                                                  bool textures, amr_render_params* tmp) {

@@ -94,6 +94,8 @@ struct DeviceState {
   // earlier ones stay for CUDA graphs that hold their addresses (sizes at least double)
   std::vector<void*> task_spaces;
   TaskSpace tasks = {};
+  cudaEvent_t task_event = nullptr;  // after the last call that used a workspace,
+  cudaStream_t task_stream = nullptr;  // on this stream
   float dense_below = -INFINITY;     // a fifth of the cells lie below this value
   int64_t task_pixels = 0;
   int64_t task_refused = INT64_MAX;  // a workspace for this many pixels could not be allocated
@@ -151,8 +153,11 @@ amr_status upload(amr_ctx* c, void* stream);
 void release_device(amr_ctx* c);
 // The split march's workspace for a call with that many 8x4 tiles, grown when it is too small
 // and the stream is not being captured; it may have fewer tiles (out of memory, or a first
-// call captured: none).
+// call captured: none).  A call on another stream waits for the workspace's last one;
+// tasks_queued marks where a call ends.  (Captured calls neither wait nor are waited for: as
+// before, a replay must not overlap other work of the context.)
 TaskPlan plan_tasks(amr_ctx* c, long long tiles, void* stream);
+cudaError_t tasks_queued(amr_ctx* c, void* stream);
 // kernels (march.cu)
 amr_status launch_render(amr_ctx* c, const RenderArgs& a, int storage, int interp, int shade,
                          int schedule, void* stream);

@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cstring>
 #include <deque>
+#include <new>
 
 #include "ctx.h"
 #include "storage16.h"
@@ -289,9 +290,15 @@ TaskPlan plan_tasks(amr_ctx* c, long long call_tiles, void* stream) {
   DeviceState& d = c->dev;
   if (call_tiles <= 0) return plan;
   const int64_t want = std::min<int64_t>(call_tiles * 32, std::max<int64_t>(kBandPixels, 32 * 8192));
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing((cudaStream_t)stream, &cap) != cudaSuccess) cudaGetLastError();
+  if (cap == cudaStreamCaptureStatusNone && !d.task_event &&
+      cudaEventCreateWithFlags(&d.task_event, cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    d.task_event = nullptr;
+    return plan;
+  }
   if (want > d.task_pixels && want < d.task_refused) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing((cudaStream_t)stream, &cap) != cudaSuccess) cudaGetLastError();
     const int64_t px = std::max(want, std::min(2 * d.task_pixels, kBandPixels));
     const int64_t tiles = px / 32;
     const int64_t under_way = std::min(tiles, kWarps) * kTileChunks * kTaskChunk * 4 / 3;
@@ -334,9 +341,24 @@ TaskPlan plan_tasks(amr_ctx* c, long long call_tiles, void* stream) {
       d.tasks.seg_blocks = (int32_t)blocks;
     }
   }
+  if (d.task_pixels == 0) return plan;
+  if (cap == cudaStreamCaptureStatusNone && d.task_stream != (cudaStream_t)stream &&
+      cudaStreamWaitEvent((cudaStream_t)stream, d.task_event, 0) != cudaSuccess) {
+    cudaGetLastError();
+    return plan;
+  }
   plan.ts = d.tasks;
   plan.tiles = d.task_pixels / 32;
   return plan;
+}
+
+cudaError_t tasks_queued(amr_ctx* c, void* stream) {
+  DeviceState& d = c->dev;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing((cudaStream_t)stream, &cap);
+  if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) return e;
+  d.task_stream = (cudaStream_t)stream;
+  return cudaEventRecord(d.task_event, (cudaStream_t)stream);
 }
 
 void release_device(amr_ctx* c) {
@@ -372,22 +394,24 @@ void release_device(amr_ctx* c) {
   cudaFree(d.log_counts);
   cudaFree(d.log_offsets);
   for (void* p : d.task_spaces) cudaFree(p);
+  if (d.task_event) cudaEventDestroy(d.task_event);
   d = DeviceState();
   c->device_built = false;
 }
 
 // The leaves beyond face f (2 axis + side) of leaf m, all in the subtree of pre-order node
-// `pre`, as a list at the end of `lists` (RayArgs::face_list): its word, or 0 when there are too
-// many, their rectangles do not fit the bytes, or the face is one of the root's.
-static uint32_t face_list(const Tree& t, const int64_t* root, size_t m, int f, int32_t pre,
+// `pre`, as a list at the end of `lists` (RayArgs::face_list): its word there, or -1 when there
+// are too many, their rectangles do not fit the bytes, or the face is one of the root's.
+static int32_t face_list(const Tree& t, const int64_t* root, size_t m, int f, int32_t pre,
                           int32_t slot, std::vector<int4>& lists) {
   const int32_t* box = &t.leaf_box[6 * m];
   const int a = f >> 1, b = a == 0 ? 1 : 0, c = a == 2 ? 1 : 2;
   const int64_t plane = (f & 1) ? box[3 + a] : box[a];
-  if (plane == ((f & 1) ? root[3 + a] : root[a])) return 0;
+  if (plane == ((f & 1) ? root[3 + a] : root[a])) return -1;
   const int64_t cell = (f & 1) ? plane : plane - 1;  // the finest cells beyond the face
   struct Rect { int32_t u0, u1, v0, v1, id; };
-  std::vector<Rect> r;
+  Rect r[kFaceListMax];
+  int n = 0;
   std::vector<int32_t> stack(1, pre);
   while (!stack.empty()) {
     const int32_t i = stack.back();
@@ -396,9 +420,9 @@ static uint32_t face_list(const Tree& t, const int64_t* root, size_t m, int f, i
     if (ax < 0) {
       const int32_t id = t.leaf[i];
       const int32_t* q = &t.leaf_box[6 * (size_t)id];
-      if (r.size() == (size_t)kFaceListMax) return 0;
-      r.push_back({std::max(q[b], box[b]) - box[b], std::min(q[3 + b], box[3 + b]) - box[b],
-                   std::max(q[c], box[c]) - box[c], std::min(q[3 + c], box[3 + c]) - box[c], id});
+      if (n == kFaceListMax) return -1;
+      r[n++] = {std::max(q[b], box[b]) - box[b], std::min(q[3 + b], box[3 + b]) - box[b],
+                   std::max(q[c], box[c]) - box[c], std::min(q[3 + c], box[3 + c]) - box[c], id};
       continue;
     }
     const int64_t sp = t.split[i], lo = ax == a ? cell : box[ax], hi = ax == a ? cell + 1 : box[3 + ax];
@@ -406,17 +430,16 @@ static uint32_t face_list(const Tree& t, const int64_t* root, size_t m, int f, i
     if (hi > sp) stack.push_back(t.right[i]);
   }
   int32_t bits = 0;  // the rectangles' unit: the largest power of two in all their corners
-  for (const Rect& q : r) bits |= q.u0 | q.u1 | q.v0 | q.v1;
-  if (bits == 0) return 0;
+  for (int k = 0; k < n; ++k) bits |= r[k].u0 | r[k].u1 | r[k].v0 | r[k].v1;
+  if (bits == 0) return -1;
   const int shift = __builtin_ctz((unsigned)bits);
-  for (const Rect& q : r)
-    if ((q.u1 >> shift) > 255 || (q.v1 >> shift) > 255) return 0;
+  for (int k = 0; k < n; ++k)
+    if ((r[k].u1 >> shift) > 255 || (r[k].v1 >> shift) > 255) return -1;
   const size_t word = lists.size();
-  if (word + 1 + kFaceListMax / 2 >= (size_t)kFaceList) return 0;
-  lists.push_back(int4{box[b], box[c], slot, (int)r.size() + 32 * shift});
-  for (size_t k = 0; k < r.size(); k += 2) {
+  lists.push_back(int4{box[b], box[c], slot, n + 32 * shift});
+  for (int k = 0; k < n; k += 2) {
     int4 w = {0, 0, 0, 0};
-    for (size_t e = 0; e < 2 && k + e < r.size(); ++e) {
+    for (int e = 0; e < 2 && k + e < n; ++e) {
       const Rect& q = r[k + e];
       const uint32_t p = (uint32_t)(q.u0 >> shift) | (uint32_t)(q.u1 >> shift) << 8 |
                          (uint32_t)(q.v0 >> shift) << 16 | (uint32_t)(q.v1 >> shift) << 24;
@@ -425,7 +448,7 @@ static uint32_t face_list(const Tree& t, const int64_t* root, size_t m, int f, i
     }
     lists.push_back(w);
   }
-  return (uint32_t)word;
+  return (int32_t)word;
 }
 
 // The value a fifth of the bricks' cells lie below, from at most about 2^16 of them.
@@ -463,14 +486,37 @@ amr_status upload(amr_ctx* c, void* stream_v) {
       (nodes[0].meta >> 30) != (uint32_t)kLeafAxis)
     nodes[0].meta &= ~kIndexMask;  // the root's children become slots 0 (itself) and 1
   std::vector<int32_t> face_slots(std::max<size_t>(1, t.face_node.size()), 0);
-  std::vector<int4> face_lists(1, int4{0, 0, 0, 0});
   for (size_t k = 0; k < t.face_node.size(); ++k) {
     const int32_t pre = t.face_node[k];
     face_slots[k] = t.axis[pre] < 0 ? (int32_t)(kFaceLeaf | (uint32_t)t.leaf[pre]) : slot_of[pre];
-    if (t.axis[pre] >= 0 && k % 12 >= 6) {
-      const uint32_t list = face_list(t, c->root, k / 12, (int)(k % 12) - 6, pre, slot_of[pre], face_lists);
-      if (list) face_slots[k] = (int32_t)(kFaceList | list);
+  }
+  // leaf lists for the faces whose node is an inner one: per leaf, then one after the other
+  std::vector<std::vector<int4>> leaf_lists(M);
+  std::vector<int32_t> list_word(6 * M, -1);
+  bool no_memory = false;  // (an exception may not leave the parallel loop)
+#pragma omp parallel for schedule(dynamic, 256)
+  for (long long m = 0; m < (long long)M; ++m) {
+    try {
+      for (int f = 0; f < 6; ++f) {
+        const int32_t pre = t.face_node[12 * (size_t)m + 6 + f];
+        if (t.axis[pre] >= 0)
+          list_word[6 * (size_t)m + f] =
+              face_list(t, c->root, (size_t)m, f, pre, slot_of[pre], leaf_lists[(size_t)m]);
+      }
+    } catch (const std::bad_alloc&) {
+#pragma omp atomic write
+      no_memory = true;
     }
+  }
+  if (no_memory) throw std::bad_alloc();
+  std::vector<int4> face_lists;
+  for (size_t m = 0; m < M; ++m) {
+    const size_t base = face_lists.size();
+    if (base + leaf_lists[m].size() >= (size_t)kFaceList) break;
+    face_lists.insert(face_lists.end(), leaf_lists[m].begin(), leaf_lists[m].end());
+    for (int f = 0; f < 6; ++f)
+      if (list_word[6 * m + f] >= 0)
+        face_slots[12 * m + 6 + f] = (int32_t)(kFaceList | (uint32_t)(base + list_word[6 * m + f]));
   }
   face_lists.resize(face_lists.size() + kFaceListMax / 2, int4{0, 0, 0, 0});
   const size_t ML = t.lod_patch.size();

@@ -1856,6 +1856,8 @@ static_assert(AMR_WARP_TILE_W == 4 || AMR_WARP_TILE_W == 8 || AMR_WARP_TILE_W ==
 template <int ST, int INTERP, int SHADE, bool QUEUE = true>
 __global__ void __launch_bounds__(128, kMinBlocks<SHADE>)
     march_kernel(const __grid_constant__ RenderArgs A) {
+  // (with a workspace: only an image that the split march did not begin)
+  if (A.ts.heads && __ldcg(A.ts.heads + kHeadTile) != 0) return;
   extern __shared__ float4 smem[];
   float4* s_tf = smem;
   int* s_nz = reinterpret_cast<int*>(smem + A.tf_n);

@@ -18,6 +18,8 @@
 // change.  (With secondary rays each light ray's transmittance is a product taken in
 // another order - 32 samples per round - so those images agree to rounding, not bits.)
 #pragma once
+#include <type_traits>
+
 #include "march.cuh"
 
 namespace amr {
@@ -433,6 +435,9 @@ __global__ void __launch_bounds__(128, AMR_MIN_BLOCKS_DEFERRED)
     dense = (int)__ldcg(A.ts.heads + kHeadDense);
     begun = (int)min(__ldcg(A.ts.heads + kHeadTile), (unsigned)all_tiles);
     if (left == 0 && dense == 0 && begun == all_tiles) return;
+    if (std::is_same<Args, RenderArgs>::value && (SHADE & kShadeShadow) == 0 &&
+        begun == 0 && all_tiles * 32LL >= kLargePixels)
+      return;  // march_kernel has rendered it
   }
   extern __shared__ float4 smem[];
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;

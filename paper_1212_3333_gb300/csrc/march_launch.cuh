@@ -1,6 +1,7 @@
 // Template launcher shared by the per-storage translation units.
 #pragma once
 #include <algorithm>
+#include <type_traits>
 
 #include "ctx.h"
 #include "march.cuh"
@@ -122,9 +123,12 @@ cudaError_t launch_rounds(int rounds, cudaStream_t s, const Args& b) {
     if (e == cudaSuccess) e = launch_stride(split_outer_kernel<ST, SHADE, Args>, base, s, b, 4);
     if (e == cudaSuccess) e = launch_stride(split_sum_kernel<Args>, 0, s, b, 4);
   }
-  if (e == cudaSuccess)
-    e = launch_tiles(deferred_kernel<ST, SHADE, Args>, base + 4 * sizeof(DeferArea), s, b);
-  return e;
+  // an image whose tiles are all dense (every sample opaque, ms: 1024^2 46 deferred, 49 per ray
+  // before; 2048^2 146 deferred, 119 per ray)
+  if constexpr (std::is_same<Args, RenderArgs>::value && (SHADE & kShadeShadow) == 0)
+    if (tiles_of(b) * 32 >= kLargePixels) e = launch_tiles(march_kernel<ST, 1, SHADE>, base, s, b);
+  if (e != cudaSuccess) return e;
+  return launch_tiles(deferred_kernel<ST, SHADE, Args>, base + 4 * sizeof(DeferArea), s, b);
 }
 
 // Deferred shading of one image: the split march in bands of rows that the workspace has tile
@@ -260,6 +264,7 @@ amr_status launch_storage(amr_ctx* c, const RenderArgs& a, int interp, int shade
     else e = launch_one(wave_kernel<ST, 0, 1>, grid, block, smem, s, a);
   }
 launched:
+  if (e == cudaSuccess && plan.tiles > 0) e = tasks_queued(c, s);
   if (e != cudaSuccess)
     return fail(c, AMR_ERR_CUDA, std::string("march launch: ") + cudaGetErrorString(e));
   return AMR_OK;

@@ -445,6 +445,8 @@ __global__ void __launch_bounds__(128, (SHADE & 3) != 0 ? AMR_SPLIT_MARCH_BLOCKS
   Area& Q = reinterpret_cast<Area*>(reinterpret_cast<char*>(smem) +
                                     StagedTf<Args>::bytes(P))[tid >> 5];
   const StagedTf<Args> staged(P, smem, tid);
+  if constexpr (SHADED && std::is_same<Args, RenderArgs>::value)
+    if (staged.clear <= A.dense_below) return;  // every tile is dense (below)
   const int lane = tid & 31;
   unsigned nsamp = 0;
   unsigned long long status = 0;

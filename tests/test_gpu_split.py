@@ -98,3 +98,28 @@ def test_first_call_captured(amr):
     torch.cuda.synchronize()
     assert float(out[1].abs().max()) > 0
     assert torch.equal(out[0], out[1]) and torch.equal(again, out[1])
+
+
+def test_calls_on_two_streams_take_turns(amr):
+    """The streams share the context's workspace: the second call waits for the first."""
+    import torch
+
+    ctx, (vmin, vmax) = _context(amr)
+    cams = [synth.orbit_camera(s, 180, 150) for s in (1, 2)]
+    tf = torch.as_tensor(_opaque_tf(), device="cuda")
+    p, _ = params_pair(amr, vmin, vmax, schedule=3, shade=1, step_factor=0.05, kappa=0.2)
+    want = []
+    for cam in cams:
+        out = torch.zeros((150, 180, 4), device="cuda")
+        ctx.amr_render(cam, tf, p, out)
+        torch.cuda.synchronize()
+        want.append(out)
+    streams = [torch.cuda.Stream() for _ in cams]
+    got = [torch.zeros_like(w) for w in want]
+    torch.cuda.synchronize()
+    for _ in range(3):
+        for cam, st, out in zip(cams, streams, got):
+            ctx.amr_render(cam, tf, p, out, stream=st)
+    torch.cuda.synchronize()
+    for g, w in zip(got, want):
+        assert torch.equal(g, w)
