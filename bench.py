@@ -594,6 +594,12 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
+def _launches(args, size: int) -> int:
+    """Kernels of one frame: one, or under deferred shading at least march, shading, outer
+    gradients, sums and what is left (one round; a frame this size takes two or more)."""
+    return 5 if args.schedule == 3 and args.storage in ("ptr", "atlas_linear") else 1
+
+
 def _config(hier, args, storage, size=SIZE):
     return {"workload": (f"c2: lognormal 5-level AMR, {hier.num_patches} patches, "
                          f"{hier.n_cells():.3g} FP32 cells; {size}x{size} view; "
@@ -626,8 +632,9 @@ def main():
     ap.add_argument("--cpu-baseline", type=int, default=1)
     ap.add_argument("--e2e", type=int, default=1, help="also time the host-buffer entry point")
     ap.add_argument("--size", type=int, default=SIZE, help="image side (the metric is at 2048)")
-    ap.add_argument("--schedule", type=int, default=0,
-                    help="0 per-ray loop, 1 warp wavefront, 2 refill, 3 deferred shading")
+    ap.add_argument("--schedule", type=int, default=None,
+                    help="0 per-ray loop, 1 warp wavefront, 2 refill, 3 deferred shading "
+                         "(default: what the library chooses, 3 with --shade 1, else 0)")
     ap.add_argument("--spi", type=int, default=16, help="samples per step, schedules 2 and 3")
     ap.add_argument("--schedules", type=int, default=1,
                     help="time schedules 0 / 2 / 3 at 2048, 1024 and 512 pixels")
@@ -653,6 +660,8 @@ def main():
     ap.add_argument("--epochs", type=int, default=3)
     ap.add_argument("--heldout", type=int, default=8)
     args = ap.parse_args()
+    if args.schedule is None:
+        args.schedule = 3 if args.shade else 0
     if args.impl == "reference":
         return run_reference(args)
 
@@ -763,7 +772,7 @@ def main():
             "counters": (f"profiles/march_counters.json, sources {prof['sources']}"
                          if prof else "stale or missing for the current kernel sources"),
             "kernel": {0: "march_kernel", 1: "wave_kernel", 2: "persist_kernel",
-                       3: "deferred_kernel"}[args.schedule] +
+                       3: "split_march_kernel and its shading kernels"}[args.schedule] +
                       f"<{variant}, trilinear, {'phong' if args.shade else 'plain'}>",
             "kernel_ms": kern_ms}
     extra = {"frames_per_s": fps, "samples_per_frame": samples, "build_s": build_s,
@@ -828,7 +837,7 @@ def main():
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": args.dtype, "data": "synthetic",
-            "config": _config(hier, args, args.storage, size), "gpu_launches": args.steps,
+            "config": _config(hier, args, args.storage, size), "gpu_launches": args.steps * _launches(args, size),
             "e2e": e2e, "roofline": roof, "clocks": clk, "extra": extra}
     if args.cpu_baseline and world == 1:
         line["cpu_baseline"] = cpu_baseline(hier, cam, tf_h, vmin, vmax, args.shade)

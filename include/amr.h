@@ -207,6 +207,12 @@ amr_status amr_build_host(amr_ctx* ctx, amr_storage storage);
  * [vmin, vmax].  Both device buffers must be 16-byte aligned.  Asynchronous on cuda_stream.  samples_out (nullable, host): when given,
  * the call synchronises the stream, checks the device status word and stores the exact
  * number of samples taken (sum over segments of the per-segment sample count).
+ * Deferred shading (schedule 3, linear storages) keeps a workspace with the context: the first
+ * call of a size that is not being captured allocates it (1.7 GB for most images, 3.5 GB at
+ * most; without it the call renders the same image with the one-kernel march), a larger one
+ * is added when a larger image needs it, and amr_destroy or another build frees them, so a
+ * captured call stays valid until then.  Calls on several streams take turns on it; a graph's
+ * replay must not overlap other work of the context.
  * 16-bit cells render trilinear with the per-ray schedule (else AMR_ERR_ARG). */
 amr_status amr_render(amr_ctx* ctx, const amr_camera* cam, const float* tf_rgba_dev,
                       int32_t tf_n, const amr_render_params* params, float* out_rgba_dev,
@@ -280,9 +286,10 @@ typedef struct {
  *                  the params' samples_per_iter)
  * Needs the ptr storage with FP32 cells, trilinear sampling, schedule 0 (per-ray loop) or
  * 3 (deferred shading, shade = 1), no learned proposal and no secondary rays (else
- * AMR_ERR_ARG).  Issues one cudaMemsetAsync and one kernel launch
- * on cuda_stream and allocates nothing, so with samples_out NULL the call can be captured
- * in a CUDA graph; samples_out (nullable, host) synchronises and returns the total sample
+ * AMR_ERR_ARG).  Deferred shading uses the context's workspace (see amr_render) and then,
+ * of the configuration, only samples_per_iter; the per-ray loop, and deferred shading without
+ * a workspace, issue one cudaMemsetAsync and one kernel launch.  With samples_out NULL the call
+ * can be captured in a CUDA graph; samples_out (nullable, host) synchronises and returns the total sample
  * count of all views (plus the device status check, as amr_render). */
 amr_status amr_render_batch(amr_ctx* ctx, const amr_view* views, int32_t n_views,
                             const float* tfs_rgba_dev, int32_t n_tf, int32_t tf_n,

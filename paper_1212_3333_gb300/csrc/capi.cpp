@@ -321,19 +321,19 @@ static bool textures(const amr_ctx* c) {
 // (schedule 3) wherever it applies - Phong, trilinear, no learned proposal - and the per-ray
 // schedule otherwise.  Every schedule gives the same image bit for bit (with secondary rays to
 // rounding), so the choice affects time only.  Single images of kLargePixels pixels and more
-// stay on the per-ray schedule in texture storages, whose deferred march has no workspace and
-// loses there (1900 x 1800: 31.8 against 37 ms), and when samples_per_iter, which only
+// stay on the per-ray schedule where deferred shading has no workspace - texture storages, calls
+// that may not allocate - and loses (textures, 1900 x 1800: 31.8 against 37 ms), and when samples_per_iter, which only
 // deferred shading reads, is outside its range.
 
 static const amr_render_params* resolve_schedule(const amr_render_params* p, int64_t pixels,
-                                                 bool textures, amr_render_params* tmp) {
+                                                 bool one_kernel, amr_render_params* tmp) {
   if (!p || p->schedule != AMR_SCHEDULE_AUTO) return p;
   *tmp = *p;
   const bool deferred_applies = p->interp == AMR_INTERP_TRILINEAR && p->shade == 1 &&
                                 p->learned == 0;
   const bool steps = p->samples_per_iter >= 1 && p->samples_per_iter <= 64;
   tmp->schedule =
-      deferred_applies && ((steps && !textures) || p->shadow || pixels < kLargePixels) ? 3 : 0;
+      deferred_applies && ((steps && !one_kernel) || p->shadow || pixels < kLargePixels) ? 3 : 0;
   return tmp;
 }
 
@@ -477,10 +477,9 @@ amr_status prepare_render_args(amr_ctx* c, const amr_camera* cam, int32_t tf_n,
                                const amr_render_params* p, RenderArgs* a) {
   return prepare_render(c, cam, tf_n, p, a);
 }
-amr_render_params resolve_render_schedule(const amr_ctx* c, const amr_camera* cam,
-                                          const amr_render_params& p) {
+amr_render_params resolve_render_schedule(const amr_camera* cam, const amr_render_params& p) {
   amr_render_params tmp;
-  return *resolve_schedule(&p, call_pixels(cam, &p), textures(c), &tmp);
+  return *resolve_schedule(&p, call_pixels(cam, &p), true, &tmp);
 }
 amr_status launch_render_args(amr_ctx* c, const RenderArgs& a, const amr_render_params* p,
                               void* stream) {

@@ -180,8 +180,7 @@ amr_status prepare_render_args(amr_ctx* c, const amr_camera* cam, int32_t tf_n,
                                const amr_render_params* p, RenderArgs* a);
 amr_status launch_render_args(amr_ctx* c, const RenderArgs& a, const amr_render_params* p,
                               void* stream);
-// params with AMR_SCHEDULE_AUTO replaced by the schedule a single-view call would use
-amr_render_params resolve_render_schedule(const amr_ctx* c, const amr_camera* cam,
-                                          const amr_render_params& p);
+// params with AMR_SCHEDULE_AUTO replaced by the schedule a call without a workspace uses
+amr_render_params resolve_render_schedule(const amr_camera* cam, const amr_render_params& p);
 
 }  // namespace amr

@@ -317,7 +317,12 @@ TaskPlan plan_tasks(amr_ctx* c, long long call_tiles, void* stream) {
     for (int k = 0; k < 10; ++k) off[k + 1] = off[k] + ((sizes[k] + 255) & ~(size_t)255);
     char* p = nullptr;
     if (cap == cudaStreamCaptureStatusNone) {
-      if (cudaMalloc((void**)&p, off[10]) != cudaSuccess) {
+      // (relaxed: another thread's capture must not be disturbed, nor refuse this)
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      cudaThreadExchangeStreamCaptureMode(&mode);
+      const cudaError_t e = cudaMalloc((void**)&p, off[10]);
+      cudaThreadExchangeStreamCaptureMode(&mode);
+      if (e != cudaSuccess) {
         cudaGetLastError();
         p = nullptr;
         d.task_refused = want;

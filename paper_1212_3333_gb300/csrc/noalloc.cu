@@ -82,7 +82,7 @@ extern "C" amr_status amr_render_host_noalloc(amr_ctx* c, const amr_camera* cam,
   if (!cam || !params_in || !tf_rgba_host || !out_rgba_host)
     return fail(c, AMR_ERR_ARG, "NULL argument");
   // the schedule follows the whole frame, not the bands it is rendered in
-  const amr_render_params resolved = resolve_render_schedule(c, cam, *params_in);
+  const amr_render_params resolved = resolve_render_schedule(cam, *params_in);
   const amr_render_params* params = &resolved;
   if (tf_n < 2 || (size_t)tf_n > kTfMax)
     return fail(c, AMR_ERR_ARG, "tf_n must be in [2, 2048] (the no-alloc staging limit)");
