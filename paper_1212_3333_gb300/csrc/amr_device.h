@@ -190,7 +190,8 @@ struct RenderArgs {
   int32_t shadow;                // secondary rays to the point light
   float light_f[3];              // light position, finest-cell units
   float light_step, light_ambient;
-  int32_t samples_per_iter;      // refill schedule: samples per lane between warp steps
+  int32_t samples_per_iter;      // schedules 2 and 3: samples per lane between warp steps (in
+                                 // [1, 64]); unchecked, and not to be read, in the others
   int32_t coarse_factor;         // learned mode 2: step multiplier below tau
   int32_t learned_min_samples;   // learned modes: segments shorter than this skip the MLP
   long long mdelta;              // stencil-maximum brick = value brick + mdelta bytes (ptr)

@@ -322,8 +322,8 @@ static bool textures(const amr_ctx* c) {
 // schedule otherwise.  Every schedule gives the same image bit for bit (with secondary rays to
 // rounding), so the choice affects time only.  Single images of kLargePixels pixels and more
 // stay on the per-ray schedule where deferred shading has no workspace - texture storages, calls
-// that may not allocate - and loses (textures, 1900 x 1800: 31.8 against 37 ms), and when samples_per_iter, which only
-// deferred shading reads, is outside its range.
+// that may not allocate - and loses (textures, 1900 x 1800: 31.8 against 37 ms), and when
+// samples_per_iter, which no kernel of schedules 0 and 1 reads, is outside its range.
 
 static const amr_render_params* resolve_schedule(const amr_render_params* p, int64_t pixels,
                                                  bool one_kernel, amr_render_params* tmp) {

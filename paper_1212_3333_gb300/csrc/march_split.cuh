@@ -87,6 +87,11 @@ __device__ __forceinline__ unsigned own_tasks(unsigned* own, int lane, unsigned 
 #ifndef AMR_SPLIT_VALUES
 #define AMR_SPLIT_VALUES 4
 #endif
+// Samples a lane takes between fetches: shaded, the caller's samples_per_iter, which the host
+// has checked to lie in [1, 64]; unshaded (schedule 0, where that field has no meaning and any
+// value) a constant.  At least one group either way, so that every pass makes progress.
+constexpr int kPlainStep = 16;
+static_assert(kPlainStep >= AMR_SPLIT_GROUP, "a pass takes samples");
 
 // A warp's part of the workspace while it marches: its block of segment records.
 struct SegBlock {
@@ -312,9 +317,10 @@ __device__ __forceinline__ int march_tile(const RenderArgs& A, const RayArgs& R,
     // A lane takes its next G samples at a time: a mask of those that may be opaque (by
     // their stencil maxima, or by their values), queued in order.  Most masks are empty.
     constexpr int G = MX ? AMR_SPLIT_GROUP : AMR_SPLIT_VALUES;
-    for (int step = 0; step < A.samples_per_iter; step += G) {
+    const int steps = SHADED ? A.samples_per_iter : kPlainStep;
+    for (int step = 0; step < steps; step += G) {
       const int kb = k;
-      const int cnt = live ? min(min(G, A.samples_per_iter - step), g.s.n - k) : 0;
+      const int cnt = live ? min(min(G, steps - step), g.s.n - k) : 0;
       unsigned mask = 0;
       float val[MX ? 1 : G];
       if (cnt > 0) {

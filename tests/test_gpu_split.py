@@ -75,6 +75,24 @@ def test_segment_bound_is_reported_for_the_same_rays(amr):
     assert seen == {True, False}
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("schedule", [0, -1])
+def test_unshaded_frames_do_not_read_samples_per_iter(amr, dtype, schedule):
+    """Schedule 0 takes any value of the field (it belongs to schedules 2 and 3)."""
+    h = random_hierarchy(3, n0=12, num_levels=3, patches_per_level=6)
+    ctx = amr.from_hierarchy(h, dtype)
+    ctx.amr_build_kdtree("ptr", halo=2, maxbrick=True)
+    vmin, vmax = h.value_range()
+    cam = synth.orbit_camera(2, 70, 53)
+    want = None
+    for spi in (16, 0, -1, 1, 65, 2 ** 31 - 1, -2 ** 31):
+        p, _ = params_pair(amr, vmin, vmax, schedule=schedule, shade=0, step_factor=0.1,
+                           samples_per_iter=spi)
+        got = gpu_render(ctx, cam, _opaque_tf(), p)
+        want = want or got
+        assert got[1] == want[1] > 0 and np.array_equal(got[0], want[0]), spi
+
+
 def test_first_call_captured(amr):
     import torch
 
