@@ -164,9 +164,10 @@ struct RenderArgs {
   const DLeaf* leaves;
   const int32_t* face_node;    // per leaf, 12: per face (2a + side) the node slot holding the
                                // leaf and the cell beyond the face, then the cell alone
-                               // (starts of neighbour lookups; the second half: ropes);
-                               // an entry with kFaceLeaf set names a leaf id instead, one
-                               // with kFaceList (second half) a list of the leaves beyond
+                               // (starts of neighbour lookups).  After those of all leaves,
+                               // per leaf, 6: the latter again as ropes.  An entry with
+                               // kFaceLeaf set names a leaf id instead, a rope with kFaceList
+                               // a list of the leaves beyond
   const int4* node_box;        // per node slot, 2: box lo (x, y, z, highest label level of
                                // a type-(a) node above it or -1), hi (x, y, z, 0), finest
                                // cells (rope restarts)

@@ -490,12 +490,15 @@ amr_status upload(amr_ctx* c, void* stream_v) {
   if (fault_injected("corrupt_node") && nodes.size() > 1 &&
       (nodes[0].meta >> 30) != (uint32_t)kLeafAxis)
     nodes[0].meta &= ~kIndexMask;  // the root's children become slots 0 (itself) and 1
-  std::vector<int32_t> face_slots(std::max<size_t>(1, t.face_node.size()), 0);
+  std::vector<int32_t> face_slots(std::max<size_t>(1, 18 * M), 0);
   for (size_t k = 0; k < t.face_node.size(); ++k) {
     const int32_t pre = t.face_node[k];
     face_slots[k] = t.axis[pre] < 0 ? (int32_t)(kFaceLeaf | (uint32_t)t.leaf[pre]) : slot_of[pre];
   }
-  // leaf lists for the faces whose node is an inner one: per leaf, then one after the other
+  // the ropes: the nodes holding the cells beyond the faces alone, again
+  for (size_t m = 0; m < M; ++m)
+    std::copy_n(&face_slots[12 * m + 6], 6, &face_slots[12 * M + 6 * m]);
+  // leaf lists for the ropes whose node is an inner one: per leaf, then one after the other
   std::vector<std::vector<int4>> leaf_lists(M);
   std::vector<int32_t> list_word(6 * M, -1);
   bool no_memory = false;  // (an exception may not leave the parallel loop)
@@ -521,7 +524,7 @@ amr_status upload(amr_ctx* c, void* stream_v) {
     face_lists.insert(face_lists.end(), leaf_lists[m].begin(), leaf_lists[m].end());
     for (int f = 0; f < 6; ++f)
       if (list_word[6 * m + f] >= 0)
-        face_slots[12 * m + 6 + f] = (int32_t)(kFaceList | (uint32_t)(base + list_word[6 * m + f]));
+        face_slots[12 * M + 6 * m + f] = (int32_t)(kFaceList | (uint32_t)(base + list_word[6 * m + f]));
   }
   face_lists.resize(face_lists.size() + kFaceListMax / 2, int4{0, 0, 0, 0});
   const size_t ML = t.lod_patch.size();

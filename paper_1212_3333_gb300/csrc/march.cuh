@@ -362,13 +362,17 @@ __device__ __forceinline__ int descend(const DNode* __restrict__ nodes, const Ra
 }
 
 // The leaf of a face list whose rectangle holds the point (u, v) on the face (finest cells on
-// its two axes, relative to (base_u, base_v)), -1 for none; slot: the node the list replaces.
-// The caller checks the leaf's box.  The list's words are loaded together, where a descent
-// from the node (31 % of the segments had one, 3.2 steps on average, the warp's longest
-// deciding) waits for one load a step.  Measured, descents / lists, ms: 640 x 479 2.76 / 2.45,
-// 1024^2 7.43 / 6.99, f16 unshaded 1917 x 1083 4.85 / 4.38, 32-view batch 27.9 / 25.1.
+// its two axes), -1 for none; slot: the node the list replaces.  The caller checks the leaf's
+// box.  The list's words are loaded together, where a descent from the node (31 % of the
+// segments had one, 3.2 steps on average, the warp's longest deciding) waits for one load a
+// step.  Measured when the lists came in, descents / lists, ms: 640 x 479 2.76 / 2.45, 1024^2
+// 7.43 / 6.99, f16 unshaded 1917 x 1083 4.85 / 4.38, 32-view batch 27.9 / 25.1.
+// For ropes only: the neighbour lookups of gradients start from the node.  With lists there too,
+// the one-kernel marches lost 8 to 25 % of dense frames (one-kernel deferred march, a fifth of
+// the cells opaque, with / without, ms: 4 levels 1024^2 7.12 / 5.82, 2048^2 22.7 / 18.4; 5 levels
+// 2048^2 55.0 / 48.1) and the split march gained nothing (8 levels 1500 x 1100 8.23 / 8.11).
 __device__ __forceinline__ int face_list_leaf(const int4* __restrict__ lists, uint32_t ent, float u,
-                                              float v, int base_u, int base_v, uint32_t& slot) {
+                                              float v, uint32_t& slot) {
   const int4* w = lists + (ent & (kFaceList - 1u));
   const int4 h = __ldg(w);
   int4 q[3];
@@ -377,8 +381,8 @@ __device__ __forceinline__ int face_list_leaf(const int4* __restrict__ lists, ui
   slot = (uint32_t)h.z;
   const int n = h.w & 31;
   const float inv = __int_as_float((127 - (h.w >> 5)) << 23);  // 1 / unit
-  const unsigned iu = (unsigned)(int)floorf((u + (float)(base_u - h.x)) * inv);
-  const unsigned iv = (unsigned)(int)floorf((v + (float)(base_v - h.y)) * inv);
+  const unsigned iu = (unsigned)(int)floorf((u - (float)h.x) * inv);
+  const unsigned iv = (unsigned)(int)floorf((v - (float)h.y) * inv);
   int leaf = -1;
   auto test = [&](int rect, int id, int k) {
     const unsigned r = (unsigned)rect;
@@ -423,13 +427,13 @@ __device__ __forceinline__ int rope_start(const int32_t* __restrict__ face_node,
                                           float& e1, int lod_min) {
   const int a = pid0 & 3;
   const bool up = sel3f(a, rf.B[0], rf.B[1], rf.B[2]) > 0.0f;
-  uint32_t ent = (uint32_t)__ldg(face_node + 12 * prev + 6 + 2 * a + (up ? 1 : 0));
+  uint32_t ent = (uint32_t)__ldg(face_node + 12 * R.n_leaves + 6 * prev + 2 * a + (up ? 1 : 0));
   if ((ent & (kFaceLeaf | kFaceList)) == kFaceList) {
     // several leaves beyond the face: the one the ray enters, to be checked like any other
     const float x0 = fmaf(tau0, rf.Dd[0], rf.Xe[0]), x1 = fmaf(tau0, rf.Dd[1], rf.Xe[1]),
                 x2 = fmaf(tau0, rf.Dd[2], rf.Xe[2]);
     uint32_t slot;
-    const int id = face_list_leaf(R.face_list, ent, a == 0 ? x1 : x0, a == 2 ? x1 : x2, 0, 0, slot);
+    const int id = face_list_leaf(R.face_list, ent, a == 0 ? x1 : x0, a == 2 ? x1 : x2, slot);
     ent = id >= 0 ? kFaceLeaf | (uint32_t)id : slot;
   }
   int blo[3], bhi[3], anc;
@@ -849,25 +853,9 @@ __device__ __forceinline__ float neighbour_slow(const RenderArgs& A, const RayAr
   // from a pruned leaf (the table covers the unpruned leaves)
   uint32_t i = 0;
   if (leaf < R.n_leaves) {
-    uint32_t ent =
+    const uint32_t ent =
         (uint32_t)__ldg(A.face_node + 12 * leaf + (beyond ? 6 : 0) + 2 * a + (sign > 0.0f ? 1 : 0));
     bool ok = true;
-    if ((ent & (kFaceLeaf | kFaceList)) == kFaceList) {
-      // several leaves beyond the face: the one whose box holds the point beyond the margin,
-      // which no descent could miss then; else from the node they replace
-      uint32_t slot;
-      const int id = face_list_leaf(R.face_list, ent, a == 0 ? x1 : x0, a == 2 ? x1 : x2,
-                                    a == 0 ? lo1 : lo0, a == 2 ? lo1 : lo2, slot);
-      ent = slot;
-      if (id >= 0) {
-        const int4* w = reinterpret_cast<const int4*>(A.leaves + id);
-        const int4 w1 = __ldg(w + 1), w2 = __ldg(w + 2);  // lo[3], hi[0] | hi[1], hi[2], ...
-        const bool holds = x0 - (float)(w1.x - lo0) > mf && (float)(w1.w - lo0) - x0 > mf &&
-                           x1 - (float)(w1.y - lo1) > mf && (float)(w2.x - lo1) - x1 > mf &&
-                           x2 - (float)(w1.z - lo2) > mf && (float)(w2.y - lo2) - x2 > mf;
-        if (holds) ent = kFaceLeaf | (uint32_t)id;
-      }
-    }
     if (pruning) {
       const int anc = (ent & kFaceLeaf) ? __ldg(&A.leaves[ent & ~kFaceLeaf].lod_anc)
                                         : __ldg(&A.node_box[2 * ent].w);
