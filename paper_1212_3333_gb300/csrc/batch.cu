@@ -133,11 +133,8 @@ amr_status launch_shape(amr_ctx* c, const BatchArgs& b, int blocks_per_sm, cudaS
   constexpr int kThreads = TW * TH;
   size_t smem = (size_t)b.n_tf * (b.A.tf_n + 1) * sizeof(int);
   if (DEFER) smem = ((smem + 15) & ~(size_t)15) + (kThreads / 32) * sizeof(DeferArea);
-  cudaError_t e = cudaSuccess;
-  if (smem > 48 * 1024)
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int dev = 0, sms = 0, occ = 0;
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = fit_carveout(k, smem, kThreads, occ);
   if (e != cudaSuccess) return fail(c, AMR_ERR_CUDA, std::string("batch launch setup: ") + cudaGetErrorString(e));

@@ -12,15 +12,27 @@
 
 namespace amr {
 
-// Shared-memory carveout: the smallest split that still holds as many blocks per SM as the
-// registers allow, so that the rest of the SM's 256 KB serves as L1 cache for the bricks
-// (measured on C2, Phong, per-ray loop at 2048^2 / deferred at 1024^2, Gsamples/s: driver's
-// choice 81.1 / 46.4, this split 81.8 / 47.7; more L1 matters - the per-ray loop with 28 KB
-// of unused shared memory per block ran at 77.6).  Returns the resident blocks per SM.
+// A block may use 48 KB of shared memory, its static arrays (`fixed`) included, unless the
+// kernel's dynamic part is allowed to be larger.
+template <typename K>
+cudaError_t allow_smem(K kernel, size_t smem, size_t fixed) {
+  if (smem + fixed <= 48 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+
+// Allows the launch its shared memory and fits the carveout: the smallest split that still
+// holds as many blocks per SM as the registers allow, so that the rest of the SM's 256 KB serves
+// as L1 cache for the bricks (measured on C2, Phong, per-ray loop at 2048^2 / deferred at 1024^2,
+// Gsamples/s: driver's choice 81.1 / 46.4, this split 81.8 / 47.7; more L1 matters - the per-ray
+// loop with 28 KB of unused shared memory per block ran at 77.6).  Returns the resident blocks
+// per SM.
 template <typename K>
 cudaError_t fit_carveout(K kernel, size_t smem, int threads, int& occ) {
   int dev = 0, max_smem = 0, reserved = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e == cudaSuccess) e = allow_smem(kernel, smem, fa.sharedSizeBytes);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess)
     e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   if (e == cudaSuccess)
@@ -29,8 +41,6 @@ cudaError_t fit_carveout(K kernel, size_t smem, int threads, int& occ) {
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, smem);
-  cudaFuncAttributes fa;
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
   if (e != cudaSuccess || occ <= 0 || max_smem <= 0) return e;
   // a block's shared memory: the dynamic part, the kernel's static arrays, the reserve
   const long long need = (long long)occ * ((long long)smem + (long long)fa.sharedSizeBytes + reserved);
@@ -41,16 +51,9 @@ cudaError_t fit_carveout(K kernel, size_t smem, int threads, int& occ) {
 template <typename K>
 cudaError_t launch_one(K kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                        const RenderArgs& a) {
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  {
-    int occ = 0;
-    cudaError_t e = fit_carveout(kernel, smem, (int)(block.x * block.y * block.z), occ);
-    if (e != cudaSuccess) return e;
-  }
+  int occ = 0;
+  const cudaError_t e = fit_carveout(kernel, smem, (int)(block.x * block.y * block.z), occ);
+  if (e != cudaSuccess) return e;
   kernel<<<grid, block, smem, s>>>(a);
   return cudaGetLastError();
 }
@@ -60,8 +63,9 @@ cudaError_t launch_one(K kernel, dim3 grid, dim3 block, size_t smem, cudaStream_
 template <typename K>
 cudaError_t launch_persist(K kernel, size_t smem, cudaStream_t s, const RenderArgs& a) {
   cudaError_t e = cudaMemsetAsync(a.counters + kQueueCounter, 0, sizeof(unsigned long long), s);
-  if (e == cudaSuccess && smem > 48 * 1024)
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncAttributes fa;
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+  if (e == cudaSuccess) e = allow_smem(kernel, smem, fa.sharedSizeBytes);
   int dev = 0, sms = 0, occ = 0;
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -84,11 +88,8 @@ inline const RenderArgs& args_of(const BatchArgs& b) { return b.A; }
 // of them per tile, and at least a warp per tile while they last.
 template <typename K, typename Args>
 cudaError_t launch_stride(K kernel, size_t smem, cudaStream_t s, const Args& a, int per_tile) {
-  cudaError_t e = cudaSuccess;
-  if (smem > 48 * 1024)
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int dev = 0, sms = 0, occ = 0;
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = fit_carveout(kernel, smem, 128, occ);
   if (e != cudaSuccess) return e;

@@ -93,6 +93,23 @@ def test_unshaded_frames_do_not_read_samples_per_iter(amr, dtype, schedule):
         assert got[1] == want[1] > 0 and np.array_equal(got[0], want[0]), spi
 
 
+# the largest transfer functions whose shared memory, with the march kernels' static arrays,
+# fits the default 48 KB, the first beyond it, those around 48 KB of their own, the longest
+@pytest.mark.parametrize("shade", [0, 1])
+@pytest.mark.parametrize("n", [1330, 1356, 1358, 1400, 1900, 1946, 2048])
+def test_long_transfer_functions(amr, n, shade):
+    ctx, (vmin, vmax) = _context(amr)
+    plain, _ = _context(amr, maxbrick=False)
+    cam = synth.orbit_camera(2, 40, 27)
+    p, _ = params_pair(amr, vmin, vmax, schedule=0, shade=shade, step_factor=0.2)
+    want = gpu_render(plain, cam, _opaque_tf(n, n // 4), p)
+    for c in (ctx, plain):
+        for schedule in (-1, 0, 2) + ((3,) if shade else ()):
+            p.schedule = schedule
+            got = gpu_render(c, cam, _opaque_tf(n, n // 4), p)
+            assert got[1] == want[1] > 0 and np.array_equal(got[0], want[0]), schedule
+
+
 def test_first_call_captured(amr):
     import torch
 
