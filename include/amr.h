@@ -19,7 +19,8 @@
  *   - Fault injection for tests (host side only): the environment variable AMR_FAULT =
  *     bad_alloc makes the host build fail with AMR_ERR_OOM, oom the device upload's first
  *     allocation (AMR_ERR_OOM), corrupt_node uploads a root node that names itself as a
- *     child (indices stay in range; renders report AMR_ERR_DEVICE).  Unset: no effect.
+ *     child (indices stay in range; renders report AMR_ERR_DEVICE), shade_launch leaves out
+ *     a launch of deferred shading and reports AMR_ERR_CUDA.  Unset: no effect.
  *   - Level l has spacing h^l = h^0 / r^l per axis (Sec. 2).  Patch boxes are int64[6]
  *     {lo_x, lo_y, lo_z, hi_x, hi_y, hi_z}, half-open, in level-l cell indices.  Level 0
  *     must tile its bounding box (the kD root, Sec. 3.1); same-level patches must be

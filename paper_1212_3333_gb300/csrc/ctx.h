@@ -20,6 +20,8 @@ namespace amr {
 //   oom           the device upload's first allocation fails   -> AMR_ERR_OOM
 //   corrupt_node  the uploaded root node names itself as a child (every index stays in
 //                 range), so descents loop until their depth bound -> AMR_ERR_DEVICE
+//   shade_launch  the split march's shading kernel is not launched and its launch reports an
+//                 error                                      -> AMR_ERR_CUDA
 // Unset or any other value: no effect.
 inline bool fault_injected(const char* what) {
   const char* v = std::getenv("AMR_FAULT");

@@ -120,6 +120,7 @@ cudaError_t launch_rounds(int rounds, cudaStream_t s, const Args& b) {
     if (r > 0) e = cudaMemsetAsync(ts.heads, 0, kRoundHeads * sizeof(unsigned), s);
     if (e == cudaSuccess)
       e = launch_stride(split_march_kernel<ST, SHADE, Args>, base + 4 * sizeof(CandArea<true>), s, b, 1);
+    if (e == cudaSuccess && fault_injected("shade_launch")) e = cudaErrorLaunchFailure;
     if (e == cudaSuccess) e = launch_stride(split_shade_kernel<ST, SHADE, Args>, base, s, b, 4);
     if (e == cudaSuccess) e = launch_stride(split_outer_kernel<ST, SHADE, Args>, base, s, b, 4);
     if (e == cudaSuccess) e = launch_stride(split_sum_kernel<Args>, 0, s, b, 4);
@@ -127,7 +128,8 @@ cudaError_t launch_rounds(int rounds, cudaStream_t s, const Args& b) {
   // an image whose tiles are all dense (every sample opaque, ms: 1024^2 46 deferred, 49 per ray
   // before; 2048^2 146 deferred, 119 per ray)
   if constexpr (std::is_same<Args, RenderArgs>::value && (SHADE & kShadeShadow) == 0)
-    if (tiles_of(b) * 32 >= kLargePixels) e = launch_tiles(march_kernel<ST, 1, SHADE>, base, s, b);
+    if (e == cudaSuccess && tiles_of(b) * 32 >= kLargePixels)
+      e = launch_tiles(march_kernel<ST, 1, SHADE>, base, s, b);
   if (e != cudaSuccess) return e;
   return launch_tiles(deferred_kernel<ST, SHADE, Args>, base + 4 * sizeof(DeferArea), s, b);
 }

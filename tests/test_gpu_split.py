@@ -110,6 +110,26 @@ def test_long_transfer_functions(amr, n, shade):
             assert got[1] == want[1] > 0 and np.array_equal(got[0], want[0]), schedule
 
 
+def test_large_images_and_a_failing_launch(amr, monkeypatch):
+    """Images of 3,000,000 pixels and more leave what the split march does not take to the
+    per-ray loop; a launch that fails before that is still reported."""
+    from paper_1212_3333_gb300 import _lib
+
+    ctx, (vmin, vmax) = _context(amr)
+    cam = synth.orbit_camera(4, 2003, 1501)
+    for clear in (16, 0):
+        p, _ = params_pair(amr, vmin, vmax, schedule=0, shade=1)
+        want = gpu_render(ctx, cam, _opaque_tf(clear=clear), p)
+        p.schedule = 3
+        monkeypatch.setenv("AMR_FAULT", "shade_launch")
+        with pytest.raises(amr.AmrError) as e:
+            gpu_render(ctx, cam, _opaque_tf(clear=clear), p)
+        assert e.value.status == _lib.AMR_ERR_CUDA
+        monkeypatch.delenv("AMR_FAULT")
+        got = gpu_render(ctx, cam, _opaque_tf(clear=clear), p)
+        assert got[1] == want[1] and np.array_equal(got[0], want[0])
+
+
 def test_first_call_captured(amr):
     import torch
 
