@@ -212,8 +212,9 @@ amr_status amr_build_host(amr_ctx* ctx, amr_storage storage);
  * call of a size that is not being captured allocates it (1.7 GB for most images, 3.5 GB at
  * most; without it the call renders the same image with the one-kernel march), a larger one
  * is added when a larger image needs it, and amr_destroy or another build frees them, so a
- * captured call stays valid until then.  Calls on several streams take turns on it; a graph's
- * replay must not overlap other work of the context.
+ * captured call stays valid until then.  Renders, batches and traces of one context take turns
+ * on the GPU, on whatever streams they are issued; a graph's replay must not overlap other work
+ * of the context, nor may segment logging on another stream.
  * 16-bit cells render trilinear with the per-ray schedule (else AMR_ERR_ARG). */
 amr_status amr_render(amr_ctx* ctx, const amr_camera* cam, const float* tf_rgba_dev,
                       int32_t tf_n, const amr_render_params* params, float* out_rgba_dev,

@@ -188,7 +188,6 @@ amr_status launch_batch(amr_ctx* c, const BatchArgs& b, int storage, int shade, 
         else e = mx ? launch_rounds<ST_PTR, 2 | kShadeMaxBit>(rounds, s, *t)
                     : launch_rounds<ST_PTR, 2>(rounds, s, *t);
       }
-      if (e == cudaSuccess) e = tasks_queued(c, stream);
       if (e != cudaSuccess)
         return fail(c, AMR_ERR_CUDA, std::string("batch launch: ") + cudaGetErrorString(e));
       return AMR_OK;

@@ -504,6 +504,8 @@ amr_status amr_render(amr_ctx* c, const amr_camera* cam, const float* tf_rgba_de
   a.tf = reinterpret_cast<const float4*>(tf_rgba_dev);
   a.out = reinterpret_cast<float4*>(out_rgba_dev);
   cudaStream_t st = (cudaStream_t)cuda_stream;
+  const WorkOrder order(c->dev, st);
+  CK(order.error);
   CK(cudaMemsetAsync(c->dev.counters, 0, kNumCounters * sizeof(unsigned long long), st));
   s = launch_render_args(c, a, params, cuda_stream);
   if (s != AMR_OK) return s;
@@ -536,6 +538,8 @@ amr_status amr_render_host(amr_ctx* c, const amr_camera* cam, const float* tf_rg
     CK(cudaMalloc(&d.img_scratch, img_bytes));
     d.img_scratch_bytes = img_bytes;
   }
+  const WorkOrder order(d, st);
+  CK(order.error);
   CK(cudaMemcpyAsync(d.tf_scratch, tf_rgba_host, (size_t)tf_n * sizeof(float4),
                      cudaMemcpyHostToDevice, st));
   a.tf = d.tf_scratch;
@@ -650,6 +654,8 @@ amr_status amr_render_batch(amr_ctx* c, const amr_view* views, int32_t n_views,
                                out_floats, cfg, b.get());
   if (s != AMR_OK) return s;
   cudaStream_t st = (cudaStream_t)cuda_stream;
+  const WorkOrder order(c->dev, st);
+  CK(order.error);
   CK(cudaMemsetAsync(c->dev.counters, 0, kNumCounters * sizeof(unsigned long long), st));
   s = launch_batch(c, *b, kernel_storage(c), kernel_shade(c, params), params->schedule, cfg,
                    cuda_stream);
@@ -679,6 +685,9 @@ amr_status amr_batch_autotune(amr_ctx* c, const amr_view* views, int32_t n_views
     cudaEventDestroy(e1);
     return r;
   };
+  const WorkOrder order(c->dev, st);
+  if (order.error != cudaSuccess)
+    return done(fail(c, AMR_ERR_CUDA, std::string("stream order: ") + cudaGetErrorString(order.error)));
   float best_ms = -1.0f;
   amr_batch_config best = c->batch_cfg;
   // candidates 0..8: tile shape x rays per thread; 9..12: the best of those with 4, 8, 16
@@ -906,6 +915,8 @@ amr_status amr_trace(amr_ctx* c, const amr_camera* cam, double lod_pixels, int32
   a.counters = c->dev.counters;
   a.ray.counters = c->dev.counters;
   cudaStream_t st = (cudaStream_t)cuda_stream;
+  const WorkOrder order(c->dev, st);
+  CK(order.error);
   CK(cudaMemsetAsync(c->dev.counters, 0, kNumCounters * sizeof(unsigned long long), st));
   s = launch_trace(c, a, cuda_stream);
   if (s != AMR_OK) return s;

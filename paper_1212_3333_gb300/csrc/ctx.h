@@ -96,11 +96,37 @@ struct DeviceState {
   // earlier ones stay for CUDA graphs that hold their addresses (sizes at least double)
   std::vector<void*> task_spaces;
   TaskSpace tasks = {};
-  cudaEvent_t task_event = nullptr;  // after the last call that used a workspace,
-  cudaStream_t task_stream = nullptr;  // on this stream
+  cudaEvent_t work_event = nullptr;  // after the last call's work (WorkOrder)
   float dense_below = -INFINITY;     // a fifth of the cells lie below this value
   int64_t task_pixels = 0;
   int64_t task_refused = INT64_MAX;  // a workspace for this many pixels could not be allocated
+};
+
+// Calls on a context share its counters and workspaces, so each one's work waits for the last
+// one's, whatever their streams (stream handles do not tell: a destroyed stream's handle may be
+// given to a new one while its work is still under way, and cudaStreamPerThread is another
+// stream in every thread).  Made before a call queues anything; the destructor marks where the
+// call's work ends, also on an error return.  Captured calls neither wait nor are waited for: a
+// replay must not overlap other work of the context.
+class WorkOrder {
+ public:
+  WorkOrder(DeviceState& d, cudaStream_t stream) : d_(d), stream_(stream) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    error = cudaStreamIsCapturing(stream, &cap);
+    captured_ = cap != cudaStreamCaptureStatusNone;
+    if (error == cudaSuccess && !captured_) error = cudaStreamWaitEvent(stream, d.work_event, 0);
+  }
+  ~WorkOrder() {
+    if (error == cudaSuccess && !captured_) cudaEventRecord(d_.work_event, stream_);
+  }
+  WorkOrder(const WorkOrder&) = delete;
+  WorkOrder& operator=(const WorkOrder&) = delete;
+  cudaError_t error;
+
+ private:
+  DeviceState& d_;
+  cudaStream_t stream_;
+  bool captured_ = false;
 };
 
 // The workspace of a call: the tiles it has records for (0: none), and the rounds for some.
@@ -155,11 +181,8 @@ amr_status upload(amr_ctx* c, void* stream);
 void release_device(amr_ctx* c);
 // The split march's workspace for a call with that many 8x4 tiles, grown when it is too small
 // and the stream is not being captured; it may have fewer tiles (out of memory, or a first
-// call captured: none).  A call on another stream waits for the workspace's last one;
-// tasks_queued marks where a call ends.  (Captured calls neither wait nor are waited for: as
-// before, a replay must not overlap other work of the context.)
+// call captured: none).  The caller holds a WorkOrder.
 TaskPlan plan_tasks(amr_ctx* c, long long tiles, void* stream);
-cudaError_t tasks_queued(amr_ctx* c, void* stream);
 // kernels (march.cu)
 amr_status launch_render(amr_ctx* c, const RenderArgs& a, int storage, int interp, int shade,
                          int schedule, void* stream);

@@ -292,12 +292,6 @@ TaskPlan plan_tasks(amr_ctx* c, long long call_tiles, void* stream) {
   const int64_t want = std::min<int64_t>(call_tiles * 32, std::max<int64_t>(kBandPixels, 32 * 8192));
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing((cudaStream_t)stream, &cap) != cudaSuccess) cudaGetLastError();
-  if (cap == cudaStreamCaptureStatusNone && !d.task_event &&
-      cudaEventCreateWithFlags(&d.task_event, cudaEventDisableTiming) != cudaSuccess) {
-    cudaGetLastError();
-    d.task_event = nullptr;
-    return plan;
-  }
   if (want > d.task_pixels && want < d.task_refused) {
     const int64_t px = std::max(want, std::min(2 * d.task_pixels, kBandPixels));
     const int64_t tiles = px / 32;
@@ -347,23 +341,9 @@ TaskPlan plan_tasks(amr_ctx* c, long long call_tiles, void* stream) {
     }
   }
   if (d.task_pixels == 0) return plan;
-  if (cap == cudaStreamCaptureStatusNone && d.task_stream != (cudaStream_t)stream &&
-      cudaStreamWaitEvent((cudaStream_t)stream, d.task_event, 0) != cudaSuccess) {
-    cudaGetLastError();
-    return plan;
-  }
   plan.ts = d.tasks;
   plan.tiles = d.task_pixels / 32;
   return plan;
-}
-
-cudaError_t tasks_queued(amr_ctx* c, void* stream) {
-  DeviceState& d = c->dev;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  cudaError_t e = cudaStreamIsCapturing((cudaStream_t)stream, &cap);
-  if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) return e;
-  d.task_stream = (cudaStream_t)stream;
-  return cudaEventRecord(d.task_event, (cudaStream_t)stream);
 }
 
 void release_device(amr_ctx* c) {
@@ -399,7 +379,7 @@ void release_device(amr_ctx* c) {
   cudaFree(d.log_counts);
   cudaFree(d.log_offsets);
   for (void* p : d.task_spaces) cudaFree(p);
-  if (d.task_event) cudaEventDestroy(d.task_event);
+  if (d.work_event) cudaEventDestroy(d.work_event);
   d = DeviceState();
   c->device_built = false;
 }
@@ -478,6 +458,7 @@ amr_status upload(amr_ctx* c, void* stream_v) {
   DeviceState& d = c->dev;
   d.dense_below = low_quantile(c);
   CK(cudaGetDevice(&d.device));
+  if (!d.work_event) CK(cudaEventCreateWithFlags(&d.work_event, cudaEventDisableTiming));
   const Tree& t = c->tree;
   const size_t P = c->patches.size();
   const size_t M = t.leaf_patch.size();
@@ -647,6 +628,7 @@ amr_status upload(amr_ctx* c, void* stream_v) {
                        stream));
   CK(cudaMemcpyAsync(d.patches, pt.data(), P * sizeof(DPatch), cudaMemcpyHostToDevice, stream));
   CK(cudaStreamSynchronize(stream));
+  CK(cudaEventRecord(d.work_event, stream));
   c->device_built = true;
   return AMR_OK;
 }

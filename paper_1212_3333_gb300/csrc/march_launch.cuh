@@ -267,7 +267,6 @@ amr_status launch_storage(amr_ctx* c, const RenderArgs& a, int interp, int shade
     else e = launch_one(wave_kernel<ST, 0, 1>, grid, block, smem, s, a);
   }
 launched:
-  if (e == cudaSuccess && plan.tiles > 0) e = tasks_queued(c, s);
   if (e != cudaSuccess)
     return fail(c, AMR_ERR_CUDA, std::string("march launch: ") + cudaGetErrorString(e));
   return AMR_OK;

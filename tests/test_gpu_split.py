@@ -156,25 +156,52 @@ def test_first_call_captured(amr):
 
 
 def test_calls_on_two_streams_take_turns(amr):
-    """The streams share the context's workspace: the second call waits for the first."""
+    """The streams share the context's workspace and counters: the second call waits for the
+    first, so images and sample counts are those of calls made one at a time."""
     import torch
 
     ctx, (vmin, vmax) = _context(amr)
-    cams = [synth.orbit_camera(s, 180, 150) for s in (1, 2)]
+    cams = [synth.orbit_camera(s, 180, 150) for s in (1, 2, 3)]
+    tf = torch.as_tensor(_opaque_tf(), device="cuda")
+    ps = [params_pair(amr, vmin, vmax, schedule=schedule, shade=shade, step_factor=0.05, kappa=0.2)[0]
+          for schedule, shade in ((3, 1), (3, 1), (0, 0))]
+    want = []
+    for cam, p in zip(cams, ps):
+        out = torch.zeros((150, 180, 4), device="cuda")
+        want.append((out, ctx.amr_render(cam, tf, p, out, count_samples=True)))
+    streams = [torch.cuda.Stream() for _ in cams]
+    got = [torch.zeros_like(w) for w, _ in want]
+    torch.cuda.synchronize()
+    for counted in (0, 1, 2, None):
+        for k in range(6):
+            i = (k + (counted or 0)) % 3
+            n = ctx.amr_render(cams[i], tf, ps[i], got[i], stream=streams[i],
+                               count_samples=i == counted)
+            assert n is None or n == want[i][1]
+    torch.cuda.synchronize()
+    for g, (w, _) in zip(got, want):
+        assert torch.equal(g, w)
+
+
+def test_calls_on_streams_that_are_destroyed_take_turns(amr):
+    """A new stream may get a destroyed one's handle while its work is still under way."""
+    import ctypes
+
+    import torch
+
+    ctx, (vmin, vmax) = _context(amr)
+    rt = torch.cuda.cudart()
+    cam = synth.orbit_camera(1, 300, 250)
     tf = torch.as_tensor(_opaque_tf(), device="cuda")
     p, _ = params_pair(amr, vmin, vmax, schedule=3, shade=1, step_factor=0.05, kappa=0.2)
-    want = []
-    for cam in cams:
-        out = torch.zeros((150, 180, 4), device="cuda")
-        ctx.amr_render(cam, tf, p, out)
-        torch.cuda.synchronize()
-        want.append(out)
-    streams = [torch.cuda.Stream() for _ in cams]
-    got = [torch.zeros_like(w) for w in want]
+    outs = [torch.zeros((250, 300, 4), device="cuda") for _ in range(12)]
+    ctx.amr_render(cam, tf, p, outs[0])
     torch.cuda.synchronize()
-    for _ in range(3):
-        for cam, st, out in zip(cams, streams, got):
-            ctx.amr_render(cam, tf, p, out, stream=st)
+    for out in outs[1:]:
+        h = ctypes.c_void_p()
+        assert int(rt.cudaStreamCreate(ctypes.addressof(h))) == 0
+        ctx.amr_render(cam, tf, p, out, stream=h.value)
+        assert int(rt.cudaStreamDestroy(h.value)) == 0
     torch.cuda.synchronize()
-    for g, w in zip(got, want):
-        assert torch.equal(g, w)
+    for out in outs[1:]:
+        assert torch.equal(out, outs[0])
