@@ -209,12 +209,13 @@ amr_status amr_build_host(amr_ctx* ctx, amr_storage storage);
  * the call synchronises the stream, checks the device status word and stores the exact
  * number of samples taken (sum over segments of the per-segment sample count).
  * Deferred shading (schedule 3, linear storages) keeps a workspace with the context: the first
- * call of a size that is not being captured allocates it (1.7 GB for most images, 3.5 GB at
- * most; without it the call renders the same image with the one-kernel march), a larger one
- * is added when a larger image needs it, and amr_destroy or another build frees them, so a
- * captured call stays valid until then.  Renders, batches and traces of one context take turns
- * on the GPU, on whatever streams they are issued; a graph's replay must not overlap other work
- * of the context, nor may segment logging on another stream.
+ * call that is not being captured allocates it (1.7 GB for most images, 3.5 GB at most; without
+ * it the call renders the same image with the one-kernel march), and a larger image replaces it
+ * by a larger one.  A workspace that captured calls use stays valid, beside its replacement,
+ * until amr_destroy or another build, which free them all (at most 10.5 GB, when graphs were
+ * captured at every size).  Renders, batches and traces of one context take turns on the GPU, on
+ * whatever streams they are issued; a graph's replay must not overlap other work of the context,
+ * nor may segment logging on another stream.
  * 16-bit cells render trilinear with the per-ray schedule (else AMR_ERR_ARG). */
 amr_status amr_render(amr_ctx* ctx, const amr_camera* cam, const float* tf_rgba_dev,
                       int32_t tf_n, const amr_render_params* params, float* out_rgba_dev,

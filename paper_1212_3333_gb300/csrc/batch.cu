@@ -175,7 +175,8 @@ amr_status launch_batch(amr_ctx* c, const BatchArgs& b, int storage, int shade, 
       t->v[v].item0 = (int32_t)std::min<int64_t>(tiles, INT32_MAX);
       tiles += (int64_t)t->v[v].tiles_x * ((b.v[v].height + 3) / 4);
     }
-    const TaskPlan plan = plan_tasks(c, tiles, stream);
+    TaskPlan plan;
+    if (tiles <= kTaskTiles) plan = plan_tasks(c, tiles, stream);
     if (tiles <= plan.tiles) {
       t->n_items = (int32_t)tiles;
       t->A.ts = plan.ts;

@@ -58,6 +58,13 @@ struct Packing {
   std::vector<int64_t> org;  // 3 per patch
 };
 
+// An allocation of the split march's workspace; captured: captured calls hold its address.
+struct TaskBuffer {
+  void* p = nullptr;
+  bool captured = false;
+};
+constexpr int64_t kTaskTiles = (int64_t)1 << 19;  // most tiles it has records for (2^24 pixels)
+
 struct DeviceState {
   DNode* nodes = nullptr;
   DLeaf* leaves = nullptr;
@@ -92,14 +99,17 @@ struct DeviceState {
   int32_t macro_cell = 1;                        // finest cells per macro cell per axis
   int32_t macro_dims[3] = {1, 1, 1};
   int device = -1;
-  // workspaces of the split march, each for up to task_pixels pixels; the last is in use,
-  // earlier ones stay for CUDA graphs that hold their addresses (sizes at least double)
-  std::vector<void*> task_spaces;
+  // workspace of the split march: its pool and its tile records (device.cpp), and what they were
+  // before they grew if captured calls hold those addresses (sizes at least double, so these
+  // take at most twice the largest)
+  TaskBuffer task_pool, task_tiles;
+  std::vector<void*> task_retired;
   TaskSpace tasks = {};
+  int64_t task_tile_cap = 0, task_left_cap = 0;  // tiles; entries of the list of tiles given up
+  int64_t task_refused = INT64_MAX;        // a pool of this many chunks could not be allocated,
+  int64_t task_tiles_refused = INT64_MAX;  // nor records of this many tiles
   cudaEvent_t work_event = nullptr;  // after the last call's work (WorkOrder)
   float dense_below = -INFINITY;     // a fifth of the cells lie below this value
-  int64_t task_pixels = 0;
-  int64_t task_refused = INT64_MAX;  // a workspace for this many pixels could not be allocated
 };
 
 // Calls on a context share its counters and workspaces, so each one's work waits for the last
@@ -133,6 +143,7 @@ class WorkOrder {
 struct TaskPlan {
   TaskSpace ts = {};
   long long tiles = 0;
+  long long left = 0;  // entries of the list of tiles given up
   int rounds(long long tiles_of_band) const;
 };
 

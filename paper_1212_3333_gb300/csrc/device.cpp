@@ -265,84 +265,138 @@ amr_status upload_max_pool(amr_ctx* c, const std::vector<std::vector<T>>& mb, cu
 
 }  // namespace
 
-// Workspace of the split march (36 bytes a task, and a segment record of 48 bytes for every
-// third): kTasksPerPixel tasks for every pixel - the 5-level hierarchy with a ramp transfer
-// function takes 23, and 8 records -, up to kMaxTasks, but kTileChunks chunks (320 tasks a
-// pixel) for every tile under way, so that dense tiles need not be given up: 1.7 GB for most
-// images, 3.5 GB at most.  (With 40 tasks a pixel alone, at 640 x 479 tiles were given up
-// and the frame took 5.4 instead of 2.7 ms.)  A call gets enough rounds for kDensePerPixel
-// tasks a pixel; what is denser goes to deferred_kernel (every sample opaque, 640 x 479, 480
-// tasks a pixel: all tasks in the workspace 14.3 ms, deferred_kernel alone 16.1).
+// Workspace of the split march: a pool (36 bytes a task, and a segment record of 48 bytes for
+// every third) and records of its tiles.  The pool has kTasksPerPixel tasks for every pixel - the
+// 5-level hierarchy with a ramp transfer function takes 23, and 8 segment records -, up to
+// kMaxTasks, but kTileChunks chunks (320 tasks a pixel) for every tile under way, so that dense
+// tiles need not be given up: 1.7 GB for most images, 3.5 GB at most.  (With 40 tasks a pixel
+// alone, at 640 x 479 tiles were given up and the frame took 5.4 instead of 2.7 ms.)  A call gets
+// enough rounds for kDensePerPixel tasks a pixel; what is denser goes to deferred_kernel (every
+// sample opaque, 640 x 479, 480 tasks a pixel: all tasks in the workspace 14.3 ms,
+// deferred_kernel alone 16.1).
 static constexpr int64_t kTasksPerPixel = 40, kDensePerPixel = 128, kTileChunks = 80;
 static constexpr int64_t kMaxTasks = (int64_t)1 << 26;
-static constexpr int64_t kBandPixels = (int64_t)1 << 24;
 static constexpr int64_t kWarps = 152 * 16;  // of the march, at once
 
-static int64_t task_rounds(int64_t pixels, int64_t chunks) {
+static int64_t task_rounds(int64_t tiles, int64_t chunks) {
   const int64_t usable = (chunks - chunks / 4) * kTaskChunk;
-  return std::min<int64_t>(64, (pixels * kDensePerPixel + usable - 1) / usable);
+  return std::min<int64_t>(64, (tiles * 32 * kDensePerPixel + usable - 1) / usable);
 }
 
-int TaskPlan::rounds(long long band) const { return (int)task_rounds(band * 32, ts.chunks); }
+int TaskPlan::rounds(long long tiles_of_band) const {
+  return (int)std::min<int64_t>(task_rounds(tiles_of_band, ts.chunks),
+                                left / std::max(1LL, tiles_of_band));
+}
+
+// A larger buffer in place of b; the old one is freed (the last call's work has ended then), or
+// kept for the captured calls that hold its address.  False, and b as it was, when out of memory.
+static bool replace_buffer(DeviceState& d, TaskBuffer& b, size_t bytes) {
+  try {
+    d.task_retired.reserve(d.task_retired.size() + 1);
+  } catch (const std::bad_alloc&) {
+    return false;
+  }
+  // (relaxed: another thread's capture must not be disturbed, nor refuse this)
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  void* p = nullptr;
+  const bool ok = cudaMalloc(&p, bytes) == cudaSuccess;
+  if (!ok) {
+    cudaGetLastError();
+  } else {
+    if (b.captured) {
+      d.task_retired.push_back(b.p);
+    } else if (b.p) {
+      cudaEventSynchronize(d.work_event);
+      cudaFree(b.p);
+    }
+    b.p = p;
+    b.captured = false;
+  }
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return ok;
+}
+
+// Offsets of consecutive arrays, each on a 256-byte boundary; returns the bytes of all.
+template <int N>
+static size_t lay_out(const size_t (&bytes)[N], size_t (&off)[N]) {
+  size_t at = 0;
+  for (int k = 0; k < N; ++k) {
+    off[k] = at;
+    at += (bytes[k] + 255) & ~(size_t)255;
+  }
+  return at;
+}
+
+static void grow_pool(DeviceState& d, int64_t tiles) {
+  const int64_t under_way = std::min(tiles, kWarps) * kTileChunks * kTaskChunk * 4 / 3;
+  const int64_t most = kMaxTasks / kTaskChunk;
+  const int64_t need =
+      std::min(std::max(tiles * 32 * kTasksPerPixel, under_way) / kTaskChunk, most);
+  if (need <= d.tasks.chunks || need >= d.task_refused) return;
+  const int64_t chunks = std::max(need, std::min<int64_t>(2 * (int64_t)d.tasks.chunks, most));
+  const size_t slots = (size_t)chunks * kTaskChunk;
+  const int64_t blocks = (int64_t)slots / 3 / kSegBlock + 2 * kWarps;
+  const size_t sizes[7] = {slots * sizeof(float4), slots * sizeof(float4), slots * sizeof(int32_t),
+                           (size_t)chunks * sizeof(int4),
+                           (size_t)blocks * kSegBlock * 3 * sizeof(float4),
+                           kHeads * sizeof(unsigned), kMaxBatchViews * sizeof(RayArgs)};
+  size_t off[7];
+  if (!replace_buffer(d, d.task_pool, lay_out(sizes, off))) {
+    d.task_refused = need;
+    return;
+  }
+  char* p = (char*)d.task_pool.p;
+  d.tasks.tasks = (float4*)(p + off[0]);
+  d.tasks.col = (float4*)(p + off[1]);
+  d.tasks.outer = (int32_t*)(p + off[2]);
+  d.tasks.meta = (int4*)(p + off[3]);
+  d.tasks.segs = (float4*)(p + off[4]);
+  d.tasks.heads = (unsigned*)(p + off[5]);
+  d.tasks.views = (RayArgs*)(p + off[6]);
+  d.tasks.chunks = (int32_t)chunks;
+  d.tasks.seg_blocks = (int32_t)blocks;
+}
+
+// (the list of tiles given up is as long as the rounds of the pool at hand need it; a larger
+// pool needs fewer)
+static void grow_tiles(DeviceState& d, int64_t need) {
+  if (need <= d.task_tile_cap || need >= d.task_tiles_refused) return;
+  const int64_t tiles = std::max(need, std::min(2 * d.task_tile_cap, kTaskTiles));
+  const int64_t left = tiles * task_rounds(tiles, d.tasks.chunks);
+  const size_t sizes[3] = {(size_t)tiles * sizeof(int2), (size_t)left * sizeof(int32_t),
+                           (size_t)tiles * sizeof(int32_t)};
+  size_t off[3];
+  if (!replace_buffer(d, d.task_tiles, lay_out(sizes, off))) {
+    d.task_tiles_refused = need;
+    return;
+  }
+  char* p = (char*)d.task_tiles.p;
+  d.tasks.tile = (int2*)(p + off[0]);
+  d.tasks.left = (int32_t*)(p + off[1]);
+  d.tasks.dense = (int32_t*)(p + off[2]);
+  d.task_tile_cap = tiles;
+  d.task_left_cap = left;
+}
 
 TaskPlan plan_tasks(amr_ctx* c, long long call_tiles, void* stream) {
   TaskPlan plan;
   DeviceState& d = c->dev;
   if (call_tiles <= 0) return plan;
-  const int64_t want = std::min<int64_t>(call_tiles * 32, std::max<int64_t>(kBandPixels, 32 * 8192));
+  const int64_t tiles = std::min<int64_t>(call_tiles, kTaskTiles);
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing((cudaStream_t)stream, &cap) != cudaSuccess) cudaGetLastError();
-  if (want > d.task_pixels && want < d.task_refused) {
-    const int64_t px = std::max(want, std::min(2 * d.task_pixels, kBandPixels));
-    const int64_t tiles = px / 32;
-    const int64_t under_way = std::min(tiles, kWarps) * kTileChunks * kTaskChunk * 4 / 3;
-    const int64_t chunks = std::min(std::max(px * kTasksPerPixel, under_way), kMaxTasks) / kTaskChunk;
-    const size_t slots = (size_t)chunks * kTaskChunk;
-    const int64_t blocks = (int64_t)slots / 3 / kSegBlock + 2 * kWarps;
-    const int64_t rounds = task_rounds(px, chunks);
-    const size_t sizes[10] = {slots * sizeof(float4), slots * sizeof(float4), slots * sizeof(int32_t),
-                             (size_t)chunks * sizeof(int4),
-                             (size_t)blocks * kSegBlock * 3 * sizeof(float4),
-                             (size_t)tiles * sizeof(int2),
-                             (size_t)(tiles * rounds) * sizeof(int32_t),
-                             (size_t)tiles * sizeof(int32_t), kHeads * sizeof(unsigned),
-                             kMaxBatchViews * sizeof(RayArgs)};
-    size_t off[11] = {0};
-    for (int k = 0; k < 10; ++k) off[k + 1] = off[k] + ((sizes[k] + 255) & ~(size_t)255);
-    char* p = nullptr;
-    if (cap == cudaStreamCaptureStatusNone) {
-      // (relaxed: another thread's capture must not be disturbed, nor refuse this)
-      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-      cudaThreadExchangeStreamCaptureMode(&mode);
-      const cudaError_t e = cudaMalloc((void**)&p, off[10]);
-      cudaThreadExchangeStreamCaptureMode(&mode);
-      if (e != cudaSuccess) {
-        cudaGetLastError();
-        p = nullptr;
-        d.task_refused = want;
-      }
-    }
-    if (p) {
-      d.task_spaces.push_back(p);
-      d.task_pixels = px;
-      d.tasks.tasks = (float4*)(p + off[0]);
-      d.tasks.col = (float4*)(p + off[1]);
-      d.tasks.outer = (int32_t*)(p + off[2]);
-      d.tasks.meta = (int4*)(p + off[3]);
-      d.tasks.segs = (float4*)(p + off[4]);
-      d.tasks.tile = (int2*)(p + off[5]);
-      d.tasks.left = (int32_t*)(p + off[6]);
-      d.tasks.dense = (int32_t*)(p + off[7]);
-      d.tasks.heads = (unsigned*)(p + off[8]);
-      d.tasks.views = (RayArgs*)(p + off[9]);
-      d.tasks.tile_chunks = (int32_t)std::max<int64_t>(1, 3 * chunks / std::min(tiles, kWarps));
-      d.tasks.chunks = (int32_t)chunks;
-      d.tasks.seg_blocks = (int32_t)blocks;
-    }
+  if (cap == cudaStreamCaptureStatusNone) {
+    grow_pool(d, tiles);
+    if (d.tasks.chunks > 0) grow_tiles(d, tiles);
+  } else {
+    d.task_pool.captured = d.task_tiles.captured = true;
   }
-  if (d.task_pixels == 0) return plan;
   plan.ts = d.tasks;
-  plan.tiles = d.task_pixels / 32;
+  plan.tiles = d.task_tile_cap;
+  plan.left = d.task_left_cap;
+  plan.ts.tile_chunks = (int32_t)std::max<int64_t>(
+      1, 3 * (int64_t)d.tasks.chunks / std::min(std::max<int64_t>(1, std::min(tiles, d.task_tile_cap)), kWarps));
   return plan;
 }
 
@@ -378,7 +432,9 @@ void release_device(amr_ctx* c) {
   cudaFree(d.img_scratch);
   cudaFree(d.log_counts);
   cudaFree(d.log_offsets);
-  for (void* p : d.task_spaces) cudaFree(p);
+  cudaFree(d.task_pool.p);
+  cudaFree(d.task_tiles.p);
+  for (void* p : d.task_retired) cudaFree(p);
   if (d.work_event) cudaEventDestroy(d.work_event);
   d = DeviceState();
   c->device_built = false;

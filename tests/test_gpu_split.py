@@ -155,6 +155,43 @@ def test_first_call_captured(amr):
     assert torch.equal(out[0], out[1]) and torch.equal(again, out[1])
 
 
+def test_one_workspace_at_a_time(amr):
+    """Images of growing sizes replace the context's workspace; one that a captured call holds
+    stays, and its replays give the same image; destroying the context gives all back."""
+    import torch
+
+    ctx, (vmin, vmax) = _context(amr)
+    tf = torch.as_tensor(_opaque_tf(), device="cuda")
+    p, _ = params_pair(amr, vmin, vmax, schedule=3, shade=1)
+    outs = [torch.zeros((h, w, 4), device="cuda") for w, h in ((97, 61), (640, 479), (1700, 1000))]
+    cams = [synth.orbit_camera(2, o.shape[1], o.shape[0]) for o in outs]
+    first = torch.zeros_like(outs[0])
+    torch.cuda.synchronize()
+    free = [torch.cuda.mem_get_info()[0]]
+
+    def render(k):
+        ctx.amr_render(cams[k], tf, p, outs[k])
+        torch.cuda.synchronize()
+        free.append(torch.cuda.mem_get_info()[0])
+
+    render(0)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        ctx.amr_render(cams[0], tf, p, first)
+    for k in (1, 2, 1, 0, 2):
+        render(k)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(first, outs[0])
+    used = [(free[0] - f) / 1e9 for f in free]
+    slack = used[1] + 0.1  # the captured call's workspace; the allocator's rounding
+    assert 1.6 < used[2] < 1.8 + slack and 3.3 < used[3] < 3.6 + slack
+    assert max(used[4:]) <= used[3] + 0.01
+    del g
+    ctx.amr_destroy()
+    assert torch.cuda.mem_get_info()[0] >= free[0] - 10 ** 8
+
+
 def test_calls_on_two_streams_take_turns(amr):
     """The streams share the context's workspace and counters: the second call waits for the
     first, so images and sample counts are those of calls made one at a time."""
