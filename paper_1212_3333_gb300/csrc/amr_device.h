@@ -38,8 +38,8 @@ constexpr int kQueueCounter = 5;       // counters[5]: head of the batched work 
 constexpr int kShadeShadowBit = 4;     // kernel shading variant bit: secondary rays
 constexpr int kShadeMaxBit = 8;        // kernel variant bit: stencil-maximum opacity test
 constexpr int kMaxBatchViews = 128;
-constexpr long long kLargePixels = 3000000;  // images where the per-ray loop beats the
-                                             // one-kernel deferred march
+constexpr long long kLargePixels = 3000000;  // images whose rays stay together: the per-ray
+                                             // loop beats the one-kernel deferred march
 // status bits raised by kernels (OR-ed into counters[1])
 constexpr unsigned long long kStatusCapacity = 1ull;   // segment or sample bound hit
 constexpr unsigned long long kStatusDevice = 2ull;     // malformed tree reached
@@ -139,7 +139,8 @@ constexpr int kTaskSampleBits = 23;  // sample number in a task; the lane's numb
 static_assert(kMaxSamplesPerSegment <= (1 << kTaskSampleBits), "sample number in a task");
 // counters of the workspace: the first kRoundHeads are zeroed for every round
 enum { kHeadChunk = 0, kHeadSegBlock = 1, kHeadOuter = 2, kRoundHeads = 3, kHeadTile = 3,
-       kHeadLeft = 4, kHeadRest = 5, kHeadReady = 6, kHeadDense = 7, kHeads = 8 };
+       kHeadLeft = 4, kHeadRest = 5, kHeadReady = 6, kHeadDense = 7, kHeadTasks = 8, kHeadSegs = 9,
+       kHeads = 10 };
 struct TaskSpace {
   float4* tasks;        // segment record, sample number | lane << 23, value, weight
   float4* col;          // per task: colour, weight
@@ -151,10 +152,12 @@ struct TaskSpace {
   int32_t* left;        // tiles given up because the workspace was full (once per round)
   int32_t* dense;       // tiles given up because they take more than tile_chunks
   unsigned* heads;      // chunks, segment blocks, outer tasks, tiles handed out; left tiles,
-                        // those of them handed out again, those of earlier rounds; dense tiles
+                        // those of them handed out again, those of earlier rounds; dense
+                        // tiles; tasks and segments of the tiles done, in 32s
   struct RayArgs* views; // batches: per view its rays (rows of the whole image)
   int32_t chunks, seg_blocks;
   int32_t tile_chunks;  // most chunks of one tile
+  float dense_ratio;    // tasks per segment beyond which the one-kernel march is faster
 };
 
 struct RenderArgs {
@@ -197,7 +200,8 @@ struct RenderArgs {
   int32_t learned_min_samples;   // learned modes: segments shorter than this skip the MLP
   long long mdelta;              // stencil-maximum brick = value brick + mdelta bytes (ptr)
   TaskSpace ts;                  // split march; heads null: none
-  float dense_below;             // a fifth of the cells lie below this value
+  float dense_below;             // split march: thresholds up to this one leave every tile to
+                                 // the one-kernel march
 };
 
 struct TraceArgs {

@@ -176,10 +176,11 @@ amr_status launch_batch(amr_ctx* c, const BatchArgs& b, int storage, int shade, 
       tiles += (int64_t)t->v[v].tiles_x * ((b.v[v].height + 3) / 4);
     }
     TaskPlan plan;
-    if (tiles <= kTaskTiles) plan = plan_tasks(c, tiles, stream);
+    if (tiles <= kTaskTiles) plan = plan_tasks(c, tiles, TaskUse::batch, stream, b.n_views);
     if (tiles <= plan.tiles) {
       t->n_items = (int32_t)tiles;
       t->A.ts = plan.ts;
+      t->A.dense_below = plan.dense_below;
       batch_views_kernel<<<1, kMaxBatchViews, 0, s>>>(*t);
       cudaError_t e = cudaGetLastError();
       const int rounds = plan.rounds(tiles);

@@ -321,10 +321,10 @@ static bool textures(const amr_ctx* c) {
 // (schedule 3) wherever it applies - Phong, trilinear, no learned proposal - and the per-ray
 // schedule otherwise.  Every schedule gives the same image bit for bit (with secondary rays to
 // rounding), so the choice affects time only.  Single images of kLargePixels pixels and more
-// stay on the per-ray schedule where deferred shading has no workspace - texture storages, calls
-// that may not allocate - and loses (textures, 1900 x 1800: 31.8 against 37 ms), and when
-// samples_per_iter, which no kernel of schedules 0 and 1 reads, is outside its range.
-
+// stay on the per-ray schedule for texture storages and calls that may not allocate (textures,
+// 1900 x 1800: 31.8 against 37 ms; on linear storages schedule 3 falls back to the per-ray loop
+// by itself), and when samples_per_iter, which no kernel of schedules 0 and 1 reads, is outside
+// its range.
 static const amr_render_params* resolve_schedule(const amr_render_params* p, int64_t pixels,
                                                  bool one_kernel, amr_render_params* tmp) {
   if (!p || p->schedule != AMR_SCHEDULE_AUTO) return p;
@@ -420,7 +420,6 @@ static amr_status prepare_render(amr_ctx* c, const amr_camera* cam, int32_t tf_n
   a->light_ambient = (float)p->light_ambient;
   a->coarse_factor = p->coarse_factor;
   a->learned_min_samples = p->learned_min_samples;
-  a->dense_below = c->dev.dense_below;
   a->mdelta = c->dev.mpool ? (long long)((char*)c->dev.mpool - (char*)c->dev.pool) : 0;
   if (c->dtype != AMR_F32 && (p->interp != AMR_INTERP_TRILINEAR || p->schedule == 1))
     return fail(c, AMR_ERR_ARG, "16-bit cells render trilinear with schedule 0, 2 or 3");

@@ -109,7 +109,8 @@ struct DeviceState {
   int64_t task_refused = INT64_MAX;        // a pool of this many chunks could not be allocated,
   int64_t task_tiles_refused = INT64_MAX;  // nor records of this many tiles
   cudaEvent_t work_event = nullptr;  // after the last call's work (WorkOrder)
-  float dense_below = -INFINITY;     // a fifth of the cells lie below this value
+  float fifth_below = -INFINITY, half_below = -INFINITY;  // so many cells lie below these values
+  double leaf_cells = 0.0;           // cells per leaf
 };
 
 // Calls on a context share its counters and workspaces, so each one's work waits for the last
@@ -144,6 +145,7 @@ struct TaskPlan {
   TaskSpace ts = {};
   long long tiles = 0;
   long long left = 0;  // entries of the list of tiles given up
+  float dense_below = 0;  // RenderArgs::dense_below of the call
   int rounds(long long tiles_of_band) const;
 };
 
@@ -192,8 +194,9 @@ amr_status upload(amr_ctx* c, void* stream);
 void release_device(amr_ctx* c);
 // The split march's workspace for a call with that many 8x4 tiles, grown when it is too small
 // and the stream is not being captured; it may have fewer tiles (out of memory, or a first
-// call captured: none).  The caller holds a WorkOrder.
-TaskPlan plan_tasks(amr_ctx* c, long long tiles, void* stream);
+// call captured: none), and has none where a one-kernel march is faster.  The caller holds a WorkOrder.
+enum class TaskUse { image, shadow, batch };
+TaskPlan plan_tasks(amr_ctx* c, long long tiles, TaskUse use, void* stream, int views = 1);
 // kernels (march.cu)
 amr_status launch_render(amr_ctx* c, const RenderArgs& a, int storage, int interp, int shade,
                          int schedule, void* stream);

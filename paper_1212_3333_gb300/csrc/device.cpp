@@ -379,10 +379,34 @@ static void grow_tiles(DeviceState& d, int64_t need) {
   d.task_left_cap = left;
 }
 
-TaskPlan plan_tasks(amr_ctx* c, long long call_tiles, void* stream) {
+// Where the split march pays.  It saves segment fetches their latency and pays for every task's
+// way through memory, so what decides is the tasks per segment (counted as tiles are done), how
+// dear a fetch is (the leaves), and how well rays of large images stay together in the one-kernel
+// marches; small images wait for their longest rays.  Measured at 300^2 to 2048^2 on hierarchies of
+// 77 to 32,198 leaves with transfer functions that make 2 to 100 % of the cells opaque (ms, split
+// / one kernel, tasks per segment): 1,175 leaves 1024^2 3.19 / 3.41 (2.3), 5.11 / 4.82 (4.9);
+// 3,998 leaves 1024^2 5.59 / 5.81 (3.5), 8.26 / 7.26 (5.6), 640 x 479 2.92 / 3.34 (7.6), 2048^2 9.56
+// / 9.94 (1.0), 11.8 / 11.3 (1.5); 30,164 leaves 1024^2 14.7 / 16.0 (4.1), 21.3 / 20.5 (6.6), 2048^2
+// 28.8 / 30.8 (1.7), 38.7 / 37.2 (2.8); 32,198 leaves of 1,150 cells, where every fourth gradient
+// leaves its leaf, 1500 x 1100 8.1 / 11.3 (2.0), 2048^2 33.8 / 36.0 (3.3); 77 leaves 64^2 0.23 /
+// 0.33, 256^2 0.308 / 0.303, 1024^2 1.26 / 1.02, batches of 64 views of 64^2 0.59 / 0.70, of 4 of
+// 900^2 3.71 / 2.52.
+constexpr int64_t kFewLeaves = 1000, kManyLeaves = 10000;  // of the hierarchy
+constexpr double kSmallLeaf = 2000.0;                      // cells
+constexpr int64_t kFewTiles = 1024;      // images that gain on any hierarchy,
+constexpr int64_t kFewViewTiles = 4096;  // and batches, with fewer tiles per view than this
+constexpr int64_t kWaveTiles = 600000 / 32;  // images of a few tiles per warp: no time to stop
+
+TaskPlan plan_tasks(amr_ctx* c, long long call_tiles, TaskUse use, void* stream, int views) {
   TaskPlan plan;
   DeviceState& d = c->dev;
+  const int64_t leaves = (int64_t)c->tree.leaf_patch.size();
+  const bool many = leaves >= kManyLeaves;
   if (call_tiles <= 0) return plan;
+  if (use != TaskUse::shadow && leaves < kFewLeaves &&
+      call_tiles > (use == TaskUse::batch ? views * kFewViewTiles : kFewTiles))
+    return plan;
+  if (use == TaskUse::image && !many && call_tiles * 32 >= kLargePixels) return plan;
   const int64_t tiles = std::min<int64_t>(call_tiles, kTaskTiles);
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing((cudaStream_t)stream, &cap) != cudaSuccess) cudaGetLastError();
@@ -395,6 +419,16 @@ TaskPlan plan_tasks(amr_ctx* c, long long call_tiles, void* stream) {
   plan.ts = d.tasks;
   plan.tiles = d.task_tile_cap;
   plan.left = d.task_left_cap;
+  const bool small_leaves = many && d.leaf_cells < kSmallLeaf;
+  plan.ts.dense_ratio = use == TaskUse::shadow ? INFINITY
+                        : use == TaskUse::image && tiles * 32 >= kLargePixels
+                            ? (small_leaves ? 4.0f : 2.5f)
+                        : small_leaves || tiles < kWaveTiles ? 12.0f
+                                                             : (many ? 6.0f : 4.0f);
+  // Not begun at all: transfer functions that make four fifths of the cells opaque, or half of
+  // them where the pool cannot hold the image whatever it shows.
+  const bool holds = (int64_t)d.tasks.chunks * kTaskChunk >= tiles * 32 * 250;
+  plan.dense_below = small_leaves || holds || use != TaskUse::image ? d.fifth_below : d.half_below;
   plan.ts.tile_chunks = (int32_t)std::max<int64_t>(
       1, 3 * (int64_t)d.tasks.chunks / std::min(std::max<int64_t>(1, std::min(tiles, d.task_tile_cap)), kWarps));
   return plan;
@@ -492,8 +526,8 @@ static int32_t face_list(const Tree& t, const int64_t* root, size_t m, int f, in
   return (int32_t)word;
 }
 
-// The value a fifth of the bricks' cells lie below, from at most about 2^16 of them.
-static float low_quantile(const amr_ctx* c) {
+// The values a fifth and half of the bricks' cells lie below, from at most about 2^16 of them.
+static void low_quantiles(amr_ctx* c) {
   size_t cells = 0, at = 0;
   for (const auto& b : c->bricks) cells += b.size();
   const size_t stride = std::max<size_t>(1, cells >> 16);
@@ -503,16 +537,23 @@ static float low_quantile(const amr_ctx* c) {
       if (!std::isnan(b[at])) v.push_back(b[at]);
     at -= b.size();
   }
-  if (v.empty()) return -INFINITY;
-  std::nth_element(v.begin(), v.begin() + v.size() / 5, v.end());
-  return v[v.size() / 5];
+  c->dev.fifth_below = c->dev.half_below = -INFINITY;
+  if (v.empty()) return;
+  const auto half = v.begin() + v.size() / 2, fifth = v.begin() + v.size() / 5;
+  std::nth_element(v.begin(), half, v.end());
+  c->dev.half_below = *half;
+  if (fifth != half) std::nth_element(v.begin(), fifth, half);
+  c->dev.fifth_below = *fifth;
 }
 
 amr_status upload(amr_ctx* c, void* stream_v) {
   cudaStream_t stream = (cudaStream_t)stream_v;
   if (c->device_built) release_device(c);
   DeviceState& d = c->dev;
-  d.dense_below = low_quantile(c);
+  low_quantiles(c);
+  double cells = 0.0;
+  for (const Patch& q : c->patches) cells += (double)(q.n[0] * q.n[1] * q.n[2]);
+  d.leaf_cells = cells / std::max<size_t>(1, c->tree.leaf_patch.size());
   CK(cudaGetDevice(&d.device));
   if (!d.work_event) CK(cudaEventCreateWithFlags(&d.work_event, cudaEventDisableTiming));
   const Tree& t = c->tree;

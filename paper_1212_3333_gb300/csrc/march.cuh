@@ -1841,11 +1841,36 @@ __device__ __forceinline__ void stage_tf(const RenderArgs& A, float4* s_tf, int*
 #endif
 static_assert(AMR_WARP_TILE_W == 4 || AMR_WARP_TILE_W == 8 || AMR_WARP_TILE_W == 16,
               "warp tile width");
+// The 8x4-pixel tiles that a one-kernel march renders: all of them, or with a workspace (A.ts)
+// those that the split march left: given up for lack of room and not taken up again, dense, and
+// not started.
+struct RestTiles {
+  int left = 0, dense = 0, retried = 0, begun = 0, all = 0;
+  __device__ __forceinline__ RestTiles() {}
+  __device__ __forceinline__ RestTiles(const RenderArgs& A, int all_tiles) : all(all_tiles) {
+    const unsigned* heads = A.ts.heads;
+    if (!heads) return;
+    retried = (int)__ldcg(heads + kHeadRest);
+    left = (int)__ldcg(heads + kHeadLeft) - retried;
+    dense = (int)__ldcg(heads + kHeadDense);
+    begun = (int)min(__ldcg(heads + kHeadTile), (unsigned)all_tiles);
+  }
+  __device__ __forceinline__ int count() const { return left + dense + all - begun; }
+  __device__ __forceinline__ int tile(const RenderArgs& A, int k) const {
+    if (k < left) return __ldcg(A.ts.left + retried + k);
+    if (k < left + dense) return __ldcg(A.ts.dense + k - left);
+    return k + begun - left - dense;
+  }
+};
+
 template <int ST, int INTERP, int SHADE, bool QUEUE = true>
 __global__ void __launch_bounds__(128, kMinBlocks<SHADE>)
     march_kernel(const __grid_constant__ RenderArgs A) {
-  // (with a workspace: only an image that the split march did not begin)
-  if (A.ts.heads && __ldcg(A.ts.heads + kHeadTile) != 0) return;
+  RestTiles rest;  // (with a workspace: the tiles that the split march left)
+  if constexpr (QUEUE && AMR_WARP_TILE_W == 8) {
+    rest = RestTiles(A, ((A.ray.width + 7) / 8) * ((A.ray.rows + 3) / 4));
+    if (rest.count() == 0) return;
+  }
   extern __shared__ float4 smem[];
   float4* s_tf = smem;
   int* s_nz = reinterpret_cast<int*>(smem + A.tf_n);
@@ -1879,7 +1904,7 @@ __global__ void __launch_bounds__(128, kMinBlocks<SHADE>)
   if constexpr (QUEUE) {
     constexpr int TW = AMR_WARP_TILE_W, TH = 32 / TW;
     const int tiles_x = (R.width + TW - 1) / TW;
-    const int n_tiles = tiles_x * ((R.rows + TH - 1) / TH);
+    const int n_tiles = TW == 8 ? rest.count() : tiles_x * ((R.rows + TH - 1) / TH);
     // each pass takes one tile, and the queue hands out every tile once
     for (;;) {
       int t = 0;
@@ -1889,6 +1914,7 @@ __global__ void __launch_bounds__(128, kMinBlocks<SHADE>)
       }
       t = __shfl_sync(0xffffffffu, t, 0);
       if (t >= n_tiles) break;
+      if (TW == 8) t = rest.tile(A, t);
       march_pixel((t % tiles_x) * TW + lane % TW, (t / tiles_x) * TH + lane / TW);
     }
   } else {

@@ -419,33 +419,21 @@ struct StagedTf<BatchArgs> {
 };
 
 // Schedule 3 in one kernel: persistent warps taking 8x4-pixel tiles from the global queue (as
-// march_kernel does for the per-ray loop), each marching its tile with deferred shading.  With
-// a workspace (A.ts) it takes the tiles that the split march left: those it gave up for lack of
-// room and did not take up again, the dense ones, and the ones it did not start.
+// march_kernel does for the per-ray loop), each marching its tile with deferred shading.
 template <int ST, int SHADE, typename Args = RenderArgs>
 __global__ void __launch_bounds__(128, AMR_MIN_BLOCKS_DEFERRED)
     deferred_kernel(const __grid_constant__ Args P) {
   const RenderArgs& A = render_args(P);
   const int all_tiles = count_tiles(P);
-  const bool rest = A.ts.heads != nullptr;
-  int left = 0, dense = 0, retried = 0, begun = all_tiles;
-  if (rest) {
-    retried = (int)__ldcg(A.ts.heads + kHeadRest);
-    left = (int)__ldcg(A.ts.heads + kHeadLeft) - retried;
-    dense = (int)__ldcg(A.ts.heads + kHeadDense);
-    begun = (int)min(__ldcg(A.ts.heads + kHeadTile), (unsigned)all_tiles);
-    if (left == 0 && dense == 0 && begun == all_tiles) return;
-    if (std::is_same<Args, RenderArgs>::value && (SHADE & kShadeShadow) == 0 &&
-        begun == 0 && all_tiles * 32LL >= kLargePixels)
-      return;  // march_kernel has rendered it
-  }
+  const RestTiles rest(A, all_tiles);
+  const int n_tiles = rest.count();
+  if (n_tiles == 0) return;
   extern __shared__ float4 smem[];
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
   DeferArea& Q = reinterpret_cast<DeferArea*>(reinterpret_cast<char*>(smem) +
                                               StagedTf<Args>::bytes(P))[tid >> 5];
   const StagedTf<Args> staged(P, smem, tid);
   const int lane = tid & 31;
-  const int n_tiles = rest ? left + dense + all_tiles - begun : all_tiles;
   unsigned nsamp = 0;
   unsigned long long status = 0;
   // each pass takes one tile, and the queue hands out every tile once
@@ -457,11 +445,7 @@ __global__ void __launch_bounds__(128, AMR_MIN_BLOCKS_DEFERRED)
     }
     t = __shfl_sync(0xffffffffu, t, 0);
     if (t >= n_tiles) break;
-    if (rest) {
-      if (t < left) t = __ldcg(A.ts.left + retried + t);
-      else if (t < left + dense) t = __ldcg(A.ts.dense + t - left);
-      else t += begun - left - dense;
-    }
+    t = rest.tile(A, t);
     const TileAt p = tile_at(P, t);
     const RayArgs& R = tile_rays(P, p);
     int i, jr;

@@ -108,6 +108,22 @@ cudaError_t launch_tiles(K kernel, size_t smem, cudaStream_t s, const Args& a) {
   return e == cudaSuccess ? launch_stride(kernel, smem, s, a, 0) : e;
 }
 
+template <int ST>
+constexpr bool kLinearStorage = ST != ST_TEXOBJ && ST != ST_ATLAS_TEX3D;
+
+// Deferred shading in one kernel, of all tiles or of those the split march left: the per-ray
+// loop for single images of kLargePixels pixels and more, whose rays stay together (2048^2, ms,
+// deferred / per ray: 77 leaves 3.7 / 2.7, 3,998 leaves ramp 11.0 / 9.7, half of the cells opaque
+// 31.2 / 25.6, 30,164 leaves 85.8 / 85.4; but ramp 17.9 / 19.0, which the split march takes).
+template <int ST, int SHADE, typename Args>
+cudaError_t launch_one_kernel(cudaStream_t s, const Args& a) {
+  const size_t base = StagedTf<Args>::bytes(a);
+  if constexpr (std::is_same<Args, RenderArgs>::value && kLinearStorage<ST> &&
+                (SHADE & kShadeShadow) == 0 && AMR_WARP_TILE_W == 8)
+    if (tiles_of(a) * 32 >= kLargePixels) return launch_tiles(march_kernel<ST, 1, SHADE>, base, s, a);
+  return launch_tiles(deferred_kernel<ST, SHADE, Args>, base + 4 * sizeof(DeferArea), s, a);
+}
+
 // One band of the split march (b carries its workspace), in rounds that each fill the
 // workspace at most once, then the tiles that were left.
 template <int ST, int SHADE, typename Args>
@@ -125,20 +141,15 @@ cudaError_t launch_rounds(int rounds, cudaStream_t s, const Args& b) {
     if (e == cudaSuccess) e = launch_stride(split_outer_kernel<ST, SHADE, Args>, base, s, b, 4);
     if (e == cudaSuccess) e = launch_stride(split_sum_kernel<Args>, 0, s, b, 4);
   }
-  // an image whose tiles are all dense (every sample opaque, ms: 1024^2 46 deferred, 49 per ray
-  // before; 2048^2 146 deferred, 119 per ray)
-  if constexpr (std::is_same<Args, RenderArgs>::value && (SHADE & kShadeShadow) == 0)
-    if (e == cudaSuccess && tiles_of(b) * 32 >= kLargePixels)
-      e = launch_tiles(march_kernel<ST, 1, SHADE>, base, s, b);
   if (e != cudaSuccess) return e;
-  return launch_tiles(deferred_kernel<ST, SHADE, Args>, base + 4 * sizeof(DeferArea), s, b);
+  return launch_one_kernel<ST, SHADE>(s, b);
 }
 
 // Deferred shading of one image: the split march in bands of rows that the workspace has tile
 // records for, or without a workspace the one-kernel march.
 template <int ST, int SHADE>
 cudaError_t launch_shaded(const TaskPlan& plan, cudaStream_t s, const RenderArgs& a) {
-  if constexpr (ST != ST_TEXOBJ && ST != ST_ATLAS_TEX3D) {
+  if constexpr (kLinearStorage<ST>) {
     const long long tiles_x = (a.ray.width + 7) / 8;
     const int band = 4 * (int)std::min(plan.tiles / tiles_x, 1LL << 20);  // rows
     if (band > 0) {
@@ -149,13 +160,13 @@ cudaError_t launch_shaded(const TaskPlan& plan, cudaStream_t s, const RenderArgs
         b.ray.row0 = a.ray.row0 + row;
         b.ray.rows = std::min(band, a.ray.rows - row);
         b.out = a.out + (size_t)row * a.ray.width;
+        b.dense_below = plan.dense_below;
         e = launch_rounds<ST, SHADE>(plan.rounds(tiles_of(b)), s, b);
       }
       return e;
     }
   }
-  return launch_tiles(deferred_kernel<ST, SHADE>, StagedTf<RenderArgs>::bytes(a) + 4 * sizeof(DeferArea),
-                      s, a);
+  return launch_one_kernel<ST, SHADE>(s, a);
 }
 
 template <int ST>
@@ -173,8 +184,8 @@ amr_status launch_storage(amr_ctx* c, const RenderArgs& a, int interp, int shade
   TaskPlan plan;
   // (not for texture storages, where it measured slower at 1900 x 1800: 37.1 against 31.8 ms;
   // nor for a caller that brings its own counters and may not allocate)
-  constexpr bool kLinear = ST != ST_TEXOBJ && ST != ST_ATLAS_TEX3D;
-  if (kLinear && schedule == 3 && a.counters == c->dev.counters) plan = plan_tasks(c, tiles_of(a), s);
+  if (kLinearStorage<ST> && schedule == 3 && a.counters == c->dev.counters) 
+    plan = plan_tasks(c, tiles_of(a), (shade & kShadeShadow) != 0 ? TaskUse::shadow : TaskUse::image, s);
   cudaError_t e;
   if (shade & kShadeShadow) {
     // secondary rays to the point light: per-ray schedule (a lane marches its samples'

@@ -21,18 +21,20 @@
 // beyond its end: they are dropped, and not counted.  (With secondary rays each light ray's
 // transmittance is a product taken 32 samples per round, so those images agree to rounding.)
 //
-// Measured (5-level hierarchy, 1.3e8 cells, Phong with every brick, one kernel against this,
-// ms): 640 x 479 3.49 / 1.99, 1024^2 9.3 / 5.3 (march 5.2, shading 0.64 + 0.95, sums 0.25
-// alone under the profiler), 2048^2 23.5 / 17.4; 8 levels, BF16, 1500 x 1100 17.0 / 10.1;
-// secondary rays 393 x 371 21.2 / 5.7 (a tile's light rays no longer wait for one another).
-// Unshaded f16 1917 x 1083 4.8 / 4.3.  The march is bound by the latency of dependent loads
-// (fetches a third of it) at 16 warps per SM; 5 and 6 blocks spill and lose.
+// Measured (5-level hierarchy, 1.3e8 cells, Phong with every brick, one kernel against this when
+// it came in, ms): 640 x 479 3.49 / 1.99, 1024^2 9.3 / 5.3 (march 5.2, shading 0.64 + 0.95, sums
+// 0.25 alone under the profiler), 2048^2 23.5 / 17.4; 8 levels, BF16, 1500 x 1100 17.0 / 10.1;
+// secondary rays 393 x 371 21.2 / 5.7 (a tile's light rays no longer wait for one another).  The
+// march is bound by the latency of dependent loads (fetches a third of it) at 16 warps per SM;
+// shaded, 5 and 6 blocks spill and lose (unshaded 5 win: fewer registers are live).
 //
 // The tasks live in a workspace of bounded size, so a launch of large or dense images goes in
-// rounds: the march hands out tiles until the workspace is nearly full, the other kernels
-// empty it, and the next round goes on.  A tile that finds it full is given up, whole, until a
-// later round.  Dense tiles, and what the last round leaves, go to deferred_kernel, which needs
-// no workspace.
+// rounds: the march hands out tiles until the rest of the workspace is what the tiles under way
+// will take, the other kernels empty it, and the next round goes on.  A tile that finds it full
+// is given up, whole, until a later round.  Every task passes through device memory, so dense
+// images are faster in the one-kernel marches: plan_tasks says where, the march counts tasks and
+// segments as it goes, and what it leaves - with dense tiles, and what the last round leaves -
+// goes to one of those, which need no workspace.
 #pragma once
 #include "march_deferred.cuh"
 
@@ -66,6 +68,7 @@ struct CandArea<false> {
   float3 col[32];
 };
 constexpr float kNoWeight = -2.0f;
+constexpr float kDenseSlack = 4096.0f;  // segments (in 32s) before the density counts
 
 // The bits of a warp's `count` tasks (lane q holds the owner of task q) that belong to the
 // calling lane.
@@ -108,7 +111,8 @@ __device__ __forceinline__ int march_tile(const RenderArgs& A, const RayArgs& R,
                                            bool active, const float4* s_tf, const int* s_nz,
                                            float clear_below, CandArea<(SHADE & 3) != 0>& Q,
                                            RayF& rf, SegBlock& blk, int tile_id, int view, float4& px,
-                                           int2& tile, unsigned& nsamp, unsigned long long& status) {
+                                           int2& tile, int& segs, unsigned& nsamp,
+                                           unsigned long long& status) {
   constexpr bool MX = (SHADE & kShadeMaxBit) != 0;  // the stencil-maximum test
   constexpr bool SHADED = (SHADE & 3) != 0;
   const unsigned FULL = 0xffffffffu;
@@ -409,6 +413,7 @@ __device__ __forceinline__ int march_tile(const RenderArgs& A, const RayArgs& R,
   if (met & kMetTree) status |= kStatusDevice;
   px.w = Acc;
   tile = make_int2(first, tasks);
+  segs = SHADED ? __reduce_add_sync(FULL, seg) : 0;
   return kTileDone;
 }
 
@@ -443,7 +448,6 @@ __global__ void __launch_bounds__(128, (SHADE & 3) != 0 ? AMR_SPLIT_MARCH_BLOCKS
     if (__ldcg(A.ts.heads + kHeadTile) >= (unsigned)n_tiles &&
         __ldcg(A.ts.heads + kHeadRest) >= ready)
       return;
-    if (ready != 0 && (blockIdx.x & 1)) return;  // there was no room: half as many tiles at once
   }
   extern __shared__ float4 smem[];
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
@@ -464,12 +468,18 @@ __global__ void __launch_bounds__(128, (SHADE & 3) != 0 ? AMR_SPLIT_MARCH_BLOCKS
     int t = n_tiles;
     if (lane == 0) {
       if constexpr (SHADED) {
-        // a quarter of the workspace is kept for the tiles that are under way; an image of
-        // mostly dense tiles is left as it is
-        const unsigned dense = __ldcg(A.ts.heads + kHeadDense);
-        if (__ldcg(A.ts.heads + kHeadChunk) < (unsigned)(A.ts.chunks - A.ts.chunks / 4) &&
-            __ldcg(A.ts.heads + kHeadSegBlock) < (unsigned)(A.ts.seg_blocks - A.ts.seg_blocks / 4) &&
-            (dense < 256u || 2u * dense < __ldcg(A.ts.heads + kHeadTile))) {
+        // Room is kept for the tiles that are under way: a quarter of the pool, or what as many
+        // tiles as there are warps take on average (with a quarter alone, dense tiles were given
+        // up by the hundred and marched again).  An image with more tasks per segment than
+        // pays is left to the one-kernel march from there on.
+        const unsigned* H = A.ts.heads;
+        const float taken = (float)max(__ldcg(H + kHeadTile), 1u), tasks = (float)__ldcg(H + kHeadTasks);
+        const float room = fmaxf(0.25f * (float)A.ts.chunks,
+                                 (float)min((int)gridDim.x * 4, n_tiles) *
+                                     (0.5f + tasks * (32.0f / kTaskChunk) / taken));
+        if ((float)__ldcg(H + kHeadChunk) + room < (float)A.ts.chunks &&
+            __ldcg(H + kHeadSegBlock) < (unsigned)(A.ts.seg_blocks - A.ts.seg_blocks / 4) &&
+            tasks <= A.ts.dense_ratio * ((float)__ldcg(H + kHeadSegs) + kDenseSlack)) {
           t = (int)min(atomicAdd(A.ts.heads + kHeadTile, 1u), (unsigned)n_tiles);
           if (t == n_tiles && ready != 0) {
             // (a warp that takes one too many puts it back)
@@ -492,17 +502,22 @@ __global__ void __launch_bounds__(128, (SHADE & 3) != 0 ? AMR_SPLIT_MARCH_BLOCKS
     const bool active = i < p.width && jr < p.rows && j < R.height;
     float4 px;
     int2 tile;
+    int segs = 0;
     // nearly everything opaque: one kernel is faster (640 x 479, 480 opaque samples a pixel:
     // 16.1 ms alone, 24.7 after a workspace full of tasks), so the tile is left to it
     int how = kTileDense;
     if (!SHADED || staged.clear_below(p) > A.dense_below)
       how = march_tile<ST, SHADE>(A, R, i, j, active, staged.tf(p), staged.nz(p),
-                                  staged.clear_below(p), Q, rf, blk, t, p.view, px, tile, nsamp,
+                                  staged.clear_below(p), Q, rf, blk, t, p.view, px, tile, segs, nsamp,
                                   status);
     if (how == kTileDone) {
       if (SHADED && tile.y == 0) px = make_float4(0.f, 0.f, 0.f, px.w);  // nothing to shade
       if (active) p.out[p.at(i, jr)] = px;
-      if (SHADED && lane == 0 && tile.y != 0) A.ts.tile[t] = tile;
+      if (SHADED && lane == 0) {
+        if (tile.y != 0) A.ts.tile[t] = tile;
+        atomicAdd(A.ts.heads + kHeadTasks, (unsigned)(tile.y + 31) >> 5);
+        atomicAdd(A.ts.heads + kHeadSegs, (unsigned)(segs + 31) >> 5);
+      }
     } else if (lane == 0) {
       if (how == kTileDense) A.ts.dense[atomicAdd(A.ts.heads + kHeadDense, 1u)] = t;
       else A.ts.left[atomicAdd(A.ts.heads + kHeadLeft, 1u)] = t;

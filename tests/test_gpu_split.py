@@ -20,10 +20,15 @@ def amr():
     return m
 
 
-def _context(amr, seed=3, maxbrick=True, gradient=True):
-    h = random_hierarchy(seed, n0=12, num_levels=3, patches_per_level=6)
-    ctx = amr.from_hierarchy(h)
-    ctx.amr_build_kdtree("ptr", gradient=gradient, halo=2, maxbrick=maxbrick)
+def _hierarchy(seed=3):
+    """1,629 leaves: the split march is for hierarchies of 1,000 and more."""
+    return random_hierarchy(seed, n0=16, num_levels=4, patches_per_level=40, max_size=8)
+
+
+def _context(amr, seed=3, maxbrick=True, gradient=True, storage="ptr", halo=2, dtype="f32"):
+    h = _hierarchy(seed)
+    ctx = amr.from_hierarchy(h, dtype)
+    ctx.amr_build_kdtree(storage, gradient=gradient, halo=halo, maxbrick=maxbrick)
     return ctx, h.value_range()
 
 
@@ -53,6 +58,23 @@ def test_full_workspace_equals_per_ray(amr, step, size, maxbrick):
         assert np.array_equal(got[0][0], got[1][0])
 
 
+@pytest.mark.parametrize("storage,dtype,maxbrick", [
+    ("ptr", "f32", True), ("ptr", "f32", False), ("ptr", "f16", True), ("ptr", "bf16", False),
+    ("atlas_linear", "f32", False), ("atlas_linear", "f16", False)])
+@pytest.mark.parametrize("gradient,halo", [(True, 2), (True, 1), (False, 1)])
+def test_storages_and_pruning_equal_per_ray(amr, storage, dtype, maxbrick, gradient, halo):
+    ctx, (vmin, vmax) = _context(amr, 5, maxbrick, gradient, storage, halo, dtype)
+    cam = synth.orbit_camera(9, 61, 50)
+    for lod, skip, row0, rows in ((0.0, 0, 0, 0), (3.0, 0, 0, 0), (0.0, 1, 13, 21)):
+        got = []
+        for schedule in (0, 3):
+            p, _ = params_pair(amr, vmin, vmax, schedule=schedule, shade=1, kappa=20.0,
+                               lod_pixels=lod, skip=skip, row0=row0, rows=rows)
+            got.append(gpu_render(ctx, cam, _opaque_tf(), p))
+        assert got[0][1] == got[1][1] > 0
+        assert np.array_equal(got[0][0], got[1][0])
+
+
 def test_segment_bound_is_reported_for_the_same_rays(amr):
     ctx, (vmin, vmax) = _context(amr)
     cam = synth.orbit_camera(5, 40, 31)
@@ -79,10 +101,7 @@ def test_segment_bound_is_reported_for_the_same_rays(amr):
 @pytest.mark.parametrize("schedule", [0, -1])
 def test_unshaded_frames_do_not_read_samples_per_iter(amr, dtype, schedule):
     """Schedule 0 takes any value of the field (it belongs to schedules 2 and 3)."""
-    h = random_hierarchy(3, n0=12, num_levels=3, patches_per_level=6)
-    ctx = amr.from_hierarchy(h, dtype)
-    ctx.amr_build_kdtree("ptr", halo=2, maxbrick=True)
-    vmin, vmax = h.value_range()
+    ctx, (vmin, vmax) = _context(amr, dtype=dtype, gradient=False)
     cam = synth.orbit_camera(2, 70, 53)
     want = None
     for spi in (16, 0, -1, 1, 65, 2 ** 31 - 1, -2 ** 31):
@@ -111,21 +130,28 @@ def test_long_transfer_functions(amr, n, shade):
 
 
 def test_large_images_and_a_failing_launch(amr, monkeypatch):
-    """Images of 3,000,000 pixels and more leave what the split march does not take to the
-    per-ray loop; a launch that fails before that is still reported."""
+    """Images of 3,000,000 pixels and more go through the split march on hierarchies of 10,000
+    leaves and more, and leave what it does not take to the per-ray loop; a launch that fails
+    before that is still reported."""
     from paper_1212_3333_gb300 import _lib
 
-    ctx, (vmin, vmax) = _context(amr)
+    h = random_hierarchy(7, n0=32, num_levels=4, patches_per_level=300, max_size=9)
+    ctx = amr.from_hierarchy(h)
+    ctx.amr_build_kdtree("ptr", gradient=True, halo=2, maxbrick=True)
+    assert ctx.amr_get_stats().num_leaves >= 10000
+    vmin, vmax = h.value_range()
     cam = synth.orbit_camera(4, 2003, 1501)
-    for clear in (16, 0):
-        p, _ = params_pair(amr, vmin, vmax, schedule=0, shade=1)
+    # a few samples opaque, so many that the march stops on the way, all of them
+    for clear, step in ((58, 0.5), (30, 0.1), (0, 0.5)):
+        p, _ = params_pair(amr, vmin, vmax, schedule=0, shade=1, step_factor=step, kappa=0.01)
         want = gpu_render(ctx, cam, _opaque_tf(clear=clear), p)
         p.schedule = 3
-        monkeypatch.setenv("AMR_FAULT", "shade_launch")
-        with pytest.raises(amr.AmrError) as e:
-            gpu_render(ctx, cam, _opaque_tf(clear=clear), p)
-        assert e.value.status == _lib.AMR_ERR_CUDA
-        monkeypatch.delenv("AMR_FAULT")
+        if clear:
+            monkeypatch.setenv("AMR_FAULT", "shade_launch")
+            with pytest.raises(amr.AmrError) as e:
+                gpu_render(ctx, cam, _opaque_tf(clear=clear), p)
+            assert e.value.status == _lib.AMR_ERR_CUDA
+            monkeypatch.delenv("AMR_FAULT")
         got = gpu_render(ctx, cam, _opaque_tf(clear=clear), p)
         assert got[1] == want[1] and np.array_equal(got[0], want[0])
 
