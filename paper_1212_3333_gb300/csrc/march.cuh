@@ -1641,13 +1641,21 @@ __device__ __forceinline__ bool sample_segment_grouped(const RenderArgs& A, cons
     if (walk.inside) mask = walk.template opaque_mask<G>(k0, n, clear_below);
     mask &= (1u << cnt) - 1u;
     nsamp += cnt;
-    while (mask != 0) {
-      const int q = __ffs(mask) - 1;
-      mask &= mask - 1;
-      if (sample_candidate<ST, SHADE>(A, R, s_tf, g, lv, k0 + q, Lx, Ly, Lz, C0, C1, C2, Acc)) {
-        nsamp -= (unsigned)(cnt - 1 - q);  // early ray termination
-        return true;
-      }
+    auto ends = [&](int q) {  // evaluates sample k0 + q; true: early ray termination
+      if (!sample_candidate<ST, SHADE>(A, R, s_tf, g, lv, k0 + q, Lx, Ly, Lz, C0, C1, C2, Acc))
+        return false;
+      nsamp -= (unsigned)(cnt - 1 - q);
+      return true;
+    };
+    if constexpr (ST != ST_PTR && (SHADE & 3) == 0) {
+      // 16-bit cells unshaded: sample by sample (by set bits the compiler's code takes twice as
+      // long: 800 x 600, 3,998 leaves, 0.80 against 1.52 ms; with FP32 cells 0.83 / 0.77)
+#pragma unroll 1
+      for (int q = 0; q < cnt; ++q)
+        if ((mask >> q & 1u) && ends(q)) return true;
+    } else {
+      for (; mask != 0; mask &= mask - 1)
+        if (ends(__ffs(mask) - 1)) return true;
     }
   }
   return false;

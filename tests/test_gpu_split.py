@@ -97,11 +97,36 @@ def test_segment_bound_is_reported_for_the_same_rays(amr):
     assert seen == {True, False}
 
 
+# unshaded: hierarchies of 2,500 leaves and more through the split march up to 350,000 pixels,
+# the others, and larger images, through the per-ray loop
+@pytest.mark.parametrize("dtype", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("patches", [40, 100])
+def test_unshaded_frames_equal_those_without_maximum_bricks(amr, dtype, patches):
+    h = random_hierarchy(4, n0=16, num_levels=4, patches_per_level=patches, max_size=8)
+    vmin, vmax = h.value_range()
+    ctx = []
+    for maxbrick in (False, True):
+        ctx.append(amr.from_hierarchy(h, dtype))
+        ctx[-1].amr_build_kdtree("ptr", halo=2, maxbrick=maxbrick)
+    assert (ctx[0].amr_get_stats().num_leaves >= 2500) == (patches == 100)
+    for size in ((67, 45), (700, 501)):
+        for kappa, ert, clear, lod in ((0.5, 0.0, 40, 0.0), (0.5, 0.0, 0, 0.0), (40.0, 1e-3, 16, 0.0),
+                                       (0.5, 0.0, 40, 3.0)):
+            p, _ = params_pair(amr, vmin, vmax, schedule=0, shade=0, step_factor=0.3, kappa=kappa,
+                               ert_eps=ert, lod_pixels=lod)
+            cam = synth.orbit_camera(6, *size)
+            (a, na), (b, nb) = (gpu_render(c, cam, _opaque_tf(clear=clear), p) for c in ctx)
+            assert na == nb > 0 and np.array_equal(a, b)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "f16"])
 @pytest.mark.parametrize("schedule", [0, -1])
 def test_unshaded_frames_do_not_read_samples_per_iter(amr, dtype, schedule):
     """Schedule 0 takes any value of the field (it belongs to schedules 2 and 3)."""
-    ctx, (vmin, vmax) = _context(amr, dtype=dtype, gradient=False)
+    h = random_hierarchy(4, n0=16, num_levels=4, patches_per_level=100, max_size=8)
+    ctx = amr.from_hierarchy(h, dtype)  # (3,000 leaves and more: the split march)
+    ctx.amr_build_kdtree("ptr", halo=2, maxbrick=True)
+    vmin, vmax = h.value_range()
     cam = synth.orbit_camera(2, 70, 53)
     want = None
     for spi in (16, 0, -1, 1, 65, 2 ** 31 - 1, -2 ** 31):
