@@ -199,7 +199,7 @@ __device__ __forceinline__ float4 march_deferred(const RenderArgs& A, const RayA
         int pid1 = kPidOut;
         float tau1 = rf.tau_out, e1 = exit_bound(rf);
         const int lmin = lod_min_level(R, A.lv, rf, i, j, pid0, tau0, e0);
-        const int lid = next_leaf(A.nodes, A.leaves, A.face_node, A.node_box, R, i, j, rf,
+        const int lid = next_leaf<kLdexp<1, SHADE>>(A.nodes, A.leaves, A.face_node, A.node_box, R, i, j, rf,
                                   start, prev, pid0, tau0, e0, pid1, tau1, e1, lmin);
         if (lid < 0) {
           status |= kStatusDevice;
