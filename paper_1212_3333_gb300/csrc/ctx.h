@@ -145,6 +145,7 @@ struct TaskPlan {
   TaskSpace ts = {};
   long long tiles = 0;
   long long left = 0;  // entries of the list of tiles given up
+  int per_pixel = 128;  // tasks a pixel the rounds are for
   float dense_below = 0;  // RenderArgs::dense_below of the call
   int rounds(long long tiles_of_band) const;
 };

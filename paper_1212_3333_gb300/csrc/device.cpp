@@ -270,21 +270,19 @@ amr_status upload_max_pool(amr_ctx* c, const std::vector<std::vector<T>>& mb, cu
 // 5-level hierarchy with a ramp transfer function takes 23, and 8 segment records -, up to
 // kMaxTasks, but kTileChunks chunks (320 tasks a pixel) for every tile under way, so that dense
 // tiles need not be given up: 1.7 GB for most images, 3.5 GB at most.  (With 40 tasks a pixel
-// alone, at 640 x 479 tiles were given up and the frame took 5.4 instead of 2.7 ms.)  A call gets
-// enough rounds for kDensePerPixel tasks a pixel; what is denser goes to deferred_kernel (every
-// sample opaque, 640 x 479, 480 tasks a pixel: all tasks in the workspace 14.3 ms,
-// deferred_kernel alone 16.1).
-static constexpr int64_t kTasksPerPixel = 40, kDensePerPixel = 128, kTileChunks = 80;
+// alone, at 640 x 479 tiles were given up and the frame took 5.4 instead of 2.7 ms.)
+static constexpr int64_t kTasksPerPixel = 40, kTileChunks = 80;
 static constexpr int64_t kMaxTasks = (int64_t)1 << 26;
 static constexpr int64_t kWarps = 152 * 16;  // of the march, at once
 
-static int64_t task_rounds(int64_t tiles, int64_t chunks) {
+// Rounds for so many tasks a pixel; the one-kernel march takes what they leave.
+static int64_t task_rounds(int64_t tiles, int64_t chunks, int64_t per_pixel) {
   const int64_t usable = (chunks - chunks / 4) * kTaskChunk;
-  return std::min<int64_t>(64, (tiles * 32 * kDensePerPixel + usable - 1) / usable);
+  return std::min<int64_t>(64, (tiles * 32 * per_pixel + usable - 1) / usable);
 }
 
 int TaskPlan::rounds(long long tiles_of_band) const {
-  return (int)std::min<int64_t>(task_rounds(tiles_of_band, ts.chunks),
+  return (int)std::min<int64_t>(task_rounds(tiles_of_band, ts.chunks, per_pixel),
                                 left / std::max(1LL, tiles_of_band));
 }
 
@@ -363,7 +361,7 @@ static void grow_pool(DeviceState& d, int64_t tiles) {
 static void grow_tiles(DeviceState& d, int64_t need) {
   if (need <= d.task_tile_cap || need >= d.task_tiles_refused) return;
   const int64_t tiles = std::max(need, std::min(2 * d.task_tile_cap, kTaskTiles));
-  const int64_t left = tiles * task_rounds(tiles, d.tasks.chunks);
+  const int64_t left = tiles * task_rounds(tiles, d.tasks.chunks, 128);
   const size_t sizes[3] = {(size_t)tiles * sizeof(int2), (size_t)left * sizeof(int32_t),
                            (size_t)tiles * sizeof(int32_t)};
   size_t off[3];
@@ -424,7 +422,10 @@ TaskPlan plan_tasks(amr_ctx* c, long long call_tiles, TaskUse use, void* stream,
                         : use == TaskUse::image && tiles * 32 >= kLargePixels
                             ? (small_leaves ? 4.0f : 2.5f)
                         : small_leaves || tiles < kWaveTiles ? 12.0f
-                                                             : (many ? 6.0f : 4.0f);
+                                                             : (many ? 6.0f : 4.3f);
+  // Rounds for the densest images that are not stopped (a round that finds nothing to do costs
+  // four launches, about 10 us).
+  plan.per_pixel = use == TaskUse::image && (!many || tiles * 32 >= kLargePixels) ? 64 : 128;
   // Not begun at all: transfer functions that make four fifths of the cells opaque, or half of
   // them where the pool cannot hold the image whatever it shows.
   const bool holds = (int64_t)d.tasks.chunks * kTaskChunk >= tiles * 32 * 250;
