@@ -302,7 +302,8 @@ amr_status amr_render_batch(amr_ctx* ctx, const amr_view* views, int32_t n_views
 
 /* Time candidate configurations on this batch, one warm-up and `reps` (1..1000) timed
  * renders each, CUDA events on cuda_stream: first the 9 tiles 8x8 / 16x8 / 16x16 x rays
- * per thread 1 / 2 / 4 (blocks_per_sm 0, the params' samples_per_iter), then - for deferred
+ * per thread 1 / 2 / 4 (blocks_per_sm 0, the params' samples_per_iter; one and the same call,
+ * timed once, where deferred shading uses the workspace), then - for deferred
  * shading (schedule 3, also as AMR_SCHEDULE_AUTO picks it for batches) - the best of those
  * with samples_per_iter 4, 8, 16 and 32.  ms_out (nullable) receives the mean milliseconds
  * of the AMR_BATCH_CANDIDATES candidates in that order (tile-major; -1 for the last four

@@ -160,10 +160,11 @@ amr_status launch_st(amr_ctx* c, const BatchArgs& b, const amr_batch_config& cfg
 }  // namespace
 
 amr_status launch_batch(amr_ctx* c, const BatchArgs& b, int storage, int shade, int schedule,
-                        const amr_batch_config& cfg, void* stream) {
+                        const amr_batch_config& cfg, void* stream, bool* split) {
   cudaStream_t s = (cudaStream_t)stream;
   const bool mx = (shade & kShadeMaxBit) != 0;  // the stencil-maximum test
   shade &= ~kShadeMaxBit;
+  if (split) *split = false;
   if (storage != ST_PTR) return fail(c, AMR_ERR_ARG, "batched rendering needs the ptr storage (FP32)");
   if (schedule == 3 && (shade == 1 || shade == 2)) {
     // the split march over 8x4 tiles of all views, when the workspace has records for them
@@ -178,6 +179,7 @@ amr_status launch_batch(amr_ctx* c, const BatchArgs& b, int storage, int shade, 
     TaskPlan plan;
     if (tiles <= kTaskTiles) plan = plan_tasks(c, tiles, TaskUse::batch, stream, b.n_views);
     if (tiles <= plan.tiles) {
+      if (split) *split = true;
       t->n_items = (int32_t)tiles;
       t->A.ts = plan.ts;
       t->A.dense_below = plan.dense_below;

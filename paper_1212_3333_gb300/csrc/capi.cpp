@@ -689,12 +689,18 @@ amr_status amr_batch_autotune(amr_ctx* c, const amr_view* views, int32_t n_views
     return done(fail(c, AMR_ERR_CUDA, std::string("stream order: ") + cudaGetErrorString(order.error)));
   float best_ms = -1.0f;
   amr_batch_config best = c->batch_cfg;
-  // candidates 0..8: tile shape x rays per thread; 9..12: the best of those with 4, 8, 16
-  // and 32 samples per iteration (deferred shading only)
+  // candidates 0..8: tile shape x rays per thread, one and the same call where the batch goes
+  // through the split march; 9..12: the best of those with 4, 8, 16 and 32 samples per iteration
+  // (deferred shading only)
+  bool split = false;
   static const int spis[4] = {4, 8, 16, 32};
   const int shade = kernel_shade(c, params);
   for (int k = 0; k < AMR_BATCH_CANDIDATES; ++k) {
     amr_batch_config cfg = {shapes[k / 3][0], shapes[k / 3][1], rpts[k % 3], 0, 0};
+    if (k >= 1 && k < 9 && split) {
+      if (ms_out) ms_out[k] = best_ms;
+      continue;
+    }
     if (k >= 9) {
       if (params->schedule != 3) {
         if (ms_out) ms_out[k] = -1.0f;
@@ -712,7 +718,7 @@ amr_status amr_batch_autotune(amr_ctx* c, const amr_view* views, int32_t n_views
       if (cudaMemsetAsync(c->dev.counters, 0, kNumCounters * sizeof(unsigned long long), st) !=
           cudaSuccess)
         return done(fail(c, AMR_ERR_CUDA, "cudaMemsetAsync"));
-      s = launch_batch(c, *b, kernel_storage(c), shade, params->schedule, cfg, cuda_stream);
+      s = launch_batch(c, *b, kernel_storage(c), shade, params->schedule, cfg, cuda_stream, &split);
       if (s != AMR_OK) return done(s);
     }
     if (cudaEventRecord(e1, st) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||

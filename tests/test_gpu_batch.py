@@ -146,6 +146,28 @@ def test_batch_graph_replay_and_autotune(amr, c1):
     assert ctx.amr_get_stats() is not None and n_ref > 0
 
 
+def test_autotune_times_the_tile_shapes_once_where_they_do_not_matter(amr):
+    """Batches through the task workspace (hierarchies of 1,000 leaves and more) take no tile
+    shape: the nine shapes are one candidate.  Per-ray batches time each."""
+    import torch
+
+    from synth.amr import random_hierarchy
+
+    h = random_hierarchy(3, n0=16, num_levels=4, patches_per_level=40, max_size=8)
+    vmin, vmax = h.value_range()
+    ctx = amr.from_hierarchy(h)
+    ctx.amr_build_kdtree("ptr", gradient=True)
+    cams, tfi = _views(6, 2)
+    tfs = torch.as_tensor(np.stack(synth.tf_variants()), device="cuda")
+    views, _, total = amr.make_views(cams, tfi)
+    out = torch.zeros((total,), device="cuda")
+    for schedule, shapes in ((3, 1), (0, 9)):
+        p, _ = params_pair(amr, vmin, vmax, shade=1, schedule=schedule)
+        best, ms = ctx.amr_batch_autotune(views, tfs, p, out, reps=3)
+        assert all(m > 0 for m in ms[:9])
+        assert len(set(ms[:9])) == 1 if shapes == 1 else len(set(ms[:9])) > 1
+
+
 def test_batch_rejects_malformed_batches(amr, c1):
     import torch
 
