@@ -20,7 +20,8 @@
  *     bad_alloc makes the host build fail with AMR_ERR_OOM, oom the device upload's first
  *     allocation (AMR_ERR_OOM), corrupt_node uploads a root node that names itself as a
  *     child (indices stay in range; renders report AMR_ERR_DEVICE), shade_launch leaves out
- *     a launch of deferred shading and reports AMR_ERR_CUDA.  Unset: no effect.
+ *     a launch of deferred shading and reports AMR_ERR_CUDA; small_pool and few_tiles make
+ *     its workspace small (the images stay the same).  Unset: no effect.
  *   - Level l has spacing h^l = h^0 / r^l per axis (Sec. 2).  Patch boxes are int64[6]
  *     {lo_x, lo_y, lo_z, hi_x, hi_y, hi_z}, half-open, in level-l cell indices.  Level 0
  *     must tile its bounding box (the kD root, Sec. 3.1); same-level patches must be
@@ -408,6 +409,12 @@ typedef struct {
 } amr_stats;
 
 amr_status amr_get_stats(const amr_ctx* ctx, amr_stats* out);
+
+/* Test hook: what the split march of deferred shading did in the last such call of the context
+ * (of its last band of rows): counts4[0] tiles handed out, [1] tiles given up for lack of room,
+ * [2] how many of those a later round took up again, [3] tiles left as too dense.  Zeros before
+ * the first such call.  Synchronises the device. */
+amr_status amr_get_task_counts(const amr_ctx* ctx, int64_t* counts4);
 
 /* Leaves in canonical order (pre-order over the tree): box int32[6*n] in finest cells,
  * patch id, level.  cap = capacity in leaves; *n receives the leaf count (also when cap

@@ -169,6 +169,12 @@ class AmrContext:
         _check(self._lib.amr_get_stats(self._h, C.byref(s)), self._h)
         return s
 
+    def amr_get_task_counts(self):
+        """Of the last split march: tiles handed out, given up, taken up again, too dense."""
+        n = (C.c_int64 * 4)()
+        _check(self._lib.amr_get_task_counts(self._h, n), self._h)
+        return tuple(n)
+
     def amr_get_leaves(self):
         n = C.c_int64(0)
         self._lib.amr_get_leaves(self._h, None, None, None, 0, C.byref(n))

@@ -112,6 +112,7 @@ _SIGS = {
     "amr_destroy": (C.c_int, [_P]),
     "amr_last_error": (C.c_char_p, [_P]),
     "amr_get_stats": (C.c_int, [_P, C.POINTER(amr_stats)]),
+    "amr_get_task_counts": (C.c_int, [_P, C.POINTER(C.c_int64)]),
     "amr_get_leaves": (C.c_int, [_P, C.POINTER(C.c_int32), C.POINTER(C.c_int32),
                                  C.POINTER(C.c_int32), C.c_int64, C.POINTER(C.c_int64)]),
     "amr_get_nodes": (C.c_int, [_P, C.POINTER(C.c_int32), C.POINTER(C.c_int32),

@@ -815,6 +815,19 @@ amr_status amr_get_stats(const amr_ctx* c, amr_stats* out) {
   return AMR_OK;
 }
 
+amr_status amr_get_task_counts(const amr_ctx* c, int64_t* counts4) {
+  if (!c || !counts4) return AMR_ERR_ARG;
+  std::fill(counts4, counts4 + 4, (int64_t)0);
+  if (!c->device_built || !c->dev.tasks.heads) return AMR_OK;
+  unsigned h[kHeads] = {0};
+  if (cudaDeviceSynchronize() != cudaSuccess ||
+      cudaMemcpy(h, c->dev.tasks.heads, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess)
+    return AMR_ERR_CUDA;
+  const int at[4] = {kHeadTile, kHeadLeft, kHeadRest, kHeadDense};
+  for (int k = 0; k < 4; ++k) counts4[k] = (int64_t)h[at[k]];
+  return AMR_OK;
+}
+
 amr_status amr_get_leaves(const amr_ctx* c, int32_t* box6, int32_t* patch, int32_t* level,
                           int64_t cap, int64_t* n) {
   if (!c || !n) return AMR_ERR_ARG;

@@ -22,6 +22,9 @@ namespace amr {
 //                 range), so descents loop until their depth bound -> AMR_ERR_DEVICE
 //   shade_launch  the split march's shading kernel is not launched and its launch reports an
 //                 error                                      -> AMR_ERR_CUDA
+//   small_pool    the split march's workspace has room for 256 chunks of tasks, so that tiles are
+//                 given up and taken again in later rounds    -> the same images
+//   few_tiles     and records for 240 tiles, so that images go in bands of rows
 // Unset or any other value: no effect.
 inline bool fault_injected(const char* what) {
   const char* v = std::getenv("AMR_FAULT");

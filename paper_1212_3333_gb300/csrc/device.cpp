@@ -332,7 +332,8 @@ static void grow_pool(DeviceState& d, int64_t tiles) {
   const int64_t need =
       std::min(std::max(tiles * 32 * kTasksPerPixel, under_way) / kTaskChunk, most);
   if (need <= d.tasks.chunks || need >= d.task_refused) return;
-  const int64_t chunks = std::max(need, std::min<int64_t>(2 * (int64_t)d.tasks.chunks, most));
+  int64_t chunks = std::max(need, std::min<int64_t>(2 * (int64_t)d.tasks.chunks, most));
+  if (fault_injected("small_pool")) chunks = std::min<int64_t>(chunks, 256);
   const size_t slots = (size_t)chunks * kTaskChunk;
   const int64_t blocks = (int64_t)slots / 3 / kSegBlock + 2 * kWarps;
   const size_t sizes[7] = {slots * sizeof(float4), slots * sizeof(float4), slots * sizeof(int32_t),
@@ -360,7 +361,8 @@ static void grow_pool(DeviceState& d, int64_t tiles) {
 // pool needs fewer)
 static void grow_tiles(DeviceState& d, int64_t need) {
   if (need <= d.task_tile_cap || need >= d.task_tiles_refused) return;
-  const int64_t tiles = std::max(need, std::min(2 * d.task_tile_cap, kTaskTiles));
+  int64_t tiles = std::max(need, std::min(2 * d.task_tile_cap, kTaskTiles));
+  if (fault_injected("few_tiles")) tiles = std::min<int64_t>(tiles, 240);
   const int64_t left = tiles * task_rounds(tiles, d.tasks.chunks, 128);
   const size_t sizes[3] = {(size_t)tiles * sizeof(int2), (size_t)left * sizeof(int32_t),
                            (size_t)tiles * sizeof(int32_t)};

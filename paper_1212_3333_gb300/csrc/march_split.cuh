@@ -68,6 +68,7 @@ struct CandArea<false> {
   float3 col[32];
 };
 constexpr float kNoWeight = -2.0f;
+constexpr unsigned kCrowded = 512;
 constexpr float kDenseSlack = 4096.0f;  // segments (in 32s) before the density counts
 
 // The bits of a warp's `count` tasks (lane q holds the owner of task q) that belong to the
@@ -103,8 +104,8 @@ struct SegBlock {
 
 // The march of pixel (i, j) of view R by one lane of a warp whose 32 lanes all call this
 // together (lanes without a pixel pass active = false).  Shaded: px receives the headlight
-// direction and the opacity, and tile the first chunk and the number of the warp's tasks;
-// unshaded: px receives the pixel.  Returns kTileDone, or why the tile was given up.
+// direction and the opacity, tile the first chunk and the number of the warp's tasks, and segs
+// the segments its rays fetched; unshaded: px receives the pixel.  Returns kTileDone, or why the tile was given up.
 enum { kTileDone = 0, kTileNoRoom = 1, kTileDense = 2 };
 template <int ST, int SHADE>
 __device__ __forceinline__ int march_tile(const RenderArgs& A, const RayArgs& R, int i, int j,
@@ -403,6 +404,8 @@ __device__ __forceinline__ int march_tile(const RenderArgs& A, const RayArgs& R,
       if (flush || full) break;
     }
   }
+  tile = make_int2(first, tasks);
+  segs = SHADED ? __reduce_add_sync(FULL, seg) : 0;
   if (full) return tasks / kTaskChunk >= A.ts.tile_chunks ? kTileDense : kTileNoRoom;
   if (SHADED && lane == 0 && tasks != 0) {
     const int last = tasks & (kTaskChunk - 1);
@@ -412,8 +415,6 @@ __device__ __forceinline__ int march_tile(const RenderArgs& A, const RayArgs& R,
   if (met & (kMetSegments | kMetSamples)) status |= kStatusCapacity;
   if (met & kMetTree) status |= kStatusDevice;
   px.w = Acc;
-  tile = make_int2(first, tasks);
-  segs = SHADED ? __reduce_add_sync(FULL, seg) : 0;
   return kTileDone;
 }
 
@@ -443,11 +444,15 @@ __global__ void __launch_bounds__(128, (SHADE & 3) != 0 ? AMR_SPLIT_MARCH_BLOCKS
   const RenderArgs& A = render_args(P);
   const int n_tiles = count_tiles(P);
   unsigned ready = 0;  // tiles that earlier rounds gave up
+  float warps = 0.0f;  // that will have a tile at once
   if constexpr (SHADED) {
     ready = __ldcg(A.ts.heads + kHeadReady);
-    if (__ldcg(A.ts.heads + kHeadTile) >= (unsigned)n_tiles &&
-        __ldcg(A.ts.heads + kHeadRest) >= ready)
-      return;
+    const unsigned again = ready - min(__ldcg(A.ts.heads + kHeadRest), ready);
+    const unsigned todo = (unsigned)n_tiles - min(__ldcg(A.ts.heads + kHeadTile), (unsigned)n_tiles) + again;
+    if (todo == 0) return;
+    // so many tiles found no room that half as many go at once
+    if (again >= kCrowded && (blockIdx.x & 1)) return;
+    warps = (float)min(gridDim.x * (again >= kCrowded ? 2u : 4u), todo);
   }
   extern __shared__ float4 smem[];
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
@@ -474,9 +479,8 @@ __global__ void __launch_bounds__(128, (SHADE & 3) != 0 ? AMR_SPLIT_MARCH_BLOCKS
         // pays is left to the one-kernel march from there on.
         const unsigned* H = A.ts.heads;
         const float taken = (float)max(__ldcg(H + kHeadTile), 1u), tasks = (float)__ldcg(H + kHeadTasks);
-        const float room = fmaxf(0.25f * (float)A.ts.chunks,
-                                 (float)min((int)gridDim.x * 4, n_tiles) *
-                                     (0.5f + tasks * (32.0f / kTaskChunk) / taken));
+        const float chunks = tasks * (32.0f / kTaskChunk) / taken;  // of a tile, but for its last
+        const float room = fmaxf(0.25f * (float)A.ts.chunks, warps * fminf(chunks + 0.5f, 2.0f * chunks));
         if ((float)__ldcg(H + kHeadChunk) + room < (float)A.ts.chunks &&
             __ldcg(H + kHeadSegBlock) < (unsigned)(A.ts.seg_blocks - A.ts.seg_blocks / 4) &&
             tasks <= A.ts.dense_ratio * ((float)__ldcg(H + kHeadSegs) + kDenseSlack)) {
@@ -501,7 +505,7 @@ __global__ void __launch_bounds__(128, (SHADE & 3) != 0 ? AMR_SPLIT_MARCH_BLOCKS
     const int j = R.row0 + jr;
     const bool active = i < p.width && jr < p.rows && j < R.height;
     float4 px;
-    int2 tile;
+    int2 tile = make_int2(-1, 0);
     int segs = 0;
     // nearly everything opaque: one kernel is faster (640 x 479, 480 opaque samples a pixel:
     // 16.1 ms alone, 24.7 after a workspace full of tasks), so the tile is left to it
@@ -510,14 +514,14 @@ __global__ void __launch_bounds__(128, (SHADE & 3) != 0 ? AMR_SPLIT_MARCH_BLOCKS
       how = march_tile<ST, SHADE>(A, R, i, j, active, staged.tf(p), staged.nz(p),
                                   staged.clear_below(p), Q, rf, blk, t, p.view, px, tile, segs, nsamp,
                                   status);
+    if (SHADED && lane == 0 && segs != 0) {
+      atomicAdd(A.ts.heads + kHeadTasks, (unsigned)(tile.y + 31) >> 5);
+      atomicAdd(A.ts.heads + kHeadSegs, (unsigned)(segs + 31) >> 5);
+    }
     if (how == kTileDone) {
       if (SHADED && tile.y == 0) px = make_float4(0.f, 0.f, 0.f, px.w);  // nothing to shade
       if (active) p.out[p.at(i, jr)] = px;
-      if (SHADED && lane == 0) {
-        if (tile.y != 0) A.ts.tile[t] = tile;
-        atomicAdd(A.ts.heads + kHeadTasks, (unsigned)(tile.y + 31) >> 5);
-        atomicAdd(A.ts.heads + kHeadSegs, (unsigned)(segs + 31) >> 5);
-      }
+      if (SHADED && lane == 0 && tile.y != 0) A.ts.tile[t] = tile;
     } else if (lane == 0) {
       if (how == kTileDense) A.ts.dense[atomicAdd(A.ts.heads + kHeadDense, 1u)] = t;
       else A.ts.left[atomicAdd(A.ts.heads + kHeadLeft, 1u)] = t;

@@ -1,8 +1,9 @@
 """GPU checks of deferred shading through the task workspace (the split march): images and
-sample counts equal the per-ray schedule's bit for bit when the workspace goes through several
-rounds, gives tiles up and leaves some to the single-kernel march; when there is no workspace
-(a first call under stream capture); and the bounds on segments are reported for the same rays
-although a ray may be marched beyond the sample that ends it."""
+sample counts equal the per-ray schedule's bit for bit, when the workspace is small and goes
+through several rounds, gives tiles up and takes them up again, in bands of rows, and leaves
+dense tiles to the single-kernel march; when there is no workspace (a first call under stream
+capture); and the bounds on segments are reported for the same rays although a ray may be marched
+beyond the sample that ends it."""
 import numpy as np
 import pytest
 
@@ -73,6 +74,40 @@ def test_storages_and_pruning_equal_per_ray(amr, storage, dtype, maxbrick, gradi
             got.append(gpu_render(ctx, cam, _opaque_tf(), p))
         assert got[0][1] == got[1][1] > 0
         assert np.array_equal(got[0][0], got[1][0])
+
+
+@pytest.mark.parametrize("maxbrick", [True, False])
+@pytest.mark.parametrize("shadow", [0, 1])
+def test_small_workspace_takes_tiles_up_again(amr, monkeypatch, maxbrick, shadow):
+    """256 chunks for 620 tiles of up to a chunk each (denser ones are left): some are given up and
+    taken up again, with the second transfer function in two rounds and more, as a round has
+    room for at most 256."""
+    ctx, (vmin, vmax) = _context(amr, maxbrick=maxbrick)
+    cam = synth.orbit_camera(2, 160, 121, fov_y_deg=18.0)
+    tfs = [_opaque_tf(clear=20), _opaque_tf(clear=8)]
+    want = []
+    for tf in tfs:
+        p, _ = params_pair(amr, vmin, vmax, schedule=0, shade=1, kappa=0.05, step_factor=8.0)
+        if shadow:
+            p.schedule = 3  # (images agree to rounding with the per-ray schedule's)
+            p.shadow, p.light_step = 1, 0.02
+            for a in range(3):
+                p.light[a] = 0.4 + 0.1 * a
+        want.append(gpu_render(ctx, cam, tf, p))
+    small, _ = _context(amr, maxbrick=maxbrick)
+    monkeypatch.setenv("AMR_FAULT", "small_pool")
+    p.schedule = 3
+    for tf, (img, n) in zip(tfs, want):
+        got = gpu_render(small, cam, tf, p)
+        assert got[1] == n and np.array_equal(got[0], img)
+        tiles, left, again, dense = small.amr_get_task_counts()
+        assert tiles >= 620 and again > (256 if tf is tfs[1] else 0) and dense > 0, (left, again)
+    few, _ = _context(amr, maxbrick=maxbrick)
+    monkeypatch.setenv("AMR_FAULT", "few_tiles")  # 20 tiles a row: three bands of 48 rows
+    for tf, (img, n) in zip(tfs, want):
+        got = gpu_render(few, cam, tf, p)
+        assert got[1] == n and np.array_equal(got[0], img)
+        assert 0 < few.amr_get_task_counts()[0] <= 240 + 2432
 
 
 def test_segment_bound_is_reported_for_the_same_rays(amr):
