@@ -77,9 +77,9 @@ __global__ void __launch_bounds__(128) forward_kernel(const unsigned char* __res
 // BF16 values (8 + 8 + 8 bits of its 24), so products are those of FP32.  The tensor cores
 // round their FP32 sums toward zero, which adds up along a chain of them, so every 16 products
 // (all three parts) start from zero and are added to the running sum by an FP32 addition:
-// error of the gradient against 64 bits, batch 16384, two seeds: FP32 chains of one thread
-// per row 3.5e-7 / 5.4e-7, chained products 7.0e-7 / 1.2e-6, this 4.0e-7 / 2.6e-7; batch 301:
-// 9.4e-8 / 9.6e-8, 3.6e-7 / 3.2e-7, 8.1e-8 / 9.3e-8.  A step (gradient, reduction, Adam) of 16384
+// error of the gradient against 64 bits, median of 12 seeds, FP32 chains of one thread per row /
+// this: batch 300 1.1e-7 / 5.7e-8, 4999 5.8e-7 / 8.0e-8, 16384 4.0e-7 / 1.4e-7, 131072 7.4e-7 / 1.4e-7
+// (chained products, two seeds at 16384: 7.0e-7 / 1.2e-6).  A step (gradient, reduction, Adam) of 16384
 // rows takes 33 us against 131 for one thread per row on the CUDA cores, of 131072 rows 99
 // against 783 us; at 16384 rows and below its latencies bound it (one tile per block).
 // Activations and deltas of the tile lie in shared memory for the weight gradients, whose

@@ -102,6 +102,65 @@ def test_mlp_gradient_against_64_bits(mods, n):
         k += r.size
 
 
+def exact_network(seed, n):
+    """Weights, features and targets whose forward is exact in FP32 whatever the order of its sums:
+    features are multiples of 2^-4, weights of 2^-3 and 2^-5 (few of them not zero), so products
+    and sums have at most 23 bits and every BF16 rounding, ties included, is the same in any
+    correct implementation."""
+    rng = np.random.default_rng(seed)
+
+    def weights(rows, cols, unit, share):
+        w = rng.integers(-4, 5, size=(rows, cols)) * unit
+        return w * (rng.uniform(size=w.shape) < share)
+
+    ps = [weights(64, 12, 2.0 ** -3, 1.0), rng.integers(-8, 9, size=64) * 2.0 ** -4,
+          weights(64, 64, 2.0 ** -5, 0.3), rng.integers(-8, 9, size=64) * 2.0 ** -4,
+          weights(64, 64, 2.0 ** -5, 0.3), rng.integers(-8, 9, size=64) * 2.0 ** -4,
+          weights(1, 64, 2.0 ** -3, 1.0), np.array([0.25])]
+    x = rng.integers(-16, 17, size=(n, 12)) / 16.0
+    p = np.concatenate([w.ravel() for w in ps]).astype(np.float32)
+    return p, x.astype(np.float32), rng.uniform(0, 1, size=n).astype(np.float32)
+
+
+def exact_gradient(proposal, p, x, t):
+    """Loss and gradient (8 flat tensors) in 64 bits, the forward's BF16 roundings in place, and
+    the sums of its terms' magnitudes."""
+    W1, b1, W2, b2, W3, b3, W4, b4 = _oracle_params(proposal, p)
+    acts = [bf16_round(x)]
+    for W, b in ((W1, b1), (W2, b2), (W3, b3)):
+        acts.append(bf16_round(np.maximum(acts[-1] @ W.T + b, 0.0)))
+    z = acts[3] @ W4[0] + b4[0]
+    d = ((1.0 / (1.0 + np.exp(-z)) - t) / len(t))[:, None]
+    ref, mag = [None] * 8, [None] * 8
+    for k, W in ((3, W4), (2, W3), (1, W2), (0, W1)):
+        ref[2 * k], ref[2 * k + 1] = (d.T @ acts[k]).ravel(), d.sum(0)
+        mag[2 * k], mag[2 * k + 1] = (abs(d).T @ abs(acts[k])).ravel(), abs(d).sum(0)
+        d = (d @ W) * (acts[k] > 0)
+    return np.mean(np.logaddexp(0.0, z) - t * z), ref, mag
+
+
+# one row, the edges of a 128-row tile, a ragged batch, and more tiles than blocks (152)
+@pytest.mark.parametrize("n", [1, 16, 127, 128, 129, 1000, 152 * 128 + 5])
+def test_mlp_gradient_of_an_exact_forward(mods, n):
+    """With nothing to differ in the forward, what is left is the output's rounding (a few 2^-24
+    of the sigmoid) and that of FP32 products and sums, a few 2^-24 of their terms'
+    magnitudes.  Deltas cut to 16 bits (two BF16 parts instead of three) would leave up to
+    2^-17 / sqrt(3) = 4.4e-6 of a single row's."""
+    torch, amr, proposal = mods
+    p, x, t = exact_network(n, n)
+    prop = proposal.Proposal(p)
+    prop.loss_grad(torch.as_tensor(x, device="cuda"), torch.as_tensor(t, device="cuda"))
+    torch.cuda.synchronize()
+    loss, ref, mag = exact_gradient(proposal, p, x, t)
+    assert abs(float(prop.loss.item()) - loss) <= 1e-6 * loss
+    g = prop.grad.cpu().numpy().astype(np.float64)
+    k = 0
+    for r, m in zip(ref, mag):
+        err = np.linalg.norm(g[k:k + r.size] - r) / np.linalg.norm(m)
+        assert err <= 8 * 2.0 ** -24, (k, err)
+        k += r.size
+
+
 def test_adam_step_matches_formula(mods):
     torch, amr, proposal = mods
     rng = np.random.default_rng(2)
