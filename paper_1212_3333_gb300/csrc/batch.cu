@@ -1,19 +1,19 @@
-// Batched multi-view rendering: one persistent launch marches many views of one dataset.
+// Batched multi-view rendering: one call marches many views of one dataset.
 //
-// The views' pixel tiles form one work queue (items in view order, tiles row-major within
-// a view).  Every block pops a tile with one atomic, builds that view's ray arguments in
-// shared memory and marches the tile's pixels with the same per-pixel code as the
-// single-view kernel, so each view's image is bit-identical to its own amr_render.  Up to
-// eight transfer functions are read from global memory (L1-cached); their prefix counts of
-// non-transparent entries are staged in shared memory once per block.  The view table travels
-// in the kernel's parameter block, so a call is one memset and one launch and can be captured
-// in a CUDA graph.
+// Per-ray schedule: one persistent launch.  The views' pixel tiles form one work queue (items in
+// view order, tiles row-major within a view).  Every block pops a tile with one atomic, builds
+// that view's ray arguments in shared memory and marches the tile's pixels with the same
+// per-pixel code as the single-view kernel, so each view's image is bit-identical to its own
+// amr_render.  Up to eight transfer functions are read from global memory (L1-cached); their
+// prefix counts of non-transparent entries are staged in shared memory once per block.  The view
+// table travels in the kernel's parameter block, so the call is one memset and one launch.
 //
-// With schedule 3 the 8x4 tiles of all views go through the split march (march_split.cuh)
-// instead, the views' rays in device memory: 32 views of 64-512 pixels of the 5-level hierarchy
-// 49.4 / 24.3 ms against one kernel, 48 of 40-90 pixels 5.96 / 3.38.  Without room for the tiles'
-// records (or in a first call under capture) each warp of the one launch marches its rays with
-// the deferred-shading loop.  The paper renders one view per pass; batching is an addition for
+// With schedule 3 the 8x4 tiles of all views go through the split march (march_split.cuh), a
+// fixed series of launches, the views' rays in device memory: 32 views of 64-512 pixels of the
+// 5-level hierarchy 49.4 / 24.3 ms against one kernel, 48 of 40-90 pixels 5.96 / 3.38.  Where it
+// does not pay (plan_tasks), without room for the tiles' records, or in a first call under
+// capture, each warp of the one launch marches its rays with the deferred-shading loop.  All can
+// be captured in a CUDA graph.  The paper renders one view per pass; batching is an addition for
 // throughput over many small and large views.
 #include <cuda_runtime.h>
 

@@ -264,11 +264,16 @@ __global__ void __launch_bounds__(128, AMR_MIN_BLOCKS) learned_kernel(const __gr
   unsigned char* wsm = reinterpret_cast<unsigned char*>(smem) + ((tf_bytes + 15) & ~(size_t)15);
   __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(wsm + kPackBytes) + warp * 32 * kStride1;
   float* ys = reinterpret_cast<float*>(wsm + kPackBytes + 4 * 32 * kStride1 * 2) + warp * 32;
-  __shared__ float s_clear;
   for (int k = tid; k < kPackBytes / 16; k += blockDim.x * blockDim.y)
     reinterpret_cast<uint4*>(wsm)[k] = reinterpret_cast<const uint4*>(A.mlp)[k];
-  stage_tf(A, s_tf, s_nz, &s_clear, tid, blockDim.x * blockDim.y);
-  const float clear_below = s_clear;
+  float clear_below = 0.0f;
+  if constexpr ((SHADE & kShadeMaxBit) != 0) {
+    __shared__ float s_clear;
+    stage_tf(A, s_tf, s_nz, &s_clear, tid, blockDim.x * blockDim.y);
+    clear_below = s_clear;
+  } else {
+    stage_tf(A, s_tf, s_nz, nullptr, tid, blockDim.x * blockDim.y);
+  }
 
   unsigned nsamp = 0;
   unsigned long long status = 0;

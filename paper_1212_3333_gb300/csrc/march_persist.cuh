@@ -24,8 +24,7 @@ __global__ void __launch_bounds__(128, kMinBlocks<SHADE>)
   float4* s_tf = smem;
   int* s_nz = reinterpret_cast<int*>(smem + A.tf_n);
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-  __shared__ float s_clear;
-  stage_tf(A, s_tf, s_nz, &s_clear, tid, blockDim.x * blockDim.y);
+  stage_tf(A, s_tf, s_nz, nullptr, tid, blockDim.x * blockDim.y);
 
   const RayArgs& R = A.ray;
   const unsigned FULL = 0xffffffffu;
