@@ -169,6 +169,14 @@ cudaError_t launch_shaded(const TaskPlan& plan, cudaStream_t s, const RenderArgs
   return launch_one_kernel<ST, SHADE>(s, a);
 }
 
+// Level-of-detail pruning from so many pixels on leaves few and long segments, as in a tree of few
+// leaves: the one-kernel marches are faster.  (ms, split / one kernel: 30,164 leaves 2048^2 at 4
+// pixels 16.6 / 18.7, at 10 5.7 / 4.8, 1024^2 at 10 0.92 / 0.82; 32,198 leaves 1024^2 at 4 5.9 / 7.8, at 10
+// 2.8 / 2.2.)
+inline bool pruned_far(const RenderArgs& a) {
+  return a.ray.lod_scale * a.ray.height >= 8.0 * 2.0 * a.ray.tan_half_fov_y;
+}
+
 // Unshaded frames with stencil-maximum bricks: the split march for images whose few warps wait
 // for fetches, on hierarchies with enough leaves to make those dear; the per-ray loop elsewhere.
 // Measured (ms, split / per ray, ramp and every sample opaque): 77 leaves 256^2 0.163 / 0.143, 0.226
@@ -178,7 +186,7 @@ cudaError_t launch_shaded(const TaskPlan& plan, cudaStream_t s, const RenderArgs
 template <int ST>
 cudaError_t launch_plain_max(size_t tf_bytes, cudaStream_t s, const RenderArgs& a) {
   const long long most = a.ray.n_leaves >= 10000 ? 600000 : a.ray.n_leaves >= 2500 ? 350000 : 0;
-  if ((long long)a.ray.width * a.ray.rows > most)
+  if ((long long)a.ray.width * a.ray.rows > most || pruned_far(a))
     return launch_tiles(march_kernel<ST, 1, kShadeMaxBit>, tf_bytes, s, a);
   return launch_tiles(split_march_kernel<ST, kShadeMaxBit>,
                       ((tf_bytes + 15) & ~(size_t)15) + 4 * sizeof(CandArea<false>), s, a);
@@ -199,7 +207,8 @@ amr_status launch_storage(amr_ctx* c, const RenderArgs& a, int interp, int shade
   TaskPlan plan;
   // (not for texture storages, where it measured slower at 1900 x 1800: 37.1 against 31.8 ms;
   // nor for a caller that brings its own counters and may not allocate)
-  if (kLinearStorage<ST> && schedule == 3 && a.counters == c->dev.counters) 
+  if (kLinearStorage<ST> && schedule == 3 && a.counters == c->dev.counters &&
+      ((shade & kShadeShadow) != 0 || !pruned_far(a)))
     plan = plan_tasks(c, tiles_of(a), (shade & kShadeShadow) != 0 ? TaskUse::shadow : TaskUse::image, s);
   cudaError_t e;
   if (shade & kShadeShadow) {

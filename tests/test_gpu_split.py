@@ -66,7 +66,7 @@ def test_full_workspace_equals_per_ray(amr, step, size, maxbrick):
 def test_storages_and_pruning_equal_per_ray(amr, storage, dtype, maxbrick, gradient, halo):
     ctx, (vmin, vmax) = _context(amr, 5, maxbrick, gradient, storage, halo, dtype)
     cam = synth.orbit_camera(9, 61, 50)
-    for lod, skip, row0, rows in ((0.0, 0, 0, 0), (3.0, 0, 0, 0), (0.0, 1, 13, 21)):
+    for lod, skip, row0, rows in ((0.0, 0, 0, 0), (3.0, 0, 0, 0), (12.0, 0, 0, 0), (0.0, 1, 13, 21)):
         got = []
         for schedule in (0, 3):
             p, _ = params_pair(amr, vmin, vmax, schedule=schedule, shade=1, kappa=20.0,
@@ -146,7 +146,7 @@ def test_unshaded_frames_equal_those_without_maximum_bricks(amr, dtype, patches)
     assert (ctx[0].amr_get_stats().num_leaves >= 2500) == (patches == 100)
     for size in ((67, 45), (700, 501)):
         for kappa, ert, clear, lod in ((0.5, 0.0, 40, 0.0), (0.5, 0.0, 0, 0.0), (40.0, 1e-3, 16, 0.0),
-                                       (0.5, 0.0, 40, 3.0)):
+                                       (0.5, 0.0, 40, 3.0), (0.5, 0.0, 40, 12.0)):
             p, _ = params_pair(amr, vmin, vmax, schedule=0, shade=0, step_factor=0.3, kappa=kappa,
                                ert_eps=ert, lod_pixels=lod)
             cam = synth.orbit_camera(6, *size)
